@@ -44,6 +44,7 @@ struct Dec {
   static constexpr int NA = RW * AB / 16, NN = RW * NB / 16, NH = RW * HB / 16;
   static constexpr int NCH = NA + NN + NH;
   static constexpr int ROUNDS = (NCH + 31) / 32;
+  static constexpr bool kGather = (AB & 3) == 0;   // gathered records by cp.async (see gather_segment)
   // one record stage of a warp tile: angle | norm | header segments
   static constexpr int R_ANG = 0;
   static constexpr int R_NRM = RW * AB;
@@ -64,11 +65,42 @@ struct Dec {
   static_assert(REC_W % 16 == 0 && W_TP % 16 == 0 && WARP_B % 16 == 0, "alignment");
 };
 
-// Stage the records of a tail tile (nrows < RW) or of gathered slots into
-// `stage`.  Contiguous slots: 16-byte cp.async chunks of the three segments,
-// the last chunk of each zero-filled past the tile.  Gathered slots: lane
-// r < nrows copies row r's record with plain loads; an out-of-range slot
-// decodes as an all-zero record.
+// Largest power of two <= 16 that divides a record segment's row bytes: the
+// copy size of gathered records (each record starts on a multiple of it).
+__host__ __device__ constexpr int row_chunk(int bytes) {
+  int c = 16;
+  while (bytes % c) c >>= 1;
+  return c;
+}
+
+// Issue the copies of one segment (BYTES a row) of a tile's gathered records
+// into dst: the L lanes of row r copy its record `rec` in chunks of CB bytes
+// (rec = -1, a slot outside the cache: zero-filled).  Gathers are bound by
+// latency, so the copies are asynchronous and a tile deep in the ring like the
+// contiguous ones, and the slots are loaded a tile before their copies: four
+// paged sequences of 3001 tokens (16 layers, 8 heads, K and V, d = 64, bf16,
+// 606 MB in and out) take 185 us (3.3 TB/s), against 340 us (1.8 TB/s) with
+// one lane copying a row by plain loads when its tile was due; 229 us without
+// the check-free inner loop, 190 us with the chunks dealt round the warp
+// (a slot shuffle per chunk).
+template <int L, int BYTES>
+__device__ __forceinline__ void gather_segment(const uint8_t* base, long long rec, uint8_t* dst, int r, int l) {
+  constexpr int CB = row_chunk(BYTES), PER = BYTES / CB;
+  static_assert(CB >= 4, "cp.async copies 4, 8 or 16 bytes");
+  const int size = rec >= 0 ? CB : 0;
+  const uint8_t* src = base + (rec >= 0 ? rec : 0) * BYTES + l * CB;
+  uint8_t* out = dst + r * BYTES + l * CB;
+#pragma unroll
+  for (int q = 0; q < PER; q += L)
+    if (q + l < PER) cp_async_ca<CB>(out + q * CB, src + q * CB, size);
+}
+
+// Stage the records of a tail tile (nrows < RW) of contiguous slots, or of
+// gathered slots whose angle records do not fall on 4-byte boundaries (odd code
+// widths at d <= 32), into `stage`.  Contiguous slots: 16-byte cp.async chunks
+// of the three segments, the last chunk of each zero-filled past the tile.
+// Gathered slots: lane r < nrows copies row r's record with plain loads; an
+// out-of-range slot decodes as an all-zero record.
 template <int AB, int NB, int HB, int R_NRM, int R_HDR>
 __device__ __noinline__ void stage_records_slow(const DecJob& J, int64_t row0, int nrows, uint8_t* stage,
                                                 int lane) {
@@ -90,28 +122,25 @@ __device__ __noinline__ void stage_records_slow(const DecJob& J, int64_t row0, i
         cp_async16(stage + R_HDR + 16 * qq, gh + 16 * qq, rem >= 16 ? 16 : rem);
       }
     }
-  } else if (lane < nrows) {
-    const int64_t s = J.slot[row0 + lane];
-    uint8_t* da = stage + lane * AB;
-    uint8_t* dn = stage + R_NRM + lane * NB;
-    float2* dh = reinterpret_cast<float2*>(stage + R_HDR) + lane;
-    if (s < 0 || s >= J.capacity) {
-      for (int q = 0; q < AB; ++q) da[q] = 0;
-      for (int q = 0; q < NB; ++q) dn[q] = 0;
-      if constexpr (HB > 0) *dh = make_float2(0.f, 0.f);
-      return;
-    }
-    const uint8_t* sa = J.codes + s * AB;
-    const uint8_t* sn = J.norms + s * NB;
-    if constexpr ((AB & 3) == 0) {
-      for (int q = 0; q < AB / 4; ++q)
-        reinterpret_cast<uint32_t*>(da)[q] = __ldg(reinterpret_cast<const uint32_t*>(sa) + q);
-    } else {
+  } else if constexpr ((AB & 3) != 0) {
+    if (lane < nrows) {
+      const int64_t s = J.slot[row0 + lane];
+      uint8_t* da = stage + lane * AB;
+      uint8_t* dn = stage + R_NRM + lane * NB;
+      float2* dh = reinterpret_cast<float2*>(stage + R_HDR) + lane;
+      if (s < 0 || s >= J.capacity) {
+        for (int q = 0; q < AB; ++q) da[q] = 0;
+        for (int q = 0; q < NB; ++q) dn[q] = 0;
+        if constexpr (HB > 0) *dh = make_float2(0.f, 0.f);
+        return;
+      }
+      const uint8_t* sa = J.codes + s * AB;
+      const uint8_t* sn = J.norms + s * NB;
       for (int q = 0; q < AB; ++q) da[q] = __ldg(sa + q);
+      for (int q = 0; q < NB / 4; ++q)
+        reinterpret_cast<uint32_t*>(dn)[q] = __ldg(reinterpret_cast<const uint32_t*>(sn) + q);
+      if constexpr (HB > 0) *dh = __ldg(reinterpret_cast<const float2*>(J.hdr) + s);
     }
-    for (int q = 0; q < NB / 4; ++q)
-      reinterpret_cast<uint32_t*>(dn)[q] = __ldg(reinterpret_cast<const uint32_t*>(sn) + q);
-    if constexpr (HB > 0) *dh = __ldg(reinterpret_cast<const float2*>(J.hdr) + s);
   }
 }
 
@@ -300,6 +329,25 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
   int64_t i_row0 = 0;            // the tile's first row within its job
   int64_t i_left = 0;            // rows of the job from i_row0
   bool p_dense = true;
+  // Gathered jobs: the L lanes of row r hold the record index of row r of the
+  // next tile (-1: outside the cache or past the job), loaded one tile ahead of
+  // its copies so that the load's latency is covered by a tile's decode.
+  const int r = lane / C::L, l = lane % C::L;
+  long long g_rec = -1;
+  auto load_slots = [&](const DecJob& J) {
+    g_rec = -1;
+    if (r < i_left) {
+      const long long s = __ldg(reinterpret_cast<const long long*>(J.slot) + i_row0 + r);
+      if (s >= 0 && s < J.capacity) g_rec = s;
+    }
+  };
+  auto gather = [&](const DecJob& J, uint8_t* stage) {
+    if constexpr (C::kGather) {
+      gather_segment<C::L, C::AB>(J.codes, g_rec, stage + C::R_ANG, r, l);
+      gather_segment<C::L, C::NB>(J.norms, g_rec, stage + C::R_NRM, r, l);
+      if constexpr (C::HB > 0) gather_segment<C::L, 8>(J.hdr, g_rec, stage + C::R_HDR, r, l);
+    }
+  };
   const uint8_t* i_src[C::ROUNDS];  // this lane's record chunk(s) of the tile
   int i_step[C::ROUNDS];            // bytes between consecutive tiles of its plane
   auto set_issue_job = [&]() {
@@ -317,6 +365,8 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
       else { i_src[q] = J.hdr + 16 * (ch - C::NA - C::NN); i_step[q] = C::RW * C::HB; }
       i_src[q] += (int64_t)rel * i_step[q];
     }
+    if constexpr (C::kGather)
+      if (!p_dense) load_slots(J);
   };
   set_issue_job();
   auto issue = [&](int stg) {
@@ -332,6 +382,8 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
           const int ch = q * 32 + lane;
           if (ch < C::NCH) cp_async16(stage + 16 * ch, i_src[q], 16);
         }
+      } else if (C::kGather && !p_dense) {
+        gather(p.job[pj], stage);
       } else {
         stage_records_slow<C::AB, C::NB, C::HB, C::R_NRM, C::R_HDR>(p.job[pj], i_row0, (int)min((int64_t)C::RW, i_left),
                                                             stage, lane);
@@ -341,6 +393,8 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
       i_row0 += C::RW;
       i_left -= C::RW;
       ++it;
+      if constexpr (C::kGather)
+        if (!p_dense && it < t_end && it < p_end) load_slots(p.job[pj]);
     }
     cp_async_commit();
   };
@@ -351,7 +405,6 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
   int c_end = t;                 // first tile after the current job (forces a job load)
   int64_t c_left = 0;            // rows of the job from the current tile's row 0
   int64_t c_step = 0;            // output bytes between consecutive tiles (RW rows)
-  const int r = lane / C::L, l = lane % C::L;
   uint8_t* o_row = nullptr;      // this lane's first output pair in the current tile
   uint2 msk[8];
 #pragma unroll
@@ -366,23 +419,47 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
   while (t < t_end) {
     if (fast > 0) {
       // A stretch of `fast` tiles, each a full tile of the current job whose
-      // prefetch is a full tile of the (contiguous) issue job: no per-tile
-      // checks, the cursors are settled once after it.
+      // prefetch is a full tile of the issue job: no per-tile checks, the
+      // cursors are settled once after it.  One loop for contiguous and one
+      // for gathered issue jobs.
       const int t_stop = t + fast;
-      for (; t < t_stop; ++t) {
-        cp_async_wait<kNS - 2>();   // this warp tile's records have landed
-        __syncwarp();               // ... and every lane is done with the previous tile
-        uint8_t* dst = wsm + C::W_REC + ((stage + kNS - 1) & (kNS - 1)) * C::REC_W;
-#pragma unroll
-        for (int q = 0; q < C::ROUNDS; ++q) {
-          const int ch = q * 32 + lane;
-          if (ch < C::NCH) cp_async16(dst + 16 * ch, i_src[q], 16);
-          i_src[q] += i_step[q];
+      auto stretch = [&](auto&& copies) {
+        for (; t < t_stop; ++t) {
+          cp_async_wait<kNS - 2>();   // this warp tile's records have landed
+          __syncwarp();               // ... and every lane is done with the previous tile
+          copies(wsm + C::W_REC + ((stage + kNS - 1) & (kNS - 1)) * C::REC_W);
+          cp_async_commit();
+          decode_body<D, TOut, N, B, MODE>(wsm + C::W_REC + stage * C::REC_W, wsm, ttab, lane, msk, o_row, true);
+          o_row += c_step;
+          stage = (stage + 1) & (kNS - 1);
         }
-        cp_async_commit();
-        decode_body<D, TOut, N, B, MODE>(wsm + C::W_REC + stage * C::REC_W, wsm, ttab, lane, msk, o_row, true);
-        o_row += c_step;
-        stage = (stage + 1) & (kNS - 1);
+      };
+      if (!C::kGather || p_dense) {
+        stretch([&](uint8_t* dst) {
+#pragma unroll
+          for (int q = 0; q < C::ROUNDS; ++q) {
+            const int ch = q * 32 + lane;
+            if (ch < C::NCH) cp_async16(dst + 16 * ch, i_src[q], 16);
+            i_src[q] += i_step[q];
+          }
+        });
+      } else if constexpr (C::kGather) {
+        // the slots of the tile after the one being copied, a tile ahead (the
+        // last one loaded is the first after the stretch: checked against the job)
+        const DecJob& J = p.job[pj];
+        const long long* sp = reinterpret_cast<const long long*>(J.slot) + i_row0 + C::RW + r;
+        const long long cap = J.capacity;
+        int64_t left = i_left - C::RW - r;
+        stretch([&](uint8_t* dst) {
+          gather(J, dst);
+          g_rec = -1;
+          if (left > 0) {
+            const long long s = __ldg(sp);
+            if (s >= 0 && s < cap) g_rec = s;
+          }
+          sp += C::RW;
+          left -= C::RW;
+        });
       }
       const int64_t adv = (int64_t)fast * C::RW;
       i_row0 += adv;
@@ -417,7 +494,7 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
     // c_left now counts the rows of the compute job from tile t, i_left those
     // of the issue job from tile it (the next to prefetch).
     const int64_t cf = c_left / C::RW;
-    const int64_t pf = p_dense ? min(min((int64_t)(p_end - it), i_left / C::RW), (int64_t)(t_end - it)) : 0;
+    const int64_t pf = C::kGather || p_dense ? min(min((int64_t)(p_end - it), i_left / C::RW), (int64_t)(t_end - it)) : 0;
     const int64_t f = min(cf, pf);
     fast = f > 0 ? (int)f : 0;
   }

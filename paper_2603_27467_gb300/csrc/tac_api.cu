@@ -71,8 +71,7 @@ static cudaError_t launch_decode(int d, int dtype, int n, int b, int mode, const
   }
   return cudaErrorInvalidValue;
 }
-cudaError_t launch_attend(int d, int dtype, int nq_max, const AttParams& p, int nrows_total, float* ws,
-                          cudaStream_t st);
+cudaError_t launch_attend(int d, int dtype, int nq_max, const AttParams& p, float* ws, int sms, cudaStream_t st);
 cudaError_t attend_static_workspace(float** ws);
 cudaError_t launch_fwht_debug(int d, const void* x, int dtype, int64_t rows, int64_t stride,
                               const uint32_t* signs, float* y, cudaStream_t st);
@@ -847,7 +846,7 @@ int run_attend(const tac_attend_job* jobs, int njobs, float* ws, cudaStream_t st
       while (i < njobs) {
         std::memset(&P, 0, sizeof(P));
         int64_t splits = 0;
-        int nrows = 0, nq_max = 1;
+        int nq_max = 1;
         while (i < njobs && P.njobs < TAC_ATTEND_MAX_JOBS) {
           const tac_attend_job& J = jobs[i];
           const int64_t ns = (J.tokens + TAC_ATTEND_SPLIT - 1) / TAC_ATTEND_SPLIT;
@@ -876,11 +875,10 @@ int run_attend(const tac_attend_job* jobs, int njobs, float* ws, cudaStream_t st
           A.cv = tac::att_norm_case(A.bv, A.mv);
           copy_signs(A.sk, &J.cfg_k);
           copy_signs(A.sv, &J.cfg_v);
-          A.split0 = (int32_t)splits;
+          A.unit0 = (int32_t)splits;
           A.ws = ws_off;
           ws_off += attend_ws_floats(J);
           splits += ns;
-          nrows += A.nq;
           nq_max = std::max(nq_max, (int)A.nq);
           ++P.njobs;
           i = next(i + 1);
@@ -889,9 +887,9 @@ int run_attend(const tac_attend_job* jobs, int njobs, float* ws, cudaStream_t st
           fork.join();
           return fail(TAC_E_UNSUPPORTED, "%s: a single job has too many tokens", who);
         }
-        P.nsplits = (int32_t)splits;
+        P.nunits = (int32_t)splits;
         P.q_bf16 = dt == TAC_BF16;
-        cudaError_t e = tac::launch_attend(d, dt, nq_max, P, nrows, ws, fork.stream(g++));
+        cudaError_t e = tac::launch_attend(d, dt, nq_max, P, ws, num_sms(), fork.stream(g++));
         if (e != cudaSuccess) {
           fork.join();
           return fail(TAC_E_CUDA, "%s: launch failed: %s", who, cudaGetErrorString(e));

@@ -9,23 +9,43 @@
 // one transform per query and one per output instead of one per cached token.
 //
 // Two kernels (flash-decoding split over tokens):
-//   attend_partial  a CTA of 4 warps serves 4 consecutive splits of 256 tokens
-//                   of one job.  The CTA rotates its queries once (fp32
-//                   butterfly, times scale * log2 e for a base-2 softmax) and
-//                   builds the K and V bin-centre tables (cos, sin)(2 pi k / n).
-//                   Each warp streams its split in steps of RW tokens: a
-//                   cp.async ring stages the six record segments (K and V
-//                   angle / norm / header) of a step; K scores in the lane
-//                   layout of the decoder (L lanes per token, 8 pairs per
-//                   lane, shuffle reduction), an online softmax per query, V
-//                   accumulated with lane l owning pairs l + 32 j.  Each warp
-//                   writes (max, sum, accumulator) of its split to the workspace.
-//   attend_combine  one warp per (job, query): merges the splits, divides,
-//                   applies D H (fp32 butterfly) and stores the row.
+//   attend_partial  persistent CTAs of 8 warps over units of 256 tokens of one
+//                   job; a CTA takes a contiguous range of units and a warp 32
+//                   tokens of each (a batch).  Both contractions run on the
+//                   tensor cores (mma.sync m16n8k16, fp16 operands, fp32 sums):
+//                   the operands are decoded straight into the registers of the
+//                   fragments, so nothing decoded touches memory.  A decoded
+//                   value r^ (cos, sin), scaled by the power of two that brings
+//                   its record's largest norm into [1, 2), is split as
+//                   hi + lo: hi on the grid of 2^-10, lo the exact residue of
+//                   the fp32 product rounded to fp16 (2^-23 of the record's
+//                   scale at most).  The queries (and, for the values, the
+//                   softmax weights) are split hi + 2^-11 lo as well, both
+//                   rounded to fp16 (2^-24 of the value), the two parts in
+//                   different columns of the other operand: one mma for A_hi
+//                   and one for A_lo give all four products.  Sums over more
+//                   than a few mma steps are taken in fp32 registers.
+//   attend_combine  one CTA per (job, query): merges the CTAs' partial results
+//                   of the job, divides, applies D H (fp32 butterfly) and
+//                   stores the row.
+// Bound: instruction issue.  About 12 instructions decode and split one pair
+// (table offset 2, lookup 1, norm code 3, products and split 4, packing 2); of
+// 91 warp-instructions a token-head 48 are these (d = 128, 4 queries), and the
+// schedulers issue in 62 % of the cycles at 16 warps per SM (128 registers).
+// With the products on the CUDA cores (114 instructions, 10 - 12 warps, and a
+// warp walking 256 tokens alone) 16 sequences of 1k to 32k tokens (8 KV heads,
+// 4 queries each, 244 MB of records) took 229 us, now 162 us (1.5 TB/s); 8
+// heads of 4097 tokens 59 us, now 21 us (a CTA of 8 warps per 256 tokens fills
+// the device; a third of it are the launches); 128 heads of 8192 tokens at
+// d = 64 143 us, now 90 us.  Error of an fp32 output against 64 bits: 5.4e-7
+// (6.0e-7 before).  A persistent grid merges a CTA's units before it writes, so
+// the combine kernel reads one result per CTA and job instead of one per 256 tokens.
 // Codebooks (n, norm bits, norm mode) are runtime parameters: K and V may
 // differ, and any codebook the encoder supports is accepted.
 #include <algorithm>
 #include <atomic>
+
+#include <cuda_fp16.h>
 
 #include "tac_attend.cuh"
 
@@ -34,452 +54,763 @@ namespace tac {
 template <int V>
 struct IC { static constexpr int value = V; };
 
-constexpr int kAttMaxWarps = 6;               // warps (splits) per CTA: 1..6, chosen per launch
-constexpr int kAttSplit = TAC_ATTEND_SPLIT;   // tokens per split (one warp)
-constexpr int kAttNS = 2;                     // staged batches per warp
+constexpr int kAttWarps = 8;                  // warps per CTA
+constexpr int kAttThreads = 32 * kAttWarps;
+constexpr int kAttUnit = TAC_ATTEND_SPLIT;    // tokens of a unit: one batch for each warp
 constexpr float kLog2e = 1.4426950408889634f;
-static_assert(kAttSplit % kAttBatch == 0, "a split is whole batches");
+static_assert(kAttUnit == kAttWarps * kAttBatch, "a unit is one batch per warp");
 
-template <int D, int NQ>
+// QT = 1: up to 4 queries, the 8 columns of an mma are 4 hi and 4 lo parts;
+// QT = 2: up to 8 queries, one column tile of hi and one of lo parts.
+template <int D, int QT>
 struct Att {
-  using G = Geo<D>;
-  static constexpr int P = G::P, L = G::L, RW = G::RW;   // K: L lanes per token, RW tokens per pass
-  static constexpr int PV = P / 32;                      // V: pairs per lane
-  static constexpr int QROW = P + P / 4;                 // skewed rotated-query row (float2 units)
-  static constexpr int PBROW = 16 + 16 * ((NQ + 1) / 2); // per token: V constants, then (p, p) per query
-  static constexpr int PB = kAttBatch * PBROW;
-  // CTA shared memory: rotated queries | K table | V table | per warp (PB, kAttNS stages)
-  static constexpr int OFF_Q = 0;
-  static constexpr int OFF_TK = OFF_Q + NQ * QROW * 8;
-  static constexpr int OFF_TV = OFF_TK + kAttTabBytes;
-  static constexpr int OFF_W = OFF_TV + kAttTabBytes;
-  static constexpr int smem(int stage, int warps) { return OFF_W + warps * (PB + kAttNS * stage); }
-  static_assert(OFF_TK % 16 == 0 && PB % 16 == 0 && P % 32 == 0, "layout");
+  static constexpr int P = D / 2, NQ = 4 * QT;
+  static constexpr int KP = P / 4;            // K: pairs of a token a lane decodes (4 lanes a token)
+  static constexpr int VP = P / 8;            // V: pairs of a token a lane decodes (8 lanes a token)
+  // Shared memory: rotated queries | K table | V table | per warp: batch
+  // constants, weights, staged batch.  The merge of the warps' results reuses
+  // the warps' part.
+  static constexpr int QB = NQ * P * 8 + 64;  // float2 rows, then one scale per query
+  static constexpr int W_KC = 0;              // float2 per token: (A, B) of K's norms
+  static constexpr int W_VC = W_KC + kAttBatch * 8;
+  static constexpr int W_KS = W_VC + kAttBatch * 8;   // float per token: 2^e of K's record
+  static constexpr int W_VS = W_KS + kAttBatch * 4;
+  static constexpr int W_W = W_VS + kAttBatch * 4;    // weights: [2][columns][16 tokens] halves
+  static constexpr int W_STG = W_W + 2 * 8 * QT * 32;
+  static constexpr int MERGE = kAttWarps * NQ * D * 4;
+  static int smem(int stage, int tables) { return QB + tables + std::max(kAttWarps * (W_STG + stage), MERGE); }
+  static_assert(QB % 16 == 0 && W_STG % 16 == 0, "alignment");
 };
-
-// The skewed position of pair i in a rotated-query row: the 16-byte granules
-// (pairs 8l + 2m, 8l + 2m + 1) of the L lanes of a token fall on distinct banks.
-__device__ __forceinline__ int qpos(int i) { return i + 2 * (i >> 3); }
 
 __device__ __forceinline__ uint32_t rotr(uint32_t x, int s) { return __funnelshift_r(x, x, s); }
 
-// A shared-memory float4 load the compiler may not hoist or merge: keeps a
-// loop-invariant operand in shared memory instead of in registers.
-__device__ __forceinline__ float4 lds_f4_reload(const void* ptr) {
-  float4 v;
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(ptr);
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-  return v;
+__device__ __forceinline__ uint32_t h2_bits(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
+__device__ __forceinline__ __half2 h2_of(uint32_t u) { return *reinterpret_cast<const __half2*>(&u); }
+
+// d += a b: one m16n8k16 step, fp16 operands, fp32 accumulators.
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Reduce-scatter over the L lanes of a token, as a tree over the passes: the
-// lane's value for the pass set {I + k S} is its half, selected by lane bit S,
-// of the two sets {I + 2kS} and {I + S + 2kS}, plus the partner's.  At the
-// top (I = 0, S = 1) lane l holds the sum over the L lanes of pass l.  The
-// two passes of a base set {I, I + L/2} are computed together (one call).
-template <int L, int I, int S, int NQ, typename PF>
-__device__ __forceinline__ void att_tree(PF& pass, int l, float (&v)[NQ]) {
-  float va[NQ], vb[NQ];
-  if constexpr (2 * S == L) {
-    pass(IC<I>{}, IC<I + S>{}, va, vb);
+// d = a b: the same from zero accumulators.
+__device__ __forceinline__ void mma_f16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};\n"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// 2^k, k clamped to [-126, 126], and 2^x for an integer-valued x (0 below 2^-126).
+__device__ __forceinline__ float exp2i(int k) { return __uint_as_float((uint32_t)(127 + min(max(k, -126), 126)) << 23); }
+__device__ __forceinline__ float exp2_whole(float x) { return x < -126.f ? 0.f : exp2i((int)fminf(x, 126.f)); }
+// The exponent of a nonnegative fp32 number (-127 for zero and subnormals).
+__device__ __forceinline__ int exp_of(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFFu) - 127; }
+
+// The split of (r, r) * cs, |r cs| < 2: nh = -(hi of both), lo the residue.
+__device__ __forceinline__ void split_pair(float r, float2 cs, float2& nh, float2& lo) {
+  constexpr float M = 12288.f;                // 1.5 * 2^13: sums round to multiples of 2^-10
+  const float2 rr = make_float2(r, r);
+  const float2 q = __ffma2_rn(rr, cs, make_float2(M, M));
+  nh = __ffma2_rn(q, make_float2(-1.f, -1.f), make_float2(M, M));
+  lo = __ffma2_rn(rr, cs, nh);
+}
+
+// x = hi + 2^-11 lo in fp16 (|x| below about 2^15).
+__device__ __forceinline__ void split_half(float x, __half& hi, __half& lo) {
+  hi = __float2half_rn(x);
+  lo = __float2half_rn((x - __half2float(hi)) * 2048.f);
+}
+
+// Batch constants of one token from its header: r^ 2^-e = A c + B for the norm
+// code c (log mode: its log2), e the exponent of the larger of the two norms.
+__device__ __forceinline__ void norm_consts(float2 h, float inv_l, bool lg, float2& ab, float& scale) {
+  const bool spread = h.y > h.x;
+  const int e = min(max(exp_of(spread ? h.y : h.x), -126), 126);
+  const float sc = exp2i(-e);
+  scale = exp2i(e);
+  if (lg) {
+    const float lo = lg2_approx(h.x);
+    ab = make_float2(spread ? (lg2_approx(h.y) - lo) * inv_l : 0.f, lo - (float)e);
   } else {
-    att_tree<L, I, 2 * S, NQ>(pass, l, va);
-    att_tree<L, I + S, 2 * S, NQ>(pass, l, vb);
+    ab = make_float2(spread ? (h.y - h.x) * inv_l * sc : 0.f, h.x * sc);
   }
-  const bool up = (l & S) != 0;
-#pragma unroll
-  for (int a = 0; a < NQ; ++a) {
-    const float kept = up ? vb[a] : va[a];
-    const float send = up ? va[a] : vb[a];
-    v[a] = kept + __shfl_xor_sync(0xffffffffu, send, S);
-  }
-}
-
-// (A, B) of one record's norms: r^ = A f + B for the code c entered as
-// f = 1 + c 2^-b (its bits in the mantissa of 1.0); log mode gives log2 r^.
-// This is the inverse of Eq. 2: base + c step = f 2^b step + (base - 2^b step).
-__device__ __forceinline__ float2 norm_ab(float2 h, float inv_l, float two_b, bool lg) {
-  const float lo = lg ? lg2_approx(h.x) : h.x;
-  const float hi = lg ? lg2_approx(h.y) : h.y;
-  const float step = h.y > h.x ? (hi - lo) * inv_l : 0.f;
-  const float A = step * two_b;
-  return make_float2(A, lo - A);
 }
 
 // In-place normalized Walsh-Hadamard transform of `rows` rows of d floats in
-// shared memory (Sylvester order), by the nthreads threads of the caller.
+// shared memory (Sylvester order), by the lanes of a warp.
 template <int D>
-__device__ __forceinline__ void smem_fwht(float* buf, int rows, int tid, int nthreads, bool block_sync) {
-  for (int h = 1; h < D; h <<= 1) {
-    if (block_sync) __syncthreads(); else __syncwarp();
-    for (int e = tid; e < rows * D / 2; e += nthreads) {
-      const int r = e / (D / 2), k = e % (D / 2);
-      const int i = (k / h) * 2 * h + (k % h);
-      float* row = buf + r * D;
-      const float a = row[i], b = row[i + h];
+__device__ __forceinline__ void warp_fwht(float* row, int lane) {
+#pragma unroll
+  for (int lh = 0; (1 << lh) < D; ++lh) {
+    __syncwarp();
+#pragma unroll
+    for (int e = lane; e < D / 2; e += 32) {
+      const int i = ((e >> lh) << (lh + 1)) + (e & ((1 << lh) - 1));
+      const float a = row[i], b = row[i + (1 << lh)];
       row[i] = a + b;
-      row[i + h] = a - b;
+      row[i + (1 << lh)] = a - b;
     }
   }
-  if (block_sync) __syncthreads(); else __syncwarp();
+  __syncwarp();
 }
 
-template <int D, int NQ>
-__global__ void __launch_bounds__(32 * kAttMaxWarps, NQ <= 4 ? 2 : 1) attend_partial(const __grid_constant__ AttParams p, float* ws) {
-  using C = Att<D, NQ>;
-  constexpr int P = C::P, L = C::L, RW = C::RW, PV = C::PV;
+// The CTA that takes unit u when `units` units go to `ctas` CTAs in contiguous
+// ranges, the first units % ctas of them one longer.
+__host__ __device__ inline int att_cta_of(int u, int units, int ctas) {
+  const int per = units / ctas, extra = units % ctas, cut = extra * (per + 1);
+  return u < cut ? u / (per + 1) : extra + (u - cut) / per;
+}
+
+template <int D, int QT>
+__global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
+    attend_partial(const __grid_constant__ AttParams p, float* ws) {
+  using C = Att<D, QT>;
+  constexpr int P = C::P, NQ = C::NQ, KP = C::KP, KS = KP / 2, VP = C::VP;
+  constexpr int NV = 4 * QT;                       // scores a lane owns in the softmax
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nthr = blockDim.x, wpc = nthr >> 5;
+  const int g = lane >> 2, t = lane & 3;           // the fragments' row group and column pair
+  float2* const qrot = reinterpret_cast<float2*>(smem);                      // [NQ][P], slot order
+  float* const qscale = reinterpret_cast<float*>(smem + NQ * P * 8);         // 2^e of each query
+  float2* const tk = reinterpret_cast<float2*>(smem + C::QB);
+  uint8_t* const wbase = smem + C::QB + p.tab_k + p.tab_v;
+  float2* const tv = reinterpret_cast<float2*>(smem + C::QB + p.tab_k);
+  uint8_t* const pw = wbase + warp * (C::W_STG + p.stage);
+  float2* const kc = reinterpret_cast<float2*>(pw + C::W_KC);
+  float2* const vc = reinterpret_cast<float2*>(pw + C::W_VC);
+  float* const ksc = reinterpret_cast<float*>(pw + C::W_KS);
+  float* const vsc = reinterpret_cast<float*>(pw + C::W_VS);
+  uint8_t* const stk = pw + C::W_STG;
 
-  // ---- the CTA's job ----
+  // the combine kernel may be launched from now on (it waits for this grid's end)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  // the CTA's units
+  const int per = p.nunits / p.nctas, extra = p.nunits % p.nctas, cta = blockIdx.x;
+  int u = cta * per + min(cta, extra);
+  const int u_end = u + per + (cta < extra ? 1 : 0);
+  int tab_nk = 0, tab_nv = 0;                      // codebooks the tables hold
+
   int jb = 0;
   {
     int lo = 0, hi = p.njobs - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (p.job[mid].cta0 <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+      if (p.job[mid].unit0 <= u) lo = mid; else hi = mid - 1;
     }
     jb = lo;
   }
-  const AttJob& J = p.job[jb];
-  const int nq = J.nq;
 
-  // ---- batch geometry of this job's records ----
-  const int ak = P * J.wk / 8, nbk = P * J.bk / 8, av = P * J.wv / 8, nbv = P * J.bv / 8;
-  const int hkb = J.mk != TAC_NORM_FP32 ? 8 : 0, hvb = J.mv != TAC_NORM_FP32 ? 8 : 0;
-  const int S_KN = kAttBatch * ak, S_KH = S_KN + kAttBatch * nbk, S_VA = S_KH + kAttBatch * hkb;
-  const int S_VN = S_VA + kAttBatch * av, S_VH = S_VN + kAttBatch * nbv;
-  const int stage = S_VH + kAttBatch * hvb + 16;   // == att_stage_bytes(...)
+  for (; u < u_end; ++jb) {                        // a segment: the CTA's units of one job
+    const AttJob& J = p.job[jb];
+    const int nunits = (int)((J.tokens + kAttUnit - 1) / kAttUnit);
+    const int u_stop = min(u_end, J.unit0 + nunits);
+    const int nq = J.nq;
+    const int ak = P * J.wk / 8, nbk = P * J.bk / 8, av = P * J.wv / 8, nbv = P * J.bv / 8;
+    const int hkb = J.mk != TAC_NORM_FP32 ? 8 : 0, hvb = J.mv != TAC_NORM_FP32 ? 8 : 0;
+    uint8_t* const st_kn = stk + kAttBatch * ak;
+    uint8_t* const st_kh = st_kn + kAttBatch * nbk;
+    uint8_t* const st_va = st_kh + kAttBatch * hkb;
+    uint8_t* const st_vn = st_va + kAttBatch * av;
+    uint8_t* const st_vh = st_vn + kAttBatch * nbv;
+    int64_t row0 = (int64_t)(u - J.unit0) * kAttUnit + warp * kAttBatch;
+    const int64_t seg_rows = min(J.tokens, (int64_t)(u_stop - J.unit0) * kAttUnit);   // the segment's end
+    const int seg = cta - att_cta_of(J.unit0, p.nunits, p.nctas);
+    u = u_stop;
 
-  // ---- rotated queries q' = H D_K q * scale * log2(e), skewed float2 rows ----
-  float* qbuf = reinterpret_cast<float*>(smem + C::OFF_W);   // staging, reused by the batches below
-  for (int e = tid; e < nq * D; e += nthr) {
-    const int a = e / D, j = e % D;
-    float x;
-    if (p.q_bf16) {
-      x = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(J.q)[(int64_t)a * J.q_stride + j]);
-    } else {
-      x = reinterpret_cast<const float*>(J.q)[(int64_t)a * J.q_stride + j];
-    }
-    qbuf[e] = ((J.sk[j >> 5] >> (j & 31)) & 1u) ? -x : x;
-  }
-  smem_fwht<D>(qbuf, nq, tid, nthr, true);
-  float2* qrot = reinterpret_cast<float2*>(smem + C::OFF_Q);
-  const float qs = J.scale * kLog2e * rsqrtf((float)D);
-  for (int e = tid; e < NQ * P; e += nthr) {   // in record (slot) order: slot i holds pair slot_pair(i)
-    const int a = e / P, i = e % P, ip = slot_pair<D>(i);
-    qrot[a * C::QROW + qpos(i)] =
-        a < nq ? make_float2(qbuf[a * D + 2 * ip] * qs, qbuf[a * D + 2 * ip + 1] * qs) : make_float2(0.f, 0.f);
-  }
-  // ---- bin-centre tables (cos, sin)(2 pi k / n), 2^lgr copies: entry k copy c
-  // at k 2^lgr + c; entries n..2^W-1 repeat entry n-1 (codes >= n clamp) ----
-  const int lgrk = J.lgrk, lgrv = J.lgrv;
-  float2* tk = reinterpret_cast<float2*>(smem + C::OFF_TK);
-  float2* tv = reinterpret_cast<float2*>(smem + C::OFF_TV);
-  for (int e = tid; e < (1 << (J.wk + lgrk)); e += nthr) tk[e] = cos_sin_q8(8 * min(e >> lgrk, J.nk - 1), J.nk);
-  for (int e = tid; e < (1 << (J.wv + lgrv)); e += nthr) tv[e] = cos_sin_q8(8 * min(e >> lgrv, J.nv - 1), J.nv);
-  __syncthreads();
-
-  // ---- this warp's split ----
-  const int split = J.split0 + ((int)blockIdx.x - J.cta0) * wpc + warp;
-  const int64_t t_begin = (int64_t)(split - J.split0) * kAttSplit;
-  if (t_begin >= J.tokens) return;
-  const int64_t t_stop = min(J.tokens, t_begin + kAttSplit);
-  const int nb = (int)((t_stop - t_begin + kAttBatch - 1) / kAttBatch);
-  uint8_t* pb = smem + C::OFF_W + warp * (C::PB + kAttNS * stage);
-  uint8_t* stg = pb + C::PB;
-
-  // Stage batch s (tokens t_begin + 32 s ...): six segments in 16-byte
-  // chunks, bytes past the last token zero-filled.
-  auto issue = [&](int s) {
-    if (s < nb) {
-      const int64_t row0 = t_begin + (int64_t)s * kAttBatch;
-      const int rows = (int)min((int64_t)kAttBatch, J.tokens - row0);
-      uint8_t* st = stg + (s % kAttNS) * stage;
-      const uint8_t* src[6] = {J.kc + row0 * ak, J.kn + row0 * nbk, J.kh + row0 * 8,
-                               J.vc + row0 * av, J.vn + row0 * nbv, J.vh + row0 * 8};
-      const int rb[6] = {ak, nbk, hkb, av, nbv, hvb};
-      const int off[6] = {0, S_KN, S_KH, S_VA, S_VN, S_VH};
-#pragma unroll
-      for (int g = 0; g < 6; ++g) {
-        const int full = kAttBatch * rb[g], valid = rows * rb[g];
-        for (int c = lane * 16; c < full; c += 32 * 16) {
-          const int rem = valid - c;
-          const int n = rem >= 16 ? 16 : (rem > 0 ? rem : 0);
-          cp_async16(st + off[g] + c, n > 0 ? src[g] + c : src[g], n);
-        }
-      }
-    }
-    cp_async_commit();
-  };
-
-  // ---- lane constants ----
-  // K: lane (r, l) takes pairs 8l..8l+7 of token r of each pass of RW tokens;
-  // its 8 codes start at bit 8 W l of the row.  A code becomes the byte offset
-  // of its table entry (copy lane % 2^lgr) by one rotate and one mask.
-  const int r = lane / L, l = lane % L;
-  const int wk = J.wk, Tk = 3 + lgrk;
-  const int kbit = 8 * wk * l, kwa = kbit >> 5, ksa = kbit & 31;
-  const bool kup = ksa + 4 * wk >= 32;                    // codes 4..7 start in the next word
-  const int ksb = (ksa + 4 * wk) & 31;
-  const uint32_t kC = (uint32_t)(lane & ((1 << lgrk) - 1)) << 3;
-  const uint32_t kM = ((1u << wk) - 1u) << Tk;
-  int kra[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) kra[j] = (wk * j - Tk) & 31;
-  // V: lane owns pairs PV lane .. PV lane + PV - 1; its codes start at bit PV W lane.
-  const int wv = J.wv, Tv = 3 + lgrv;
-  const int vbit = PV * wv * lane, vwa = vbit >> 5, vsa = vbit & 31;
-  const uint32_t vC = (uint32_t)(lane & ((1 << lgrv) - 1)) << 3;
-  const uint32_t vM = ((1u << wv) - 1u) << Tv;
-  int vra[PV];
-#pragma unroll
-  for (int j = 0; j < PV; ++j) vra[j] = (wv * j - Tv) & 31;
-  const float kinv = J.inv_lk, vinv = J.inv_lv;
-  const bool vlog = J.mv == TAC_NORM_LOG;
-  const float v2b = J.mv == TAC_NORM_FP32 ? 0.f : (float)(1 << J.bv);
-
-  float m_run[NQ], l_run[NQ];
-  float2 acc[NQ][PV];
-#pragma unroll
-  for (int a = 0; a < NQ; ++a) {
-    m_run[a] = -INFINITY;
-    l_run[a] = 0.f;
-#pragma unroll
-    for (int j = 0; j < PV; ++j) acc[a][j] = make_float2(0.f, 0.f);
-  }
-
-  // Scores of the batch in `st`: after the passes and the reduction, lane
-  // (r, l) holds, for each query, the score of token RW l + r.
-  auto scores = [&](const uint8_t* st, float (&keep)[NQ], auto kc_) {
-    constexpr int KC = decltype(kc_)::value;
-    constexpr bool F32 = KC == 4, LOG = KC == 1 || KC == 3;
-    constexpr int KB = KC <= 1 ? 4 : 8;
-    // Decoded norms r^ and packed angle codes of this lane's 8 pairs of one token.
-    auto load_row = [&](int row, uint32_t& x0, uint32_t& x1, float (&rh)[8]) {
-      const uint32_t* arow = reinterpret_cast<const uint32_t*>(st + row * ak);
-      const uint32_t w0 = arow[kwa], w1 = arow[kwa + 1], w2 = arow[kwa + 2];
-      x0 = __funnelshift_r(w0, w1, ksa);
-      x1 = kup ? __funnelshift_r(w1, w2, ksb) : __funnelshift_r(w0, w1, ksb);
-      if constexpr (F32) {
-        const float4* nr = reinterpret_cast<const float4*>(st + S_KN + row * nbk + 32 * l);
-        const float4 n0 = nr[0], n1 = nr[1];
-        rh[0] = n0.x; rh[1] = n0.y; rh[2] = n0.z; rh[3] = n0.w;
-        rh[4] = n1.x; rh[5] = n1.y; rh[6] = n1.z; rh[7] = n1.w;
-      } else {
-        const float2 ab = norm_ab(*reinterpret_cast<const float2*>(st + S_KH + row * 8), kinv, (float)(1 << KB), LOG);
-        uint32_t nw[2];
-        if constexpr (KB == 8) {
-          const uint2 v = *reinterpret_cast<const uint2*>(st + S_KN + row * nbk + 8 * l);
-          nw[0] = v.x; nw[1] = v.y;
-        } else {
-          nw[0] = nw[1] = *reinterpret_cast<const uint32_t*>(st + S_KN + row * nbk + 4 * l);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          constexpr uint32_t NM = ((1u << KB) - 1u) << (23 - KB);
-          const int bit = KB * j;
-          const uint32_t fb = (rotr(nw[bit >> 5], ((bit & 31) - (23 - KB)) & 31) & NM) | 0x3F800000u;
-          float v = __fmaf_rn(__uint_as_float(fb), ab.x, ab.y);
-          if constexpr (LOG) v = ex2_approx(v);
-          rh[j] = v;
-        }
-      }
-    };
-    auto ydec = [&](uint32_t x, int j, float rh) {
-      const uint32_t o = (rotr(x, kra[j & 3]) & kM) | kC;
-      const float2 c = *reinterpret_cast<const float2*>(reinterpret_cast<const uint8_t*>(tk) + o);
-      return mul2(make_float2(rh, rh), c);
-    };
-    // Partial scores of tokens kA RW + r and kB RW + r over this lane's pairs;
-    // each rotated-query granule is loaded once for both.
-    auto pass = [&](auto ka_, auto kb_, float (&pa)[NQ], float (&pb)[NQ]) {
-      uint32_t xa0, xa1, xb0, xb1;
-      float ra[8], rb[8];
-      load_row(decltype(ka_)::value * RW + r, xa0, xa1, ra);
-      load_row(decltype(kb_)::value * RW + r, xb0, xb1, rb);
-      float2 sa[NQ], sb[NQ];
-#pragma unroll
-      for (int a = 0; a < NQ; ++a) sa[a] = sb[a] = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const float2 ya0 = ydec(m < 2 ? xa0 : xa1, 2 * m, ra[2 * m]);
-        const float2 ya1 = ydec(m < 2 ? xa0 : xa1, 2 * m + 1, ra[2 * m + 1]);
-        const float2 yb0 = ydec(m < 2 ? xb0 : xb1, 2 * m, rb[2 * m]);
-        const float2 yb1 = ydec(m < 2 ? xb0 : xb1, 2 * m + 1, rb[2 * m + 1]);
-#pragma unroll
-        for (int a = 0; a < NQ; ++a) {
-          const float2* qa = qrot + a * C::QROW + 10 * l + 2 * m;
-          const float4 q = NQ >= 4 ? lds_f4_reload(qa) : *reinterpret_cast<const float4*>(qa);
-          sa[a] = __ffma2_rn(make_float2(q.x, q.y), ya0, sa[a]);
-          sa[a] = __ffma2_rn(make_float2(q.z, q.w), ya1, sa[a]);
-          sb[a] = __ffma2_rn(make_float2(q.x, q.y), yb0, sb[a]);
-          sb[a] = __ffma2_rn(make_float2(q.z, q.w), yb1, sb[a]);
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < NQ; ++a) {
-        pa[a] = sa[a].x + sa[a].y;
-        pb[a] = sb[a].x + sb[a].y;
-      }
-    };
-    att_tree<L, 0, 1, NQ>(pass, l, keep);
-  };
-
-  // V accumulation over the batch's valid tokens: acc += p_t y^V_t.
-  auto values = [&](const uint8_t* st, int valid, auto vc_) {
-    constexpr int VC = decltype(vc_)::value;
-    constexpr bool F32 = VC == 4, LOG = VC == 1 || VC == 3;
-    constexpr int VB = VC <= 1 ? 4 : 8;
-    constexpr uint32_t NM = ((1u << VB) - 1u) << (23 - VB);
-    const int nbit = PV * VB * lane, nwa = nbit >> 5;
-    int nra[PV];
-#pragma unroll
-    for (int j = 0; j < PV; ++j) nra[j] = ((nbit & 31) + VB * j - (23 - VB)) & 31;
+    // ---- staging: 32 rows of the K or V planes, zero-filled past the last token ----
+    auto copy_rows = [&](const uint8_t* src, uint8_t* dst, int row_bytes, int rows) {
+      const int full = kAttBatch * row_bytes, valid = rows * row_bytes;
+      if (rows == kAttBatch) {
 #pragma unroll 4
-    for (int t = 0; t < valid; ++t) {
-      const uint32_t* arow = reinterpret_cast<const uint32_t*>(st + S_VA + t * av);
-      const uint32_t x = __funnelshift_r(arow[vwa], arow[vwa + 1], vsa);
-      const uint8_t* prow = pb + t * C::PBROW;
-      float rh[PV];
-      if constexpr (F32) {
-        const float* nr = reinterpret_cast<const float*>(st + S_VN + t * nbv) + PV * lane;
-        if constexpr (PV == 2) {
-          const float2 v = *reinterpret_cast<const float2*>(nr);
-          rh[0] = v.x; rh[1] = v.y;
-        } else {
-          rh[0] = nr[0];
-        }
+        for (int c = lane * 16; c < full; c += 512) cp_async16(dst + c, src + c, 16);
       } else {
-        const float2 ab = *reinterpret_cast<const float2*>(prow);
-        const uint32_t w = reinterpret_cast<const uint32_t*>(st + S_VN + t * nbv)[nwa];
-#pragma unroll
-        for (int j = 0; j < PV; ++j) {
-          const uint32_t fb = (rotr(w, nra[j]) & NM) | 0x3F800000u;
-          float v = __fmaf_rn(__uint_as_float(fb), ab.x, ab.y);
-          if constexpr (LOG) v = ex2_approx(v);
-          rh[j] = v;
+        for (int c = lane * 16; c < full; c += 512) {
+          const int n = min(max(valid - c, 0), 16);
+          cp_async16(dst + c, n > 0 ? src + c : src, n);
         }
       }
-      float2 pp[NQ];
-#pragma unroll
-      for (int a = 0; a < NQ; a += 2) {
-        if (a + 1 < NQ) {
-          const float4 q = *reinterpret_cast<const float4*>(prow + 16 + 8 * a);
-          pp[a] = make_float2(q.x, q.y);
-          pp[a + 1] = make_float2(q.z, q.w);
-        } else {
-          pp[a] = *reinterpret_cast<const float2*>(prow + 16 + 8 * a);
-        }
+    };
+    auto issue_k = [&](int64_t row) {
+      if (row < seg_rows) {
+        const int rows = (int)min((int64_t)kAttBatch, J.tokens - row);
+        copy_rows(J.kc + row * ak, stk, ak, rows);
+        copy_rows(J.kn + row * nbk, st_kn, nbk, rows);
+        if (hkb) copy_rows(J.kh + row * 8, st_kh, 8, rows);
       }
-#pragma unroll
-      for (int j = 0; j < PV; ++j) {
-        const uint32_t o = (rotr(x, vra[j]) & vM) | vC;
-        const float2 cs = *reinterpret_cast<const float2*>(reinterpret_cast<const uint8_t*>(tv) + o);
-        const float2 y = mul2(make_float2(rh[j], rh[j]), cs);
-#pragma unroll
-        for (int a = 0; a < NQ; ++a) acc[a][j] = __ffma2_rn(pp[a], y, acc[a][j]);
+      cp_async_commit();
+    };
+    auto issue_v = [&](int64_t row) {
+      if (row < seg_rows) {
+        const int rows = (int)min((int64_t)kAttBatch, J.tokens - row);
+        copy_rows(J.vc + row * av, st_va, av, rows);
+        copy_rows(J.vn + row * nbv, st_vn, nbv, rows);
+        if (hvb) copy_rows(J.vh + row * 8, st_vh, 8, rows);
       }
+      cp_async_commit();
+    };
+    __syncthreads();                               // the previous segment's merge is done with the warps' memory
+    issue_k(row0);
+    issue_v(row0);
+
+    // ---- bin-centre tables (cos, sin)(2 pi k / n), 2^lgr copies: entry k copy c
+    // at k 2^lgr + c; entries n..2^W-1 repeat entry n-1 (codes >= n clamp) ----
+    const int lgrk = J.lgrk, lgrv = J.lgrv;
+    if (tab_nk != J.nk || tab_nv != J.nv) {
+      const int ek = 1 << J.wk, ev = 1 << J.wv;
+      for (int e = tid; e < ek + ev; e += kAttThreads) {
+        const bool v = e >= ek;
+        const int i = v ? e - ek : e, n = v ? J.nv : J.nk, lg = v ? lgrv : lgrk;
+        float2* tab = (v ? tv : tk) + (i << lg);
+        const float2 cs = cos_sin_q8(8 * min(i, n - 1), n);
+        for (int c = 0; c < (1 << lg); ++c) tab[c] = cs;
+      }
+      tab_nk = J.nk;
+      tab_nv = J.nv;
     }
-  };
-
-  issue(0);
-  for (int s = 0; s < nb; ++s) {
-    issue(s + 1);
-    cp_async_wait<1>();
-    __syncwarp();
-    const uint8_t* st = stg + (s % kAttNS) * stage;
-    const int valid = (int)min((int64_t)kAttBatch, t_stop - (t_begin + (int64_t)s * kAttBatch));
-
-    float keep[NQ];
-    switch (J.ck) {
-      case 0: scores(st, keep, IC<0>{}); break;
-      case 1: scores(st, keep, IC<1>{}); break;
-      case 2: scores(st, keep, IC<2>{}); break;
-      case 3: scores(st, keep, IC<3>{}); break;
-      default: scores(st, keep, IC<4>{}); break;
-    }
-
-    // ---- online softmax (base 2); lane (r, l) owns token t = RW l + r ----
-    const int t = RW * l + r;
-    const bool live = t < valid;
-    uint8_t* prow = pb + t * C::PBROW;
-    float pw[NQ];
+    // ---- rotated queries q' = H D_K q * scale * log2(e), one warp a query,
+    // scaled by 2^-e into [-2, 2) ----
+    if (warp < NQ) {
+      float2* const q2 = qrot + warp * P;
+      float* const qrow = reinterpret_cast<float*>(q2);
+      const int64_t off = (int64_t)warp * J.q_stride;
 #pragma unroll
-    for (int a = 0; a < NQ; ++a) {
-      const float sa = live ? keep[a] : -INFINITY;
-      float mx = sa;
+      for (int j = lane; j < D; j += 32) {
+        float x = 0.f;
+        if (warp < nq)
+          x = p.q_bf16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(J.q)[off + j])
+                       : reinterpret_cast<const float*>(J.q)[off + j];
+        qrow[j] = ((J.sk[j >> 5] >> (j & 31)) & 1u) ? -x : x;
+      }
+      warp_fwht<D>(qrow, lane);
+      float2 y[P / 32];
+      float mx = 0.f;
+      const float qs = J.scale * kLog2e * rsqrtf((float)D);
+#pragma unroll
+      for (int k = 0; k < P / 32; ++k) {           // in record (slot) order: slot i holds pair slot_pair(i)
+        y[k] = q2[slot_pair<D>(lane + 32 * k)];
+        y[k].x *= qs;
+        y[k].y *= qs;
+        mx = fmaxf(mx, fmaxf(fabsf(y[k].x), fabsf(y[k].y)));
+      }
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float mn = fmaxf(m_run[a], mx);
-      const float f = ex2_approx(m_run[a] - mn);   // m_run = -inf at first: f = 0
-      pw[a] = ex2_approx(sa - mn);
-      l_run[a] = __fmaf_rn(l_run[a], f, pw[a]);
-      m_run[a] = mn;
+      const int e = min(max(exp_of(mx), -126), 126);
+      const float sc = exp2i(-e);
+      __syncwarp();
 #pragma unroll
-      for (int j = 0; j < PV; ++j) acc[a][j] = mul2(acc[a][j], make_float2(f, f));
+      for (int k = 0; k < P / 32; ++k) q2[lane + 32 * k] = make_float2(y[k].x * sc, y[k].y * sc);
+      if (lane == 0) qscale[warp] = exp2i(e);
     }
-    if (live && J.mv != TAC_NORM_FP32)
-      *reinterpret_cast<float2*>(prow) = norm_ab(*reinterpret_cast<const float2*>(st + S_VH + t * 8), vinv, v2b, vlog);
-#pragma unroll
-    for (int a = 0; a < NQ; a += 2) {
-      if (a + 1 < NQ) *reinterpret_cast<float4*>(prow + 16 + 8 * a) = make_float4(pw[a], pw[a], pw[a + 1], pw[a + 1]);
-      else *reinterpret_cast<float2*>(prow + 16 + 8 * a) = make_float2(pw[a], pw[a]);
-    }
-    __syncwarp();
+    __syncthreads();
 
-    switch (J.cv) {
-      case 0: values(st, valid, IC<0>{}); break;
-      case 1: values(st, valid, IC<1>{}); break;
-      case 2: values(st, valid, IC<2>{}); break;
-      case 3: values(st, valid, IC<3>{}); break;
-      default: values(st, valid, IC<4>{}); break;
+    // ---- lane constants ----
+    // K: lane (g, t) decodes slots KP t .. KP t + KP - 1 of tokens g and g + 8 of
+    // each 16; codes 4 q .. 4 q + 3 start at bit wk (KP t + 4 q) of the row.  A
+    // code becomes the byte offset of its table entry (copy lane % 2^lgr) by one
+    // rotate and one mask.
+    const int wk = J.wk, Tk = 3 + lgrk;
+    const uint32_t kC = (uint32_t)(lane & ((1 << lgrk) - 1)) << 3;
+    const uint32_t kM = ((1u << wk) - 1u) << Tk;
+    int kra[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) kra[j] = (wk * j - Tk) & 31;
+    const uint8_t* const tkb = reinterpret_cast<const uint8_t*>(tk);
+    int koff[KP / 4], ksh[KP / 4];                 // word and shift of codes 4 q .. 4 q + 3
+#pragma unroll
+    for (int q = 0; q < KP / 4; ++q) {
+      const int bit = wk * (KP * t + 4 * q);
+      koff[q] = (bit >> 5) * 4;
+      ksh[q] = bit & 31;
     }
-    __syncwarp();
-  }
-  cp_async_wait<0>();
+    // V: lane (g, t) decodes slots VP g .. VP g + VP - 1 of tokens 4 t .. 4 t + 3 of each 16.
+    const int wv = J.wv, Tv = 3 + lgrv;
+    const uint32_t vC = (uint32_t)(lane & ((1 << lgrv) - 1)) << 3;
+    const uint32_t vM = ((1u << wv) - 1u) << Tv;
+    int vra[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) vra[j] = (wv * j - Tv) & 31;
+    const uint8_t* const tvb = reinterpret_cast<const uint8_t*>(tv);
+    int voff[VP / 4], vsh[VP / 4];
+#pragma unroll
+    for (int q = 0; q < VP / 4; ++q) {
+      const int bit = wv * (VP * g + 4 * q);
+      voff[q] = (bit >> 5) * 4;
+      vsh[q] = bit & 31;
+    }
+    const float kinv = J.inv_lk, vinv = J.inv_lv;
+    const bool klog = J.mk == TAC_NORM_LOG, vlog = J.mv == TAC_NORM_LOG;
+    // Query fragments: step ks takes the slots k_slot(ks, 0) and k_slot(ks, 1) of
+    // every lane's run: neighbours, or (4-bit norms, whose codes are unpacked four
+    // apart) slots four apart.
+    const bool k4 = J.ck <= 1;
+    uint32_t bq[KS][QT][2];
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = KP * t + (k4 ? 8 * (ks >> 2) + (ks & 3) + 4 * h : 2 * ks + h);
+        const float2 y = qrot[(QT == 1 ? g & 3 : g) * P + i];
+        __half xh, xl, yh, yl;
+        split_half(y.x, xh, xl);
+        split_half(y.y, yh, yl);
+        const uint32_t hi = h2_bits(__halves2half2(xh, yh)), lo = h2_bits(__halves2half2(xl, yl));
+        if constexpr (QT == 1) {
+          bq[ks][0][h] = g < 4 ? hi : lo;
+        } else {
+          bq[ks][0][h] = hi;
+          bq[ks][1][h] = lo;
+        }
+      }
+    // The lane's queries in the softmax: two neighbours, the same as its columns
+    // of the value accumulators.
+    const int q0 = QT == 1 ? 2 * (t & 1) : 2 * t;
+    const float qsc[2] = {qscale[q0], qscale[q0 + 1]};
 
-  // ---- the split's partial results: (max, sum, accumulator) per query ----
-  float* rec = ws + J.ws + (int64_t)(split - J.split0) * nq * att_rec_floats(D);
+    // Running softmax state of the lane's two queries (the same on every lane
+    // that owns them): m a whole number not more than 8 below the largest score
+    // (log2 units), l the lane's part of the sum of 2^(s - m); accumulators in
+    // units of 2^m / c, c a power of two (infinite while they are empty).
+    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, c_run[2] = {INFINITY, INFINITY};
+    float acc[QT][VP][4];
 #pragma unroll
-  for (int a = 0; a < NQ; ++a) {
-    float ls = l_run[a];
+    for (int x = 0; x < QT; ++x)
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
-    if (a < nq) {
-      float* ra = rec + a * att_rec_floats(D);
-      if (lane == 0) { ra[0] = m_run[a]; ra[1] = ls; }
+      for (int j = 0; j < VP; ++j)
 #pragma unroll
-      for (int j = 0; j < PV; ++j)   // accumulators are per slot; the record holds pairs in order
-        *reinterpret_cast<float2*>(ra + 2 + 2 * slot_pair<D>(PV * lane + j)) = acc[a][j];
+        for (int i = 0; i < 4; ++i) acc[x][j][i] = 0.f;
+
+    // fp32 norms: no header; the largest norm of each token of the batch sets its scale.
+    auto fp32_consts = [&](const uint8_t* norms, int row_bytes, float2* ab, float* scale) {
+      for (int i = 0; i < kAttBatch / 4; ++i) {
+        const int tok = 4 * i + (lane >> 3);
+        const float* nr = reinterpret_cast<const float*>(norms + tok * row_bytes) + VP * (lane & 7);
+        float mx = 0.f;
+#pragma unroll
+        for (int k = 0; k < VP; k += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(nr + k);
+          mx = fmaxf(fmaxf(fmaxf(mx, v.x), fmaxf(v.y, v.z)), v.w);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const int e = min(max(exp_of(mx), -126), 126);
+        if ((lane & 7) == 0) {
+          ab[tok] = make_float2(exp2i(-e), 0.f);
+          scale[tok] = exp2i(e);
+        }
+      }
+    };
+
+    // Scores of the staged batch.  Rows of the fragments are tokens, columns the
+    // queries (QT = 1: their hi and lo parts), the steps run over the slots.
+    // sv: QT = 1 tokens 16 (t / 2) + 8 (i / 2) + g, query q0 + (i & 1);
+    //     QT = 2 tokens 16 (i / 4) + 8 (i / 2 & 1) + g, query q0 + (i & 1).
+    auto scores = [&](float (&sv)[4 * QT], auto kc_) {
+      constexpr int KC = decltype(kc_)::value;
+      constexpr bool F32 = KC == 4, LOG = KC == 1 || KC == 3;
+      constexpr int KB = KC <= 1 ? 4 : 8, KW = F32 ? 1 : KP * KB / 32;
+      float s0[4], s1[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s0[i] = s1[i] = 0.f;
+#pragma unroll 1
+      for (int mt = 0; mt < 2; ++mt) {
+        uint32_t x[2][KP / 4], nw[2][KW];
+        float2 ab[2];
+        const float* nf[2] = {nullptr, nullptr};
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) {
+          const int row = 16 * mt + 8 * rr + g;
+          const uint8_t* arow = stk + row * ak;
+#pragma unroll
+          for (int q = 0; q < KP / 4; ++q) {
+            const uint32_t* aw = reinterpret_cast<const uint32_t*>(arow + koff[q]);
+            x[rr][q] = __funnelshift_r(aw[0], aw[1], ksh[q]);
+          }
+          ab[rr] = kc[row];
+          const uint8_t* nr = st_kn + row * nbk;
+          if constexpr (F32) {
+            nf[rr] = reinterpret_cast<const float*>(nr) + KP * t;
+          } else if constexpr (KW == 4) {
+            const uint4 v = *reinterpret_cast<const uint4*>(nr + 16 * t);
+            nw[rr][0] = v.x; nw[rr][1] = v.y; nw[rr][2] = v.z; nw[rr][3] = v.w;
+          } else if constexpr (KW == 2) {
+            const uint2 v = *reinterpret_cast<const uint2*>(nr + 8 * t);
+            nw[rr][0] = v.x; nw[rr][1] = v.y;
+          } else {
+            nw[rr][0] = *reinterpret_cast<const uint32_t*>(nr + 4 * t);
+          }
+        }
+        float ch[2][4], cl[4], cx[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ch[0][i] = ch[1][i] = cl[i] = cx[i] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          uint32_t ah[4], al[4];
+#pragma unroll
+          for (int rr = 0; rr < 2; ++rr) {
+            float rv[2];
+            if constexpr (F32) {
+              const float2 v = *reinterpret_cast<const float2*>(nf[rr] + 2 * ks);
+              rv[0] = v.x * ab[rr].x;
+              rv[1] = v.y * ab[rr].x;
+            } else {
+              uint32_t hb;
+              if constexpr (KB == 8) hb = __byte_perm(nw[rr][ks >> 1], 0x64646464u, (ks & 1) ? 0x4342 : 0x4140);
+              else hb = ((nw[rr][ks >> 2] >> (4 * (ks & 3))) & 0x000F000Fu) | 0x64006400u;
+              const float2 cc = __half22float2(__hsub2(h2_of(hb), h2_of(0x64006400u)));
+              rv[0] = __fmaf_rn(cc.x, ab[rr].x, ab[rr].y);
+              rv[1] = __fmaf_rn(cc.y, ab[rr].x, ab[rr].y);
+              if constexpr (LOG) { rv[0] = ex2_approx(rv[0]); rv[1] = ex2_approx(rv[1]); }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int i = (KB == 4 && !F32) ? 8 * (ks >> 2) + (ks & 3) + 4 * h : 2 * ks + h;
+              const uint32_t o = (rotr(x[rr][i >> 2], kra[i & 3]) & kM) | kC;
+              float2 nh, lo;
+              split_pair(rv[h], *reinterpret_cast<const float2*>(tkb + o), nh, lo);
+              ah[2 * h + rr] = h2_bits(__floats2half2_rn(nh.x, nh.y));
+              al[2 * h + rr] = h2_bits(__floats2half2_rn(lo.x, lo.y));
+            }
+          }
+          mma_f16(ch[ks & 1], ah, bq[ks][0][0], bq[ks][0][1]);
+          mma_f16(cl, al, bq[ks][0][0], bq[ks][0][1]);
+          if constexpr (QT == 2) mma_f16(cx, ah, bq[ks][QT - 1][0], bq[ks][QT - 1][1]);
+        }
+        if constexpr (QT == 1) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) { s0[i] = s1[i]; s1[i] = cl[i] - (ch[0][i] + ch[1][i]); }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            s0[i] = s1[i];
+            s1[i] = __fmaf_rn(cx[i], -0.00048828125f, cl[i] - (ch[0][i] + ch[1][i]));
+          }
+        }
+      }
+      if constexpr (QT == 1) {
+        // lanes t < 2 hold the hi parts of their queries, t >= 2 the lo parts of the same ones
+        const bool up = t >= 2;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float kept = up ? s1[i] : s0[i];
+          const float got = __shfl_xor_sync(0xffffffffu, up ? s0[i] : s1[i], 2);
+          sv[i] = __fmaf_rn(up ? kept : got, 0.00048828125f, up ? got : kept);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { sv[i] = s0[i]; sv[4 * (QT - 1) + i] = s1[i]; }
+      }
+    };
+
+    // Values: acc += sum_t w_t y^V_t.  Rows of the fragments are the (cos, sin) of
+    // slot VP g + j, columns the queries' weights, the steps run over the tokens.
+    auto values = [&](auto vc_) {
+      constexpr int VC = decltype(vc_)::value;
+      constexpr bool F32 = VC == 4, LOG = VC == 1 || VC == 3;
+      constexpr int VB = VC <= 1 ? 4 : 8;
+      constexpr bool N16 = VB == 4 && VP == 4 && !F32;   // a lane's norms of a token in 16 bits
+      constexpr int VW = F32 ? 1 : (VP * VB + 31) / 32;
+#pragma unroll 1
+      for (int kk = 0; kk < 2; ++kk) {
+        uint32_t x[4][VP / 4], nw[4][VW];
+        float2 ab[4];
+        const float* nf[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int tok = 16 * kk + 4 * t + i;
+          const uint8_t* arow = st_va + tok * av;
+#pragma unroll
+          for (int q = 0; q < VP / 4; ++q) {
+            const uint32_t* aw = reinterpret_cast<const uint32_t*>(arow + voff[q]);
+            x[i][q] = __funnelshift_r(aw[0], aw[1], vsh[q]);
+          }
+          ab[i] = vc[tok];
+          const uint8_t* nr = st_vn + tok * nbv;
+          nf[i] = reinterpret_cast<const float*>(nr) + VP * g;
+          if constexpr (F32) {
+          } else if constexpr (VW == 2) {
+            const uint2 v = *reinterpret_cast<const uint2*>(nr + 8 * g);
+            nw[i][0] = v.x; nw[i][1] = v.y;
+          } else if constexpr (N16) {
+            nw[i][0] = *reinterpret_cast<const uint16_t*>(nr + 2 * g);
+          } else {
+            nw[i][0] = *reinterpret_cast<const uint32_t*>(nr + 4 * g);
+          }
+        }
+        if constexpr (N16) {                       // the norms of two tokens in one word
+          nw[0][0] |= nw[1][0] << 16;
+          nw[2][0] |= nw[3][0] << 16;
+        }
+        uint32_t b[QT][2], nb[QT][2];
+#pragma unroll
+        for (int x2 = 0; x2 < QT; ++x2) {
+          const uint2 v = *reinterpret_cast<const uint2*>(pw + C::W_W + ((kk * QT + x2) * 8 + g) * 32 + 8 * t);
+          b[x2][0] = v.x; b[x2][1] = v.y;
+          nb[x2][0] = v.x ^ 0x80008000u; nb[x2][1] = v.y ^ 0x80008000u;
+        }
+#pragma unroll
+        for (int jj = 0; jj < VP / 2; ++jj) {      // two slots at a time
+          const int ja = (VB == 4 && !F32 && !N16) ? 8 * (jj >> 2) + (jj & 3) : 2 * jj;
+          const int js[2] = {ja, (VB == 4 && !F32 && !N16) ? ja + 4 : ja + 1};
+          float rv[4][2];
+          if constexpr (N16) {
+#pragma unroll
+            for (int i = 0; i < 4; i += 2)
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const uint32_t hb = ((nw[i][0] >> (4 * js[h])) & 0x000F000Fu) | 0x64006400u;
+                const float2 cc = __half22float2(__hsub2(h2_of(hb), h2_of(0x64006400u)));
+                rv[i][h] = __fmaf_rn(cc.x, ab[i].x, ab[i].y);
+                rv[i + 1][h] = __fmaf_rn(cc.y, ab[i + 1].x, ab[i + 1].y);
+              }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if constexpr (F32) {
+                const float2 v = *reinterpret_cast<const float2*>(nf[i] + 2 * jj);
+                rv[i][0] = v.x * ab[i].x;
+                rv[i][1] = v.y * ab[i].x;
+              } else {
+                uint32_t hb;
+                if constexpr (VB == 8) hb = __byte_perm(nw[i][(jj >> 1) % VW], 0x64646464u, (jj & 1) ? 0x4342 : 0x4140);
+                else hb = ((nw[i][0] >> (4 * (jj & 3))) & 0x000F000Fu) | 0x64006400u;
+                const float2 cc = __half22float2(__hsub2(h2_of(hb), h2_of(0x64006400u)));
+                rv[i][0] = __fmaf_rn(cc.x, ab[i].x, ab[i].y);
+                rv[i][1] = __fmaf_rn(cc.y, ab[i].x, ab[i].y);
+              }
+            }
+          }
+          if constexpr (LOG) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { rv[i][0] = ex2_approx(rv[i][0]); rv[i][1] = ex2_approx(rv[i][1]); }
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int j = js[h];
+            uint32_t ah[4], al[4];
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+              float2 n0, l0, n1, l1;
+              const uint32_t o0 = (rotr(x[i][j >> 2], vra[j & 3]) & vM) | vC;
+              const uint32_t o1 = (rotr(x[i + 1][j >> 2], vra[j & 3]) & vM) | vC;
+              split_pair(rv[i][h], *reinterpret_cast<const float2*>(tvb + o0), n0, l0);
+              split_pair(rv[i + 1][h], *reinterpret_cast<const float2*>(tvb + o1), n1, l1);
+              ah[i] = h2_bits(__floats2half2_rn(n0.x, n1.x));
+              ah[i + 1] = h2_bits(__floats2half2_rn(n0.y, n1.y));
+              al[i] = h2_bits(__floats2half2_rn(l0.x, l1.x));
+              al[i + 1] = h2_bits(__floats2half2_rn(l0.y, l1.y));
+            }
+#pragma unroll
+            for (int x2 = 0; x2 < QT; ++x2) {
+              float c[4];
+              if (x2 == 0) {
+                mma_f16_zero(c, al, b[x2][0], b[x2][1]);
+                mma_f16(c, ah, nb[x2][0], nb[x2][1]);
+              } else {
+                mma_f16_zero(c, ah, nb[x2][0], nb[x2][1]);
+              }
+              float2* a2 = reinterpret_cast<float2*>(acc[x2][j]);
+              a2[0] = add2(a2[0], make_float2(c[0], c[1]));
+              a2[1] = add2(a2[1], make_float2(c[2], c[3]));
+            }
+          }
+        }
+      }
+    };
+
+    for (; row0 < seg_rows; row0 += kAttUnit) {
+      const int valid = (int)min((int64_t)kAttBatch, J.tokens - row0);
+      cp_async_wait<1>();                          // this batch's K rows have landed
+      __syncwarp();
+      if (hkb) norm_consts(reinterpret_cast<const float2*>(st_kh)[lane], kinv, klog, kc[lane], ksc[lane]);
+      else fp32_consts(st_kn, nbk, kc, ksc);
+      __syncwarp();
+      float sv[NV];
+      switch (J.ck) {
+        case 0: scores(sv, IC<0>{}); break;
+        case 1: scores(sv, IC<1>{}); break;
+        case 2: scores(sv, IC<2>{}); break;
+        case 3: scores(sv, IC<3>{}); break;
+        default: scores(sv, IC<4>{}); break;
+      }
+      auto token = [&](int i) { return QT == 1 ? 16 * (t >> 1) + 8 * (i >> 1) + g : 16 * (i >> 2) + 8 * ((i >> 1) & 1) + g; };
+      bool over = false;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int tok = token(i);
+        sv[i] = tok < valid ? sv[i] * qsc[i & 1] * ksc[tok] : -INFINITY;
+        over |= !(sv[i] <= m_run[i & 1] + 8.f);
+      }
+      __syncwarp();                                // every lane is done with the K rows
+      issue_k(row0 + kAttUnit);
+
+      // ---- softmax (base 2): the reference m moves only when a score passes it by more than 8 ----
+      if (__any_sync(0xffffffffu, over)) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int i = q; i < NV; i += 2) mx = fmaxf(mx, sv[i]);
+#pragma unroll
+          for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          const float mn = fmaxf(m_run[q], ceilf(mx));
+          if (mn > m_run[q]) {
+            l_run[q] *= exp2_whole(m_run[q] - mn);
+            c_run[q] *= ex2_approx(mn - m_run[q]);   // whole (or infinite) argument: exact
+            m_run[q] = mn;
+          }
+        }
+      }
+      cp_async_wait<1>();                          // this batch's V rows have landed
+      __syncwarp();
+      if (hvb) norm_consts(reinterpret_cast<const float2*>(st_vh)[lane], vinv, vlog, vc[lane], vsc[lane]);
+      else fp32_consts(st_vn, nbv, vc, vsc);
+      __syncwarp();
+      // weights 2^(s - m) 2^e in the accumulators' units, which move only when a
+      // weight passes 2^8
+      float w[NV];
+      over = false;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const float pr = ex2_approx(sv[i] - m_run[i & 1]);
+        l_run[i & 1] += pr;
+        w[i] = pr * vsc[token(i)];
+        over |= !(w[i] * c_run[i & 1] <= 256.f);
+      }
+      if (__any_sync(0xffffffffu, over)) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float mx = 0.f;
+#pragma unroll
+          for (int i = q; i < NV; i += 2) mx = fmaxf(mx, w[i]);
+#pragma unroll
+          for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          if (!(mx * c_run[q] <= 256.f)) {
+            const float cn = exp2i(-(exp_of(mx) + 1));
+            const float f = cn / c_run[q];           // 0 for empty accumulators
+            c_run[q] = cn;
+#pragma unroll
+            for (int x = 0; x < QT; ++x)
+#pragma unroll
+              for (int j = 0; j < VP; ++j) {
+                acc[x][j][q] *= f;
+                acc[x][j][2 + q] *= f;
+              }
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        __half hi, lo;
+        split_half(w[i] * c_run[i & 1], hi, lo);
+        const int tok = token(i), q = q0 + (i & 1);
+        __half* base = reinterpret_cast<__half*>(pw + C::W_W) + (tok >> 4) * QT * 128 + (tok & 15);
+        base[q * 16] = hi;
+        base[(QT == 1 ? q + 4 : q + 8) * 16] = lo;
+      }
+      __syncwarp();
+      switch (J.cv) {
+        case 0: values(IC<0>{}); break;
+        case 1: values(IC<1>{}); break;
+        case 2: values(IC<2>{}); break;
+        case 3: values(IC<3>{}); break;
+        default: values(IC<4>{}); break;
+      }
+      __syncwarp();                                // every lane is done with the V rows and the weights
+      issue_v(row0 + kAttUnit);
+    }
+    cp_async_wait<0>();
+
+    // ---- merge the warps: the segment's (max, sum, accumulator) per query ----
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) l_run[q] += __shfl_xor_sync(0xffffffffu, l_run[q], o);
+    __syncthreads();                               // every warp is done with its memory and the queries
+    float* const red = reinterpret_cast<float*>(smem);        // [warp][NQ][2]: m, l
+    if (g == 0 && (QT == 2 || t < 2)) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        red[(warp * NQ + q0 + q) * 2] = m_run[q];
+        red[(warp * NQ + q0 + q) * 2 + 1] = l_run[q];
+      }
+    }
+    __syncthreads();
+    float* const mrg = reinterpret_cast<float*>(wbase);       // [warp][NQ][D]
+    float f[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float M = -INFINITY;
+#pragma unroll
+      for (int x = 0; x < kAttWarps; ++x) M = fmaxf(M, red[(x * NQ + q0 + q) * 2]);
+      // an empty warp (no tokens) has m = -inf, c = inf and adds nothing; NaN scores stay NaN
+      f[q] = m_run[q] == -INFINITY && M > -INFINITY ? 0.f : exp2_whole(m_run[q] - M) * (1.f / c_run[q]);
+      if (M == -INFINITY) f[q] = 1.f;
+    }
+#pragma unroll
+    for (int j = 0; j < VP; ++j) {
+      const int at = 2 * slot_pair<D>(VP * g + j);
+      float o[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if constexpr (QT == 1) {
+          const float a = acc[0][j][i] * f[i & 1];
+          const float b = __shfl_xor_sync(0xffffffffu, a, 2);   // hi lanes t < 2, lo lanes t >= 2
+          o[i] = __fmaf_rn(b, 0.00048828125f, a);
+        } else {
+          o[i] = __fmaf_rn(acc[QT - 1][j][i], 0.00048828125f, acc[0][j][i]) * f[i & 1];
+        }
+      }
+      if (QT == 2 || t < 2) {
+        float* d0 = mrg + (warp * NQ + q0) * D + at;
+        *reinterpret_cast<float2*>(d0) = make_float2(o[0], o[2]);
+        *reinterpret_cast<float2*>(d0 + D) = make_float2(o[1], o[3]);
+      }
+    }
+    __syncthreads();
+    float* const rec = ws + J.ws + (int64_t)seg * nq * att_rec_floats(D);
+    for (int e = tid; e < nq * D; e += kAttThreads) {
+      const int a = e / D, j = e % D;
+      float s = 0.f;
+#pragma unroll
+      for (int x = 0; x < kAttWarps; ++x) s += mrg[(x * NQ + a) * D + j];
+      rec[a * att_rec_floats(D) + 2 + j] = s;
+    }
+    if (tid < nq) {
+      float M = -INFINITY, l = 0.f;
+#pragma unroll
+      for (int x = 0; x < kAttWarps; ++x) M = fmaxf(M, red[(x * NQ + tid) * 2]);
+#pragma unroll
+      for (int x = 0; x < kAttWarps; ++x) {
+        const float mw = red[(x * NQ + tid) * 2];
+        l += red[(x * NQ + tid) * 2 + 1] * (mw == M ? 1.f : exp2_whole(mw - M));
+      }
+      rec[tid * att_rec_floats(D)] = M;
+      rec[tid * att_rec_floats(D) + 1] = l;
     }
   }
 }
 
-// One CTA of 4 warps per (job, query): warp w merges splits w, w + 4, ...
+// One CTA of 4 warps per (job, query): warp w merges segments w, w + 4, ...
 // against the row's overall max, the warps' sums are added in shared memory,
 // and warp 0 normalizes, applies D H (fp32 butterfly) and stores the row.
 template <int D, typename TO>
-__global__ void __launch_bounds__(128) attend_combine(const __grid_constant__ AttParams p, const float* ws,
-                                                      int nrows_total) {
+__global__ void __launch_bounds__(128) attend_combine(const __grid_constant__ AttParams p, const float* ws) {
   constexpr int ESZ = (int)sizeof(TO);
   constexpr int E = D / 32;
   __shared__ float part[4][D];
   __shared__ float red[4][2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = blockIdx.x;                      // global (job, query) index
-  if (g >= nrows_total) return;
-  int jb = 0, base = 0;
-  for (; jb < p.njobs; ++jb) {
-    if (g < base + p.job[jb].nq) break;
-    base += p.job[jb].nq;
-  }
-  const AttJob& J = p.job[jb];
-  const int a = g - base;
-  const int nsp = (int)((J.tokens + kAttSplit - 1) / kAttSplit);
+  const AttJob& J = p.job[blockIdx.y];
+  const int a = blockIdx.x;
+  if (a >= J.nq) return;
+  const int last = J.unit0 + (int)((J.tokens + kAttUnit - 1) / kAttUnit) - 1;
+  const int nsp = att_cta_of(last, p.nunits, p.nctas) - att_cta_of(J.unit0, p.nunits, p.nctas) + 1;
   const float* recs = ws + J.ws + (int64_t)a * att_rec_floats(D);
-  const int64_t stride = (int64_t)J.nq * att_rec_floats(D);   // between splits
+  const int64_t stride = (int64_t)J.nq * att_rec_floats(D);   // between segments
+  // launched while the partial kernel runs: wait for its results
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   float M = -INFINITY;
   for (int s = threadIdx.x; s < nsp; s += 128) M = fmaxf(M, recs[s * stride]);
 #pragma unroll
@@ -511,7 +842,7 @@ __global__ void __launch_bounds__(128) attend_combine(const __grid_constant__ At
     const int j = lane + 32 * e;
     row[j] = (part[0][j] + part[1][j] + part[2][j] + part[3][j]) * inv;
   }
-  smem_fwht<D>(row, 1, lane, 32, false);
+  warp_fwht<D>(row, lane);
   const float sc = rsqrtf((float)D);
   uint8_t* orow = reinterpret_cast<uint8_t*>(J.out) + (int64_t)a * J.out_stride * ESZ;
 #pragma unroll
@@ -524,31 +855,12 @@ __global__ void __launch_bounds__(128) attend_combine(const __grid_constant__ At
   }
 }
 
-// Warps per CTA for a launch: the count (1..kAttMaxWarps) that keeps the most
-// warps resident per SM, given the CTA's shared memory (which grows with the
-// warps) and the kernel's registers; ties go to more warps per CTA.
-static int att_warps_per_cta(int smem_fixed, int smem_per_warp, int regs) {
-  constexpr int kSmemSM = 228 * 1024, kSmemCTA = 227 * 1024, kReserved = 1024;
-  const int regs_warp = ((regs * 32 + 255) / 256) * 256;
-  int best = 1, best_res = -1;
-  for (int w = 1; w <= kAttMaxWarps; ++w) {
-    const int sm = smem_fixed + w * smem_per_warp;
-    if (sm > kSmemCTA) break;
-    const int by_smem = kSmemSM / (sm + kReserved);
-    const int by_regs = 65536 / (regs_warp * w);
-    const int by_warps = 64 / w;
-    const int res = std::min(by_smem, std::min(by_regs, by_warps)) * w;
-    if (res >= best_res) { best_res = res; best = w; }
-  }
-  return best;
-}
-
-// Launches the partial and combine kernels for one group of jobs.  The CTA
-// assignment (cta0 per job, nctas) is made here, after the warps per CTA.
-template <int D, typename TQ, int NQ>
-static cudaError_t launch_attend_t(const AttParams& p_in, int nrows_total, float* ws, cudaStream_t st) {
-  using C = Att<D, NQ>;
-  auto kp = attend_partial<D, NQ>;
+// Launches the partial and combine kernels for one group of jobs.  The grid
+// is every CTA that fits on the device at once, or one per unit.
+template <int D, typename TQ, int QT>
+static cudaError_t launch_attend_t(const AttParams& p_in, int nq_max, float* ws, int sms, cudaStream_t st) {
+  using C = Att<D, QT>;
+  auto kp = attend_partial<D, QT>;
   // per device, set on the first launch; atomic so that host threads making
   // first calls at once do not race (each sets the same values)
   static std::atomic<int> regs[64];
@@ -564,25 +876,33 @@ static cudaError_t launch_attend_t(const AttParams& p_in, int nrows_total, float
     regs[dev].store(fa.numRegs > 0 ? fa.numRegs : 1, std::memory_order_release);
   }
   AttParams p = p_in;
-  int stage = 0;
+  p.stage = p.tab_k = p.tab_v = 0;
   for (int j = 0; j < p.njobs; ++j) {
     const AttJob& J = p.job[j];
-    stage = std::max(stage, att_stage_bytes(D, J.wk, J.bk, J.mk, J.wv, J.bv, J.mv));
+    p.stage = std::max(p.stage, att_stage_bytes(D, J.wk, J.bk, J.mk, J.wv, J.bv, J.mv));
+    p.tab_k = std::max(p.tab_k, 8 << (J.wk + J.lgrk));
+    p.tab_v = std::max(p.tab_v, 8 << (J.wv + J.lgrv));
   }
-  const int wpc = att_warps_per_cta(C::smem(stage, 0), C::smem(stage, 1) - C::smem(stage, 0), regs[dev].load(std::memory_order_relaxed));
-  int64_t ctas = 0;
-  for (int j = 0; j < p.njobs; ++j) {
-    AttJob& J = p.job[j];
-    const int64_t ns = (J.tokens + kAttSplit - 1) / kAttSplit;
-    J.cta0 = (int32_t)ctas;
-    ctas += (ns + wpc - 1) / wpc;
-  }
-  p.nctas = (int32_t)ctas;
-  if (p.nctas > 0) kp<<<p.nctas, 32 * wpc, C::smem(stage, wpc), st>>>(p, ws);
+  const int smem = C::smem(p.stage, p.tab_k + p.tab_v);
+  const int regs_cta = ((regs[dev].load(std::memory_order_relaxed) * 32 + 255) / 256) * 256 * kAttWarps;
+  const int per_sm = std::max(1, std::min(228 * 1024 / (smem + 1024), 65536 / regs_cta));
+  p.nctas = (int32_t)std::min<int64_t>(p.nunits, (int64_t)sms * per_sm);
+  if (p.nctas < 1) return cudaSuccess;
+  kp<<<p.nctas, kAttThreads, smem, st>>>(p, ws);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (nrows_total > 0) attend_combine<D, TQ><<<nrows_total, 128, 0, st>>>(p, ws, nrows_total);
-  return cudaGetLastError();
+  // the combine kernel starts as the partial kernel's CTAs leave and waits for
+  // its results on the device: its launch latency overlaps the partial kernel
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nq_max, (unsigned)p.njobs);
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, attend_combine<D, TQ>, p, (const float*)ws);
 }
 
 // The workspace of tac_attend_multi_static: one array per device, in the
@@ -608,15 +928,13 @@ cudaError_t attend_static_workspace(float** ws) {
   return cudaSuccess;
 }
 
-// nq_max: the largest query count of the jobs (the kernel is built for 1, 2, 4, 8).
-cudaError_t launch_attend(int d, int dtype, int nq_max, const AttParams& p, int nrows_total, float* ws,
+// nq_max: the largest query count of the jobs (the kernel is built for up to 4 and up to 8).
+cudaError_t launch_attend(int d, int dtype, int nq_max, const AttParams& p, float* ws, int sms,
                           cudaStream_t st) {
   const bool bf = dtype == TAC_BF16;
-#define TAC_ATT_NQ(DD, T)                                                           \
-  if (nq_max <= 1) return launch_attend_t<DD, T, 1>(p, nrows_total, ws, st);        \
-  if (nq_max <= 2) return launch_attend_t<DD, T, 2>(p, nrows_total, ws, st);        \
-  if (nq_max <= 4) return launch_attend_t<DD, T, 4>(p, nrows_total, ws, st);        \
-  return launch_attend_t<DD, T, 8>(p, nrows_total, ws, st);
+#define TAC_ATT_NQ(DD, T)                                                                 \
+  return nq_max <= 4 ? launch_attend_t<DD, T, 1>(p, nq_max, ws, sms, st)              \
+                     : launch_attend_t<DD, T, 2>(p, nq_max, ws, sms, st);
   if (d == 64) { if (bf) { TAC_ATT_NQ(64, __nv_bfloat16) } else { TAC_ATT_NQ(64, float) } }
   if (d == 128) { if (bf) { TAC_ATT_NQ(128, __nv_bfloat16) } else { TAC_ATT_NQ(128, float) } }
 #undef TAC_ATT_NQ

@@ -20,28 +20,30 @@ struct AttJob {
   int32_t lgrk, lgrv;                // log2 of the bin-centre table copies (K, V)
   int32_t ck, cv;                    // norm case (att_norm_case) of K and V
   uint32_t sk[4], sv[4];             // D of K and of V
-  int32_t split0;                    // first global split of this job
-  int32_t cta0;                      // first CTA of this job
+  int32_t unit0;                     // first unit (of TAC_ATTEND_SPLIT tokens) of this job in the launch
   int64_t ws;                        // first workspace float of this job
 };
 
 struct AttParams {
   int32_t njobs;
   int32_t nctas;
-  int32_t nsplits;
+  int32_t nunits;
+  int32_t stage, tab_k, tab_v;       // shared memory: a warp's staged batch, the two tables (largest of the jobs)
   int32_t q_bf16;                    // queries (and outputs) are bf16 rows, else fp32
   AttJob job[TAC_ATTEND_MAX_JOBS];   // 200 bytes each: within the 32 KB of kernel parameters
 };
 
-// Per-split workspace record: max (log2 units), sum, accumulator (d floats).
+// Workspace record of one segment (a CTA's tokens of one job) and query: max
+// (log2 units), sum, accumulator (d floats).  A job has at most one segment per
+// TAC_ATTEND_SPLIT tokens.
 __host__ __device__ constexpr int att_rec_floats(int d) { return d + 2; }
 
-// Attention staging: a warp takes its split in batches of 32 tokens; one
-// staged batch holds 32 rows of each record plane (K angle | K norm | K header |
-// V angle | V norm | V header, headers absent for fp32 norms) plus 16 bytes of
-// slack for word reads past a row's end.
+// Attention staging: a warp takes its tokens in batches of 32; a staged batch
+// holds 32 rows of each record plane (K angle | K norm | K header | V angle |
+// V norm | V header, headers absent for fp32 norms) plus 16 bytes of slack for
+// word reads past a row's end.
 constexpr int kAttBatch = 32;
-constexpr int kAttTabBytes = 4096;   // per bin-centre table, all copies
+constexpr int kAttTabBytes = 16384;  // at most, per bin-centre table, all copies
 __host__ __device__ inline int att_stage_bytes(int d, int wk, int bk, int mk, int wv, int bv, int mv) {
   const int P = d / 2;
   return kAttBatch * (P * wk / 8 + P * bk / 8 + (mk != TAC_NORM_FP32 ? 8 : 0) + P * wv / 8 + P * bv / 8 +

@@ -1,0 +1,77 @@
+"""Attention from records at the edges of the kernel's tiles: every norm storage
+of K and V, batches of 32 and units of 256 tokens and their remainders, jobs that
+span several CTAs and CTAs that span several jobs, and value rows whose scale
+varies by 2^40 from token to token (the running scales of the accumulators).
+
+Same oracle and tolerance as test_gpu_attend.
+"""
+import math
+
+import numpy as np
+import pytest
+
+import parity
+import test_gpu_attend as base
+
+pytestmark = pytest.mark.gpu
+
+NORMS = [(4, 0), (4, 1), (8, 0), (8, 1), (32, 2)]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("nq", [3, 7])
+def test_norm_storage_and_batch_edges(tac_gpu, orc, d, nq):
+    ns = [2, 16, 48, 128, 256]
+    spec = []
+    for i, kn in enumerate(NORMS):
+        for j, vn in enumerate(NORMS):
+            T = (1, 31, 32, 33, 255, 256, 257, 600)[(5 * i + j) % 8]
+            spec.append(dict(d=d, T=T, nq=nq, k=(ns[(i + j) % 5], *kn), v=(ns[(2 * i + j) % 5], *vn), seed=10 * i + j))
+    base._check(orc, tac_gpu, spec)
+
+
+@pytest.mark.parametrize("nq", [1, 8])
+def test_jobs_across_ctas(tac_gpu, orc, nq):
+    """More units than CTAs fit on the device at once, of jobs of very different lengths."""
+    lens = [9000, 1, 70001, 256, 5000, 31, 12345, 513]
+    spec = [dict(d=128, T=T, nq=nq, k=(64, 8, 0), v=(64, 4, 1), seed=i) for i, T in enumerate(lens)]
+    base._check(orc, tac_gpu, spec)
+
+
+@pytest.mark.parametrize("order", ["up", "down", "mixed"])
+def test_value_scales_per_token(tac_gpu, orc, order):
+    """The output is compared row by row against sum_t p_t |v^_t|, so tokens that
+    weigh little because their values are small must not disturb the others: the
+    error of an output element stays below 2^-18 of that sum (fp32 scores of
+    magnitude below 2^5 carry 2^-20, each weight and value 2^-22)."""
+    import torch
+    tac, d, T, nq = tac_gpu, 128, 700, 4
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    e = torch.linspace(-20, 20, T, device="cuda")
+    if order == "down":
+        e = e.flip(0)
+    elif order == "mixed":
+        e = e[torch.randperm(T, generator=g, device="cuda")]
+    xk = torch.randn((T, d), generator=g, device="cuda")
+    xv = torch.randn((T, d), generator=g, device="cuda") * torch.exp2(torch.round(e))[:, None]
+    kcfg, vcfg = tac.layer_cfg(d, 64, 8, 0, 0, 1, 0), tac.layer_cfg(d, 64, 8, 0, 0, 1, 1)
+    kc, vc = tac.encode(xk, kcfg), tac.encode(xv, vcfg)
+    # the first query attends to everything, the others ever more sharply to tokens
+    # of small values: along (a multiple of) the mean of their keys
+    small = xk[e < -10].mean(0)
+    q = torch.stack([0.2 * torch.randn(d, generator=g, device="cuda")] +
+                    [s * small * d / small.norm() ** 2 for s in (0.02, 0.05, 0.1)])
+    out = torch.empty_like(q)
+    tac.attend_multi([tac.AttendJob(kcfg, kc, vcfg, vc, T, q, out, 1.0 / math.sqrt(d))])
+    torch.cuda.synchronize()
+    kh = base._oracle_rows(orc, tac, kcfg, kc, T)
+    vh = base._oracle_rows(orc, tac, vcfg, vc, T)
+    q64 = parity.to_f64(q)
+    s = q64 @ kh.T / math.sqrt(d)
+    p = np.exp(s - s.max(1, keepdims=True))
+    p /= p.sum(1, keepdims=True)
+    want = orc.attend(q64, kh, vh, 1.0 / math.sqrt(d))
+    size = p @ np.linalg.norm(vh, axis=1)           # sum_t p_t ||v^_t||
+    err = np.abs(parity.to_f64(out) - want).max(1)
+    assert np.all(err <= 2.0**-18 * size), err / size

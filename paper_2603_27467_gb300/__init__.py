@@ -393,7 +393,7 @@ def _enc_workspace(jobs, workspace):
 
 def encode_multi(jobs, stream=None, workspace=None):
     """tac_encode_multi_ws: one encode launch and one fix-up launch per kernel
-    group (see launch_count); allocates the re-decision workspace (torch) when
+    group, or one launch for a small call (see launch_count); allocates the re-decision workspace (torch) when
     none is given.  Returns the workspace."""
     arr = _enc_array(jobs)
     workspace = _enc_workspace(jobs, workspace)
@@ -508,10 +508,11 @@ def attend_multi_static(jobs, stream=None):
 
 
 def launch_count(jobs) -> int:
-    """Kernel launches one encode_multi / decode_multi call makes for `jobs`:
-    jobs with rows are grouped by kernel (d, dtype, n, norm bits, norm mode),
-    at most MAX_JOBS jobs per group; a decode group is one launch, an encode
-    group two (the encode and its fix-up)."""
+    """Kernel launches one (not small) encode_multi / decode_multi call makes
+    for `jobs`: jobs with rows are grouped by kernel (d, dtype, n, norm bits,
+    norm mode), at most MAX_JOBS jobs per group; a decode group is one launch,
+    an encode group two (the encode and its fix-up).  A small encode call (see
+    tac_encode_multi) makes fewer: one per (d, dtype)."""
     groups: dict = {}
     per = 1
     for j in jobs:

@@ -390,10 +390,36 @@ struct DecGroup {
 
 namespace {
 
+constexpr int64_t kEncCtrBytes = 64, kEncEntryBytes = 32;
+int64_t enc_ovf_bytes(int64_t tile_rows_total) { return ((tile_rows_total + 127) / 128) * 16; }
+int64_t enc_job_bytes(int64_t njobs) { return ((njobs * (int64_t)sizeof(tac::EncJob) + 15) / 16) * 16; }
+// The part of a launch's workspace that must be there (see run_encode).
+int64_t enc_min_bytes(int64_t tile_rows_total, int64_t njobs) {
+  return kEncCtrBytes + enc_ovf_bytes(tile_rows_total) + enc_job_bytes(njobs);
+}
+
+// Small calls run on the kernel that takes every codebook shape: one launch for
+// each (d, dtype), which re-decides its own codes, instead of a launch and a
+// fix-up per shape, the workspace's zeroing (or allocation) and the helper
+// streams' events.  Its tiles take about 1.8 times the instructions, so the
+// limit grows with the launches it saves.  Measured (us, shape kernels / this
+// one): 4 shapes, d = 128, bf16: 128 tiles 37 / 12, 8192 tiles 38 / 21, 32768
+// tiles 58 / 47, 65536 tiles 78 / 84; one shape, d = 64, fp32 norms: 22000
+// tiles 31 / 29, 66000 tiles 54 / 70.
+constexpr int64_t kSmallEncodeTiles = 16384, kSmallEncodePerShape = 10240;
+constexpr int kSmallEncodeShapes = 4;
+
+// How an encode call is grouped into launches: by kernel shape, or (a small
+// call) by (d, dtype) alone.
+enum class EncPlan { kShapes, kSmallOrShapes };
+
 // Validates an encode call and groups its jobs by kernel: (d, dtype, n, norm
 // bits, norm mode), one launch per group and up to TAC_MAX_JOBS jobs each,
-// largest groups first.  Returns 0 or the call's tac status.
-int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vector<EncGroup>& groups) {
+// largest groups first.  With kSmallOrShapes a small call is grouped by (d,
+// dtype) alone, *small is set and *min_ws gets the workspace minimum of its
+// grouping by shape.  Returns 0 or the call's tac status.
+int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vector<EncGroup>& groups,
+                EncPlan how = EncPlan::kShapes, bool* small = nullptr, int64_t* min_ws = nullptr) {
   groups.clear();
   if (njobs < 0) return fail(TAC_E_INVAL, "%s: njobs = %d", who, njobs);
   if (njobs > 0 && !jobs) return fail(TAC_E_INVAL, "%s: jobs is NULL", who);
@@ -421,10 +447,34 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
     const tac_encode_job& J = jobs[j];
     return (((J.cfg.d * 4 + J.x.dtype) * 512 + J.cfg.n_angle) * 64 + J.cfg.norm_bits) * 4 + J.cfg.norm_mode;
   };
+  auto job_tiles = [&](int j) {
+    const int64_t tr = tile_rows(jobs[j].cfg.d);
+    return (jobs[j].x.rows + tr - 1) / tr;
+  };
   std::stable_sort(live.begin(), live.end(), [&](int a, int b) { return kernel_key(a) < kernel_key(b); });
+  int key_shift = 0;                                   // key bits that tell launches apart
+  if (how == EncPlan::kSmallOrShapes) {
+    int64_t total = 0;
+    int shapes = 0;
+    for (size_t k = 0; k < live.size(); ++k) {
+      total += job_tiles(live[k]);
+      shapes += k == 0 || kernel_key(live[k]) != kernel_key(live[k - 1]);
+    }
+    *small = total < kSmallEncodeTiles + kSmallEncodePerShape * std::min(shapes, kSmallEncodeShapes);
+    if (*small) {
+      key_shift = 17;                                  // (d, dtype)
+      *min_ws = 0;
+      for (size_t a = 0, b; a < live.size(); a = b) {  // the launches by shape: their counters, bitmaps, job tables
+        int64_t tiles = 0;
+        for (b = a; b < live.size() && b - a < TAC_MAX_JOBS && kernel_key(live[b]) == kernel_key(live[a]); ++b)
+          tiles += job_tiles(live[b]);
+        *min_ws += enc_min_bytes(tiles * tile_rows(jobs[live[a]].cfg.d), (int64_t)(b - a));
+      }
+    }
+  }
   size_t i = 0;
   while (i < live.size()) {
-    const int key = kernel_key(live[i]);
+    const int key = kernel_key(live[i]) >> key_shift;
     const tac_layer_cfg& c0 = jobs[live[i]].cfg;
     const int d = c0.d, dt = jobs[live[i]].x.dtype;
     groups.emplace_back();
@@ -433,10 +483,10 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
     tac::EncParams& P = G.p;
     std::memset(&P, 0, sizeof(P));
     int64_t tiles = 0;
-    while (i < live.size() && P.njobs < TAC_MAX_JOBS && kernel_key(live[i]) == key) {
+    while (i < live.size() && P.njobs < TAC_MAX_JOBS && (kernel_key(live[i]) >> key_shift) == key) {
       const tac_encode_job& J = jobs[live[i]];
       const int64_t tr = tile_rows(d);
-      const int64_t jt = (J.x.rows + tr - 1) / tr;
+      const int64_t jt = job_tiles(live[i]);
       if (tiles + jt > 0x7fffffff / tr) break;          // warp-tile rows must index in 31 bits
       tac::EncJob& E = P.job[P.njobs];
       E.x = J.x.data;
@@ -449,7 +499,7 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
       E.rows = J.x.rows;
       E.stride = J.x.row_stride;
       copy_signs(E.signs, &J.cfg);
-      E.w = tac::code_bits(J.cfg.n_angle);
+      E.n = J.cfg.n_angle;
       E.b = J.cfg.norm_bits;
       E.mode = J.cfg.norm_mode;
       E.tile0 = (int32_t)tiles;
@@ -474,14 +524,6 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
 // of every workload queue about one per 2400 pairs); with less room the
 // capacities shrink in proportion, down to none (then every row with a code to
 // re-decide is re-decided whole through the bitmap).
-constexpr int64_t kEncCtrBytes = 64, kEncEntryBytes = 32;
-int64_t enc_ovf_bytes(const EncGroup& G) {
-  const int64_t bits = (int64_t)G.p.ntiles * tile_rows(G.d);
-  return ((bits + 127) / 128) * 16;
-}
-int64_t enc_job_bytes(const EncGroup& G) {
-  return (((int64_t)G.p.njobs * (int64_t)sizeof(tac::EncJob) + 15) / 16) * 16;
-}
 int64_t enc_rec_cap(const EncGroup& G) {
   int64_t pairs = 0;
   for (int j = 0; j < G.p.njobs; ++j) pairs += G.p.job[j].rows * (G.d / 2);
@@ -494,8 +536,8 @@ EncWs enc_ws(const std::vector<EncGroup>& groups) {
   EncWs w;
   w.zero = kEncCtrBytes * (int64_t)groups.size();
   for (const EncGroup& G : groups) {
-    w.zero += enc_ovf_bytes(G);
-    w.jobs += enc_job_bytes(G);
+    w.zero += enc_ovf_bytes((int64_t)G.p.ntiles * tile_rows(G.d));
+    w.jobs += enc_job_bytes(G.p.njobs);
     w.rec_entries += enc_rec_cap(G);
   }
   w.min = w.zero + w.jobs;
@@ -519,8 +561,8 @@ int run_encode(std::vector<EncGroup>& groups, uint8_t* ws, int64_t ws_bytes, cud
     P.gq = reinterpret_cast<uint4*>(ws + q_off);
     P.gq_cap = cap;
     P.gjobs = reinterpret_cast<tac::EncJob*>(ws + job_off);
-    ovf_off += enc_ovf_bytes(groups[g]);
-    job_off += enc_job_bytes(groups[g]);
+    ovf_off += enc_ovf_bytes((int64_t)P.ntiles * tile_rows(groups[g].d));
+    job_off += enc_job_bytes(P.njobs);
     q_off += kEncEntryBytes * cap;
   }
   cudaError_t e = cudaMemsetAsync(ws, 0, (size_t)w.zero, st);
@@ -558,6 +600,26 @@ int run_encode(std::vector<EncGroup>& groups, uint8_t* ws, int64_t ws_bytes, cud
   return 0;
 }
 
+// Launches a planned small call: one kernel per group, no workspace.
+int run_encode_small(const std::vector<EncGroup>& groups, cudaStream_t st, const char* who) {
+  const int sms = num_sms();
+  if (sms <= 0) return fail(TAC_E_CUDA, "%s: no CUDA device", who);
+  GroupFork fork(st, (int)groups.size());
+  if (fork.error() != cudaSuccess) return fail(TAC_E_CUDA, "%s: %s", who, cudaGetErrorString(fork.error()));
+  for (size_t g = 0; g < groups.size(); ++g) {
+    const EncGroup& G = groups[g];
+    const cudaError_t e =
+        tac::launch_encode(G.d, G.dt, G.na, G.nb, G.mode, G.p, sms, fork.stream((int)g), tac::kEncAny);
+    if (e != cudaSuccess) {
+      fork.join();
+      return fail(TAC_E_CUDA, "%s: launch failed: %s", who, cudaGetErrorString(e));
+    }
+  }
+  const cudaError_t e = fork.join();
+  if (e != cudaSuccess) return fail(TAC_E_CUDA, "%s: %s", who, cudaGetErrorString(e));
+  return 0;
+}
+
 }  // namespace
 
 int64_t tac_encode_workspace_bytes(const tac_encode_job* jobs, int njobs, int64_t* min_bytes) {
@@ -573,27 +635,36 @@ int tac_encode_multi_ws(const tac_encode_job* jobs, int njobs, void* workspace, 
                         tac_stream_t stream) {
   static const char* who = "tac_encode_multi_ws";
   static thread_local std::vector<EncGroup> groups;
-  int rc = plan_encode(jobs, njobs, who, groups);
+  bool small = false;
+  int64_t min_ws = 0;
+  int rc = plan_encode(jobs, njobs, who, groups, EncPlan::kSmallOrShapes, &small, &min_ws);
   if (rc) return rc;
   if (groups.empty()) return ok();
-  const EncWs w = enc_ws(groups);
+  if (!small) min_ws = enc_ws(groups).min;
   if (!workspace || !aligned16(workspace)) return fail(TAC_E_INVAL, "%s: workspace NULL or not 16-byte aligned", who);
-  if (workspace_bytes < w.min)
+  if (workspace_bytes < min_ws)
     return fail(TAC_E_INVAL, "%s: workspace of %lld bytes < the minimum %lld", who, (long long)workspace_bytes,
-                (long long)w.min);
-  rc = run_encode(groups, static_cast<uint8_t*>(workspace), workspace_bytes, reinterpret_cast<cudaStream_t>(stream),
-                  who);
+                (long long)min_ws);
+  const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  rc = small ? run_encode_small(groups, st, who)
+             : run_encode(groups, static_cast<uint8_t*>(workspace), workspace_bytes, st, who);
   return rc ? rc : ok();
 }
 
 int tac_encode_multi(const tac_encode_job* jobs, int njobs, tac_stream_t stream) {
   static const char* who = "tac_encode_multi";
   static thread_local std::vector<EncGroup> groups;
-  int rc = plan_encode(jobs, njobs, who, groups);
+  bool small = false;
+  int64_t min_ws = 0;
+  int rc = plan_encode(jobs, njobs, who, groups, EncPlan::kSmallOrShapes, &small, &min_ws);
   if (rc) return rc;
   if (groups.empty()) return ok();
-  const EncWs w = enc_ws(groups);
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (small) {
+    rc = run_encode_small(groups, st, who);
+    return rc ? rc : ok();
+  }
+  const EncWs w = enc_ws(groups);
   void* ws = nullptr;
   cudaError_t e = cudaMallocAsync(&ws, (size_t)w.rec, st);
   if (e != cudaSuccess) return fail(TAC_E_CUDA, "%s: workspace allocation: %s", who, cudaGetErrorString(e));

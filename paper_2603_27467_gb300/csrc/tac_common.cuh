@@ -133,13 +133,16 @@ struct EncJob {
   int64_t rows;
   int64_t stride;      // elements
   uint32_t signs[4];
-  int32_t w;           // log2 n
-  int32_t b;           // norm bits (4 or 8)
-  int32_t mode;        // 0 linear, 1 log
+  int32_t n;           // angle bins
+  int32_t b;           // norm bits (4, 8, 32)
+  int32_t mode;        // tac_norm_mode
   int32_t tile0;       // first global tile of this job
 };
 
 static_assert(sizeof(EncJob) == 104 && sizeof(EncJob) % 8 == 0, "EncJob: the workspace copy is sized by it");
+
+// Phase of an encode launch that stands for the small-call kernel.
+constexpr int kEncAny = 4;
 
 struct EncParams {
   int32_t njobs;
@@ -188,6 +191,19 @@ struct DecParams {
   int32_t ntiles;
   DecJob job[TAC_MAX_JOBS];
 };
+
+// Largest power of two <= 16 that divides a record segment's row bytes: the
+// copy size of single records (each starts on a multiple of it).
+__host__ __device__ constexpr int row_chunk(int bytes) {
+  int c = 16;
+  while (bytes % c) c >>= 1;
+  return c;
+}
+template <int U> struct CopyUnit { using type = uint8_t; };
+template <> struct CopyUnit<2> { using type = uint16_t; };
+template <> struct CopyUnit<4> { using type = uint32_t; };
+template <> struct CopyUnit<8> { using type = uint2; };
+template <> struct CopyUnit<16> { using type = uint4; };
 
 // Job owning global tile t (jobs are sorted by tile0, job 0 starts at tile 0).
 template <typename Params>

@@ -65,14 +65,6 @@ struct Dec {
   static_assert(REC_W % 16 == 0 && W_TP % 16 == 0 && WARP_B % 16 == 0, "alignment");
 };
 
-// Largest power of two <= 16 that divides a record segment's row bytes: the
-// copy size of gathered records (each record starts on a multiple of it).
-__host__ __device__ constexpr int row_chunk(int bytes) {
-  int c = 16;
-  while (bytes % c) c >>= 1;
-  return c;
-}
-
 // Issue the copies of one segment (BYTES a row) of a tile's gathered records
 // into dst: the L lanes of row r copy its record `rec` in chunks of CB bytes
 // (rec = -1, a slot outside the cache: zero-filled).  Gathers are bound by

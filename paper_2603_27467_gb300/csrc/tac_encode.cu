@@ -34,6 +34,14 @@
 //      shared memory, moved to a queue in the call's workspace when it fills;
 //      a fix-up kernel after the encode re-decides them (a double-float second
 //      look, then exact integer sums of the row) and patches the records.
+// Small calls run the same code built once for every shape (AnyShape): latency
+// and launches bound them, so one launch takes all jobs of a (d, dtype), needs
+// no workspace, and re-decides its codes itself when its tiles are done, the
+// entries of a CTA's eight queues dealt to its warps.  One token for each of
+// 64 caches (8 rows each, four shapes) takes 12 us, 34 us as four launches and
+// four fix-ups; one token for each of 256 sequences 51 us, 67 us before.  The
+// slowest CTA's exact rows are the last 5 to 8 us (row load, 64-bit butterfly,
+// extremes and decision in a chain), the tiles 38 us.
 #include <algorithm>
 #include <atomic>
 
@@ -59,6 +67,22 @@ constexpr DfEdgeTable make_df_edge_table() {
 }  // namespace cx
 __constant__ cx::DfEdgeTable g_edge_df = cx::make_df_edge_table();
 
+// The same directions rounded to fp32, in global memory: the small-call
+// kernel's edge tables (any n) are a coalesced copy of it.
+namespace cx {
+struct EdgeTable { float2 v[kTabEntries]; };
+constexpr EdgeTable make_edge_table() {
+  EdgeTable t{};
+  for (int idx = 0; idx < kTabEntries; ++idx) {
+    const int n = tab_n_of(idx), e = idx - tab_offset_n(n);
+    const CS cs = cos_sin_q8(8 * e + 4 + n, n);
+    t.v[idx] = float2{(float)cs.c, (float)cs.s};
+  }
+  return t;
+}
+}  // namespace cx
+__device__ const cx::EdgeTable g_edge_f32 = cx::make_edge_table();
+
 constexpr int kNS = 4;  // pipeline stages per warp: kNS - 1 warp tiles in flight
 constexpr int kQ = 96;  // entries of a warp's re-decision queue
 // CTA shape of the encode: 8 warps, two CTAs per SM (16 warps, up to 128
@@ -68,20 +92,41 @@ constexpr int kQ = 96;  // entries of a warp's re-decision queue
 constexpr int kEncWarps = 8;
 constexpr int kEncThreads = 32 * kEncWarps;
 
-// Shape of one kernel: n bins (W = ceil(log2 n) bits per angle code), B norm
-// bits (4, 8, or 32 for fp32 norms), MODE; HB header bytes per row (8, none
-// for fp32 norms).
-template <int D, typename TIn, int N, int B, int MODE>
+// Codebook shape of a job: n bins (W = ceil(log2 n) bits per angle code), B norm
+// bits (4, 8, or 32 for fp32 norms), the norm mode.  A kernel is built for one
+// shape (FixedShape: every use folds at compile time) or for all of them
+// (AnyShape, read from the job: the kernel of small calls).
+template <int N_, int B_, int MODE_>
+struct FixedShape {
+  static constexpr bool fixed = true;
+  static constexpr int n = N_, W = code_bits(N_), B = B_, mode = MODE_;
+};
+struct AnyShape {
+  static constexpr bool fixed = false;
+  int n = 2, W = 1, B = 8, mode = 0;
+  __device__ __forceinline__ void set(const EncJob& J) {
+    n = J.n;
+    W = 32 - __clz(J.n - 1);
+    B = J.b;
+    mode = J.mode;
+  }
+};
+
+// The sizes a kernel's layout is made for: those of its shape, or the largest.
+template <class S> struct ShapeMax { static constexpr int W = S::W, B = S::B, H = S::mode == TAC_NORM_FP32 ? 0 : 8, n = S::n; };
+template <> struct ShapeMax<AnyShape> { static constexpr int W = kMaxW, B = 32, H = 8, n = kTabEntries; };
+
+// Layout of one kernel (AnyShape: record segments with room for the largest
+// records, and the edge directions of every supported n, one copy).
+template <int D, typename TIn, class S>
 struct Enc {
   using G = Geo<D>;
   using IT = RowTile<D, (int)sizeof(TIn)>;
   static constexpr int P = G::P, L = G::L, RW = G::RW;
   static constexpr int ESZ = (int)sizeof(TIn);
-  static constexpr int n = N;
-  static constexpr int W = code_bits(N);
-  static constexpr int AB = P * W / 8;        // angle record bytes per row
-  static constexpr int NB = P * B / 8;        // norm record bytes per row
-  static constexpr int HB = (MODE == TAC_NORM_FP32) ? 0 : 8;
+  static constexpr int AB = P * ShapeMax<S>::W / 8;   // angle record bytes per row
+  static constexpr int NB = P * ShapeMax<S>::B / 8;   // norm record bytes per row
+  static constexpr int HB = ShapeMax<S>::H;           // header bytes per row (none for fp32 norms)
   // A warp tile's records: RW*AB = 32 W and RW*NB = 32 B bytes, RW*HB header
   // bytes: every segment is a whole number of 16-byte chunks.
   static constexpr int NA = RW * AB / 16, NN = RW * NB / 16, NH = RW * HB / 16;
@@ -98,10 +143,11 @@ struct Enc {
   static constexpr int W_JOB = W_HDR + RW * HB;             // current job (WarpJob)
   static constexpr int W_RC = W_JOB + 64;                    // the rows' fp32 (smin, smax, ty) for the queue
   static constexpr int W_Q = W_RC + RW * 16;                 // re-decision queue (kQ entries of 32 bytes)
-  static constexpr int WARP_B = W_Q + kQ * 32;
-  static constexpr int TABR = tab_copies(n, 8192);           // edge table copies
-  static constexpr int OFF_TAB = kEncWarps * WARP_B;           // fp32 edge table of this n (TABR copies)
-  static constexpr int SMEM = OFF_TAB + n * TABR * 8;
+  static constexpr int W_X = W_Q + kQ * 32;                  // AnyShape: scratch of the exact path (2 P longs)
+  static constexpr int WARP_B = W_X + (S::fixed ? 0 : 16 * P);
+  static constexpr int TABR = S::fixed ? tab_copies(ShapeMax<S>::n, 8192) : 1;   // edge table copies
+  static constexpr int OFF_TAB = kEncWarps * WARP_B;           // fp32 edge table of this n (TABR copies), or all
+  static constexpr int SMEM = OFF_TAB + ShapeMax<S>::n * TABR * 8;
   static_assert((RW * AB) % 16 == 0 && (RW * NB) % 16 == 0 && (RW * HB) % 16 == 0, "record segments");
   static_assert(W_TP % 16 == 0 && W_ANG % 16 == 0 && W_JOB % 16 == 0 && WARP_B % 16 == 0, "alignment");
   static_assert(32 % CPR == 0 && RW % RPQ == 0, "chunk map");
@@ -115,7 +161,6 @@ struct WarpJob {
   uint8_t* hdr;
   const int64_t* slot;
   int64_t capacity;
-  uint32_t signs[4];
   int32_t job;         // its index in the launch's job table
 };
 static_assert(sizeof(WarpJob) <= 64, "WarpJob");
@@ -137,11 +182,27 @@ __device__ __forceinline__ void store_bytes(uint8_t* dst, uint32_t lo, uint32_t 
   }
 }
 
+// The low nbytes (<= 8) bytes of (hi:lo) to a shared address aligned to 2 when
+// nbytes is even.
+__device__ __forceinline__ void store_bytes_any(uint8_t* dst, uint32_t lo, uint32_t hi, int nbytes) {
+  if (nbytes & 1) {
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+      if (q < nbytes) dst[q] = (uint8_t)((q < 4 ? lo : hi) >> (8 * (q & 3)));
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (2 * q < nbytes) reinterpret_cast<uint16_t*>(dst)[q] = (uint16_t)((q < 2 ? lo : hi) >> (16 * (q & 1)));
+  }
+}
+
 // v mod n for v in [-n, 2n).
-template <int N>
-__device__ __forceinline__ int wrap_bin(int v) {
-  if constexpr (is_pow2(N)) return v & (N - 1);
-  else return v < 0 ? v + N : (v >= N ? v - N : v);
+template <class S>
+__device__ __forceinline__ int wrap_bin(const S& sh, int v) {
+  if constexpr (S::fixed) {
+    if constexpr (is_pow2(S::n)) return v & (S::n - 1);
+  }
+  return v < 0 ? v + sh.n : (v >= sh.n ? v - sh.n : v);
 }
 
 // Candidate edge for the pair (E, O) (butterfly halves, y = (E + O, E - O))
@@ -174,15 +235,24 @@ __device__ __forceinline__ int candidate_bits(float E, float O) {
 }
 
 // The candidate edge in [0, n).
-template <int N>
-__device__ __forceinline__ int candidate_edge(float E, float O) {
-  const int bits = candidate_bits<N>(E, O);
-  if constexpr (is_pow2(N)) {
-    return bits & (N - 1);
-  } else {
+template <class S>
+__device__ __forceinline__ int candidate_edge(const S& sh, float E, float O) {
+  if constexpr (S::fixed) {
+    const int bits = candidate_bits<S::n>(E, O);
+    if constexpr (is_pow2(S::n)) return bits & (S::n - 1);
     // 0x4B400000 = bits of M; the clamp keeps a zero pair's NaN inside [0, n).
-    const int e = wrap_bin<N>(bits - 0x4B400000);
-    return (int)min((uint32_t)e, (uint32_t)(N - 1));
+    return (int)min((uint32_t)wrap_bin(sh, bits - 0x4B400000), (uint32_t)(S::n - 1));
+  } else {
+    // candidate_bits for a runtime n, by the direct conversion; the angle lies in
+    // [-n/2, n/2] (or is NaN, which converts to 0), the edge in [-3 n/8 - 1, 5 n/8]
+    const float n = (float)sh.n, aE = fabsf(E), aO = fabsf(O);
+    const float t = (aO - aE) * rcp_approx(aO + aE);
+    const float nb = n * 0.15915494309189535f;
+    const float dq = __fmaf_rn(t, __fmaf_rn(t * t, -0.19194795f * nb, 0.97239412f * nb), -0.125f * n);
+    const float fb = 0.25f * n + __uint_as_float(__float_as_uint(dq) ^ (__float_as_uint(E) & 0x80000000u));
+    const float ab = __uint_as_float(__float_as_uint(fb) ^ (__float_as_uint(O) & 0x80000000u));
+    const int v = __float2int_rd(0.125f * n - ab);
+    return v + (v < 0 ? sh.n : 0);
   }
 }
 
@@ -192,19 +262,21 @@ __device__ __forceinline__ int candidate_edge(float E, float O) {
 // the cross product with the sign turned (k is the next bin when m < 0); its
 // magnitude is the certification margin, and a pair with m == 0 is never
 // certified, so which side the fast path gives it does not matter.
-template <int N, int R>
-__device__ __forceinline__ uint32_t edge_test(float E, float O, const float2* et, float& m) {
-  if constexpr (is_pow2(N)) {
-    const int bits = candidate_bits<N>(E, O);
-    const float2 dir = et[(bits & (N - 1)) * R];
-    m = __fmaf_rn(O, dir.y, -__fmul_rn(E, dir.x));
-    return (uint32_t)(bits + (int)(__float_as_uint(m) >> 31)) & (uint32_t)(N - 1);
-  } else {
-    const int e = candidate_edge<N>(E, O);
-    const float2 dir = et[e * R];
-    m = __fmaf_rn(O, dir.y, -__fmul_rn(E, dir.x));
-    return (uint32_t)wrap_bin<N>(e + (int)(__float_as_uint(m) >> 31));
+template <int R, class S>
+__device__ __forceinline__ uint32_t edge_test(const S& sh, float E, float O, const float2* et, float& m) {
+  if constexpr (S::fixed) {
+    if constexpr (is_pow2(S::n)) {
+      const int bits = candidate_bits<S::n>(E, O);
+      const float2 dir = et[(bits & (S::n - 1)) * R];
+      m = __fmaf_rn(O, dir.y, -__fmul_rn(E, dir.x));
+      return (uint32_t)(bits + (int)(__float_as_uint(m) >> 31)) & (uint32_t)(S::n - 1);
+    }
   }
+  const int e = candidate_edge(sh, E, O);
+  const float2 dir = et[e * R];
+  m = __fmaf_rn(O, dir.y, -__fmul_rn(E, dir.x));
+  const int k = e + (int)(__float_as_uint(m) >> 31);
+  return (uint32_t)(k == sh.n ? 0 : k);
 }
 
 // ---------------------------------------------------------------------------
@@ -255,7 +327,7 @@ __device__ __forceinline__ float2 df_mulf(float2 a, float b) {
   const float p = __fmul_rn(a.x, b);
   return df_fast2sum(p, __fmaf_rn(a.y, b, __fmaf_rn(a.x, b, -p)));
 }
-__device__ __forceinline__ float2 df_div(float2 a, float2 b) {
+static __device__ __noinline__ float2 df_div(float2 a, float2 b) {
   const float r = rcp_approx(b.x);                       // b.x normal and nonzero at every caller
   const float q1 = __fmul_rn(a.x, r);
   const float2 res = df_add(a, df_neg(df_mulf(b, q1)));  // a - q1 b
@@ -294,7 +366,7 @@ __device__ __forceinline__ float2 ll_to_df(long long v) {
 }
 
 // Pair energy E^2 + O^2 in double-float from the exact sums.
-__device__ __forceinline__ float2 df_energy(longlong2 eo) {
+static __device__ __noinline__ float2 df_energy(longlong2 eo) {
   const float2 e = ll_to_df(eo.x), o = ll_to_df(eo.y);
   return df_add(df_mul(e, e), df_mul(o, o));
 }
@@ -303,19 +375,19 @@ __device__ __forceinline__ float2 df_energy(longlong2 eo) {
 // from the fp32 polynomial on the leading parts, then the edge test
 // m = E cos psi - O sin psi in double-float against the double-float edge
 // direction (the code is the next bin when m >= 0).
-template <int N>
-__device__ __noinline__ int fix_angle_code(longlong2 eo) {
+template <class S>
+__device__ __noinline__ int fix_angle_code(S sh, longlong2 eo) {
   if (eo.x == 0 && eo.y == 0) return 0;  // pair (0, 0) -> bin 0
   const float2 e = ll_to_df(eo.x), o = ll_to_df(eo.y);
-  const int ec = candidate_edge<N>(e.x, o.x);
-  const float4 dir = g_edge_df.v[tab_offset_n(N) + ec];
+  const int ec = candidate_edge(sh, e.x, o.x);
+  const float4 dir = g_edge_df.v[tab_offset_n(sh.n) + ec];
   const float2 m = df_add(df_mul(e, make_float2(dir.x, dir.y)), df_neg(df_mul(o, make_float2(dir.z, dir.w))));
-  return wrap_bin<N>(ec + (df_sign(m) >= 0 ? 1 : 0));
+  return wrap_bin(sh, ec + (df_sign(m) >= 0 ? 1 : 0));
 }
 
 // log2 of a double-float >= 1, to about 2e-7 absolute: exponent plus log2 of
 // the leading part's significand plus the first-order term of the tail.
-__device__ __forceinline__ float df_log2_est(float2 a) {
+static __device__ __noinline__ float df_log2_est(float2 a) {
   const int e = (int)((__float_as_uint(a.x) >> 23) & 0xFFu) - 127;
   const float mh = a.x * pow2i(-e), ml = a.y * pow2i(-e);
   return (float)e + log2f(mh) + ml / mh * 1.4426950408889634f;
@@ -324,41 +396,49 @@ __device__ __forceinline__ float df_log2_est(float2 a) {
 // The exponent of a positive normal fp32 number.
 __device__ __forceinline__ int f32_exp(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFFu) - 127; }
 
-// a^n for a double-float a >= 1 and n >= 0, as m 2^e with m in [1, 2) (a
-// double-float) and an integer e: every product is brought back to [1, 2),
-// so nothing overflows for any n the codes need (n <= 2 * 255 + 1).
-__device__ __forceinline__ void df_pow(float2 a, int n, float2& m, int& e) {
-  int eb = f32_exp(a.x);
-  float2 b = df_scale(a, -eb);
-  m = make_float2(1.f, 0.f);
-  e = 0;
-  while (n) {
-    if (n & 1) {
-      m = df_mul(m, b);
-      e += eb;
-      const int k = f32_exp(m.x);
-      m = df_scale(m, -k);
-      e += k;
-    }
-    n >>= 1;
-    if (n) {
-      b = df_mul(b, b);
-      eb *= 2;
-      const int k = f32_exp(b.x);
-      b = df_scale(b, -k);
-      eb += k;
+// r1^n1 >= r2^n2 for double-floats r >= 1 and n >= 0, the two powers side by
+// side as m 2^e with m >= 1.  Significands are brought back to [1, 2) after
+// every product when an exponent passes 60, so nothing overflows (at most
+// m < 2^64 otherwise); the final ones always are.
+static __device__ __noinline__ bool df_pow_ge(float2 r1, int n1, float2 r2, int n2) {
+  const bool big = max(n1, n2) > 60;
+  float2 m[2] = {make_float2(1.f, 0.f), make_float2(1.f, 0.f)}, b[2] = {r1, r2};
+  int e[2] = {0, 0}, eb[2], n[2] = {n1, n2};
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    eb[x] = f32_exp(b[x].x);
+    b[x] = df_scale(b[x], -eb[x]);
+  }
+#pragma unroll 1
+  while (n[0] | n[1]) {
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      if (n[x] & 1) {
+        m[x] = df_mul(m[x], b[x]);
+        e[x] += eb[x];
+      }
+      n[x] >>= 1;
+      if (n[x]) {
+        b[x] = df_mul(b[x], b[x]);
+        eb[x] *= 2;
+      }
+      if (big) {
+        const int k = f32_exp(m[x].x), kb = f32_exp(b[x].x);
+        m[x] = df_scale(m[x], -k);
+        e[x] += k;
+        b[x] = df_scale(b[x], -kb);
+        eb[x] += kb;
+      }
     }
   }
-}
-
-// rho1^n1 >= rho2^n2 for double-floats rho >= 1 and n >= 0.
-static __device__ __noinline__ bool df_pow_ge(float2 r1, int n1, float2 r2, int n2) {
-  float2 m1, m2;
-  int e1, e2;
-  df_pow(r1, n1, m1, e1);
-  df_pow(r2, n2, m2, e2);
-  if (e1 != e2) return e1 > e2;                          // both significands in [1, 2)
-  return !df_less(m1, m2);
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int k = f32_exp(m[x].x);
+    m[x] = df_scale(m[x], -k);
+    e[x] += k;
+  }
+  if (e[0] != e[1]) return e[0] > e[1];                  // both significands in [1, 2)
+  return !df_less(m[0], m[1]);
 }
 
 // Eq. 2 code of a pair from double-float energies s = E^2 + O^2 (unnormalized:
@@ -373,11 +453,11 @@ static __device__ __noinline__ bool df_pow_ge(float2 r1, int n1, float2 r2, int 
 // linear by the sign of Lq (r - r_min) - (c - 1/2)(r_max - r_min) in
 // double-float; log-space by (s/s_lo)^(2 Lq) >= (s_max/s_lo)^(2c - 1), the
 // same inequality raised to integer powers.
-template <int B, int MODE>
-__device__ __noinline__ int fix_norm_code(float2 sa, float2 smn, float2 smx) {
-  constexpr int Lq = (1 << B) - 1;
+template <class S>
+__device__ __noinline__ int fix_norm_code(S sh, float2 sa, float2 smn, float2 smx) {
+  const int Lq = (1 << (sh.B & 15)) - 1;
   int c;
-  if constexpr (MODE == TAC_NORM_LINEAR) {
+  if (sh.mode == TAC_NORM_LINEAR) {
     const float2 a = df_sqrt(sa), m = df_sqrt(smn), M = df_sqrt(smx);
     const float2 A = df_add(a, df_neg(m)), R = df_add(M, df_neg(m));
     if (!(R.x > 0.f)) return 0;                          // r_max = r_min
@@ -387,8 +467,8 @@ __device__ __noinline__ int fix_norm_code(float2 sa, float2 smn, float2 smx) {
     const float2 w = df_add(df_div(df_mulf(A, (float)Lq), R), make_float2(0.5f, 0.f));
     c = (int)floorf(w.x);
     const float fr = __fadd_rn(__fsub_rn(w.x, (float)c), w.y);   // the double-float value is good to 1e-9
-    if (fr > 1e-6f && fr < 1.f - 1e-6f) return min(max(c, 0), Lq);
     c = min(max(c, 0), Lq);
+    if (fr > 1e-6f && fr < 1.f - 1e-6f) return c;
     while (c > 0 && !at_least(c)) --c;
     while (c < Lq && at_least(c + 1)) ++c;
   } else {
@@ -403,10 +483,15 @@ __device__ __noinline__ int fix_norm_code(float2 sa, float2 smn, float2 smx) {
     c = (int)floorf(v);
     const float fr = v - (float)c;
     const float tol = (float)Lq * 1e-6f / l2 + 1e-5f;      // the two estimates are good to 2e-7 each
-    if (fr > tol && fr < 1.f - tol) return min(max(c, 0), Lq);
     c = min(max(c, 0), Lq);
-    while (c > 0 && !at_least(c)) --c;
-    while (c < Lq && at_least(c + 1)) ++c;
+    if (fr > tol && fr < 1.f - tol) return c;
+    if (tol < 0.25f) {                                     // only the boundary it is close to is in doubt
+      const int edge = fr < 0.5f ? c : c + 1;
+      if (edge > 0 && edge <= Lq) c = at_least(edge) ? edge : edge - 1;
+    } else {
+      while (c > 0 && !at_least(c)) --c;
+      while (c < Lq && at_least(c + 1)) ++c;
+    }
   }
   return c;
 }
@@ -414,7 +499,7 @@ __device__ __noinline__ int fix_norm_code(float2 sa, float2 smn, float2 smx) {
 // Set bits [bit, bit + w) (w <= 8) of the byte stream at base to code, in
 // global memory.  Atomic on the aligned words they touch, so lanes that patch
 // different codes of one word do not lose each other's bits.
-__device__ __forceinline__ void patch_bits(uint8_t* base, int bit, int w, uint32_t code) {
+static __device__ __noinline__ void patch_bits(uint8_t* base, int bit, int w, uint32_t code) {
   const uintptr_t a = reinterpret_cast<uintptr_t>(base) + (uintptr_t)(bit >> 3);
   uint32_t* word = reinterpret_cast<uint32_t*>(a & ~(uintptr_t)3);
   const int sh = (int)(a & 3u) * 8 + (bit & 7);
@@ -459,11 +544,11 @@ __device__ __forceinline__ constexpr float norm_kappa() { return D >= 64 ? 0.015
 // that only the transform's error is left.  Returns the code when the Eq. 2
 // value lies farther than norm_kappa() times that bound from a rounding
 // midpoint, else -1.
-template <int D, int B, int MODE>
-__device__ __noinline__ int norm_second_look(float s, float smin, float smax, float ty) {
-  constexpr int Lq = (1 << B) - 1;
+template <int D, class S>
+__device__ __noinline__ int norm_second_look(S sh, float s, float smin, float smax, float ty) {
+  const int Lq = (1 << (sh.B & 15)) - 1;
   constexpr float kappa = norm_kappa<D>();
-  if constexpr (MODE == TAC_NORM_LINEAR) {
+  if (sh.mode == TAC_NORM_LINEAR) {
     const float2 m = df_sqrt(make_float2(smin, 0.f)), M = df_sqrt(make_float2(smax, 0.f));
     const float2 R = df_add(M, df_neg(m));
     if (!(R.x > 0.f)) return -1;
@@ -504,17 +589,17 @@ __device__ __noinline__ int norm_second_look(float s, float smin, float smax, fl
 // under the fast path's small-norm threshold (same expression, same value)
 // always go on to the exact path: their fp32 angle may be off by more than the
 // candidate edge allows for.
-template <int D, int N>
-__device__ __noinline__ int angle_second_look(float E, float O, float ty) {
+template <int D, class S>
+__device__ __noinline__ int angle_second_look(S sh, float E, float O, float ty) {
   const float s = __fmaf_rn(E, E, __fmul_rn(O, O));
-  const float rthr = ty * (4.f * (float)N / 3.14159265f);
+  const float rthr = ty * (4.f * (float)sh.n / 3.14159265f);
   if (s < rthr * rthr || !(s > 0.f)) return -1;
-  const int ec = candidate_edge<N>(E, O);
-  const float4 dir = g_edge_df.v[tab_offset_n(N) + ec];
+  const int ec = candidate_edge(sh, E, O);
+  const float4 dir = g_edge_df.v[tab_offset_n(sh.n) + ec];
   const float2 m = df_add(df_mulf(make_float2(dir.x, dir.y), E), df_neg(df_mulf(make_float2(dir.z, dir.w), O)));
   const float band = norm_kappa<D>() * ty * 1.001f + 1.0e-12f * sqrt_approx(s);
   if (!(fabsf(m.x) > band)) return -1;
-  return wrap_bin<N>(ec + (m.x > 0.f ? 1 : 0));
+  return wrap_bin(sh, ec + (m.x > 0.f ? 1 : 0));
 }
 
 // The words of one input row a lane takes for the exact path: for pair
@@ -618,7 +703,7 @@ __device__ __forceinline__ void exact_row(const FixWords<D, TIn>& f, long long* 
     }
   }
   __syncwarp();
-#pragma unroll
+#pragma unroll 1
   for (int lh = 0; (1 << lh) < P; ++lh) {
     const int h = 1 << lh;
 #pragma unroll
@@ -674,7 +759,7 @@ __device__ __noinline__ void exact_extremes(const long long* x, int lane, float2
   }
   const unsigned bmn = __ballot_sync(0xffffffffu, cmn), bmx = __ballot_sync(0xffffffffu, cmx);
   if (__popc(bmn) > 1 || __popc(bmx) > 1) {
-#pragma unroll
+#pragma unroll 1
     for (int off = 16; off > 0; off >>= 1) {
       const float2 omn = make_float2(__shfl_xor_sync(0xffffffffu, mn.x, off), __shfl_xor_sync(0xffffffffu, mn.y, off));
       const float2 omx = make_float2(__shfl_xor_sync(0xffffffffu, mx.x, off), __shfl_xor_sync(0xffffffffu, mx.y, off));
@@ -690,24 +775,22 @@ __device__ __noinline__ void exact_extremes(const long long* x, int lane, float2
   }
 }
 
-// Works through qn entries of the queue (all lanes of a warp call it), 32 at a
+// Works through qn entries of the queue (entry(e) its e-th; all lanes of a warp call it), 32 at a
 // time, one entry a lane: first the second look at each angle and norm code;
 // then, warp-wide and a row at a time, the exact transform of every row that
 // still has codes left (a row's entries are consecutive in the queue), from
 // which each lane takes its entry's exact sums and the row's exact extreme
 // energies; last, each lane decides its own code.  The records in global
 // memory are patched.  scratch: 2P longs of the warp's shared memory.
-template <int D, typename TIn, int N, int B, int MODE>
-__device__ __forceinline__ void flush_queue(const EncJob* jobs, const uint4* q, int qn, long long* scratch, int lane) {
+template <int D, typename TIn, class S, class Q>
+__device__ __forceinline__ void flush_queue(const EncJob* jobs, const Q& entry, int qn, long long* scratch, int lane) {
   constexpr int P = Geo<D>::P;
-  constexpr int W = code_bits(N);
-  constexpr bool FP32N = MODE == TAC_NORM_FP32;
-  constexpr int AB = P * W / 8, NB = P * (FP32N ? 32 : B) / 8;
-  auto record = [&](const EncJob& J, long long row, uint8_t*& codes, uint8_t*& norms) -> bool {
+  constexpr bool kNorms = ShapeMax<S>::H != 0;      // norm codes: not with a fixed shape of fp32 norms
+  auto record = [&](const S& sh, const EncJob& J, long long row, uint8_t*& codes, uint8_t*& norms) -> bool {
     const long long sl = J.slot ? J.slot[row] : row;
     if (sl < 0 || sl >= J.capacity) return false;   // skipped slots get no record
-    codes = J.codes + sl * AB;
-    norms = J.norms + sl * NB;
+    codes = J.codes + sl * (P * sh.W / 8);
+    norms = J.norms + sl * (P * sh.B / 8);
     return true;
   };
   auto row_src = [&](const EncJob& J, uint32_t row) {
@@ -719,26 +802,30 @@ __device__ __forceinline__ void flush_queue(const EncJob* jobs, const uint4* q, 
     uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
     uint32_t kind = 3u;
     if (e < qn) {
-      a = q[2 * e];
-      b = q[2 * e + 1];
+      const uint4* q = entry(e);
+      a = q[0];
+      b = q[1];
       kind = (a.x >> 14) & 3u;
     }
     const uint32_t ej = a.x & 0xFFu;
     const int v = (int)((a.x >> 8) & 63u);
+    S sh;                                            // this entry's shape
+    if constexpr (!S::fixed)
+      if (kind != 3u) sh.set(jobs[ej]);
     // ---- second look ----
     int c = -1;
     if (kind == 0u) {
-      c = angle_second_look<D, N>(__uint_as_float(a.z), __uint_as_float(a.w), __uint_as_float(b.y));
+      c = angle_second_look<D>(sh, __uint_as_float(a.z), __uint_as_float(a.w), __uint_as_float(b.y));
     } else if (kind == 1u) {
-      if constexpr (!FP32N)
-        c = norm_second_look<D, B, MODE>(__uint_as_float(a.z), __uint_as_float(a.w), __uint_as_float(b.x),
-                                         __uint_as_float(b.y));
+      if constexpr (kNorms)
+        c = norm_second_look<D>(sh, __uint_as_float(a.z), __uint_as_float(a.w), __uint_as_float(b.x),
+                                __uint_as_float(b.y));
     }
     if (c >= 0) {
       uint8_t *codes, *norms;
-      if (record(jobs[ej], (long long)a.y, codes, norms)) {
-        if (kind == 0u) patch_bits(codes, v * W, W, (uint32_t)c);
-        else patch_bits(norms, v * B, B, (uint32_t)c);
+      if (record(sh, jobs[ej], (long long)a.y, codes, norms)) {
+        if (kind == 0u) patch_bits(codes, v * sh.W, sh.W, (uint32_t)c);
+        else patch_bits(norms, v * sh.B, sh.B, (uint32_t)c);
       }
     }
     const bool need = kind != 3u && c < 0;
@@ -766,7 +853,7 @@ __device__ __forceinline__ void flush_queue(const EncJob* jobs, const uint4* q, 
       exact_row<D, TIn>(fw, scratch, lane);
       const bool mine = mys == rs;
       float2 rmn = make_float2(0.f, 0.f), rmx = make_float2(0.f, 0.f);
-      if constexpr (!FP32N) {
+      if constexpr (kNorms) {
         if (__ballot_sync(0xffffffffu, mine && kind != 0u) != 0u) exact_extremes<D>(scratch, lane, rmn, rmx);
       }
       if (mine) {
@@ -779,13 +866,16 @@ __device__ __forceinline__ void flush_queue(const EncJob* jobs, const uint4* q, 
       }
       if (__ballot_sync(0xffffffffu, mine && kind == 2u) != 0u) {   // the whole row, a pair a lane
         uint8_t *codes, *norms;
-        if (record(R, (long long)rr, codes, norms)) {
+        S rs_;                                       // the row's shape
+        if constexpr (!S::fixed) rs_.set(R);
+        if (record(rs_, R, (long long)rr, codes, norms)) {
           for (int ip = lane; ip < P; ip += 32) {
             const longlong2 pe = make_longlong2(scratch[ip], scratch[P + ip]);
             const int vs = pair_slot<D>(ip);
-            patch_bits(codes, vs * W, W, (uint32_t)fix_angle_code<N>(pe));
-            if constexpr (!FP32N)
-              patch_bits(norms, vs * B, B, (uint32_t)fix_norm_code<B, MODE>(df_energy(pe), rmn, rmx));
+            patch_bits(codes, vs * rs_.W, rs_.W, (uint32_t)fix_angle_code(rs_, pe));
+            if constexpr (kNorms)
+              if (rs_.mode != TAC_NORM_FP32)
+                patch_bits(norms, vs * rs_.B, rs_.B, (uint32_t)fix_norm_code(rs_, df_energy(pe), rmn, rmx));
           }
         }
       }
@@ -794,11 +884,12 @@ __device__ __forceinline__ void flush_queue(const EncJob* jobs, const uint4* q, 
     // ---- exact decisions, one entry a lane ----
     if (need && kind != 2u) {
       uint8_t *codes, *norms;
-      if (record(jobs[ej], (long long)a.y, codes, norms)) {
+      if (record(sh, jobs[ej], (long long)a.y, codes, norms)) {
         if (kind == 0u) {
-          patch_bits(codes, v * W, W, (uint32_t)fix_angle_code<N>(eo));
+          patch_bits(codes, v * sh.W, sh.W, (uint32_t)fix_angle_code(sh, eo));
         } else {
-          if constexpr (!FP32N) patch_bits(norms, v * B, B, (uint32_t)fix_norm_code<B, MODE>(df_energy(eo), smn, smx));
+          if constexpr (kNorms)
+            patch_bits(norms, v * sh.B, sh.B, (uint32_t)fix_norm_code(sh, df_energy(eo), smn, smx));
         }
       }
     }
@@ -828,24 +919,24 @@ __device__ __forceinline__ void spill_queue(const EncParams& p, const uint4* q, 
 }
 
 // Encode this lane's 8 pairs of warp-tile row r (lane l of the row) and stage
-// the records; N bins, B = norm bits, MODE = TAC_NORM_LINEAR / TAC_NORM_LOG /
-// TAC_NORM_FP32 (B = 32: the pair norms themselves, no header).
-template <int D, typename TIn, int N, int B, int MODE>
-__device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const float2* et, int nrows,
+// the records; sh: the codebook shape (norm mode TAC_NORM_FP32: B = 32, the pair
+// norms themselves, no header).
+template <int D, typename TIn, class S>
+__device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_t* wsm, const float2* et, int nrows,
                                           int lane, const uint2 (&msk)[8], uint4* q, int& qn, int t,
                                           const EncParams& p) {
   // bf16: msk[m].x holds the sign bits of the pair's two elements (bits 15
   // and 31), msk[m].y the low element's bit moved to bit 31.  The low element
   // widens as w * 2^16 + msk.y (adding bit 31 is an XOR of it: one integer
   // multiply-add), the high one as (w ^ msk.x) & 0xFFFF0000 (one logic op).
-  using C = Enc<D, TIn, N, B, MODE>;
+  using C = Enc<D, TIn, S>;
   using G = Geo<D>;
   using IT = typename C::IT;
   constexpr int P = C::P, L = C::L;
-  constexpr int n = N, W = C::W;
-  constexpr int AB = C::AB, NB = C::NB;
-  constexpr bool FP32N = MODE == TAC_NORM_FP32;
-  constexpr int Lq = FP32N ? 0 : (1 << B) - 1;
+  const int n = sh.n, W = sh.W, B = sh.B, mode = sh.mode;
+  const int AB = P * W / 8, NB = P * B / 8;
+  const bool fp32n = mode == TAC_NORM_FP32;
+  const int Lq = fp32n ? 0 : (1 << (B & 15)) - 1;
   const int r = lane / L, l = lane % L;
   const bool live = r < nrows;
   static_assert(P == 8 * L, "geometry");
@@ -927,13 +1018,23 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     float m;
-    const uint32_t k = edge_test<N, C::TABR>(v[j].x, v[j].y, et, m);
+    const uint32_t k = edge_test<C::TABR>(sh, v[j].x, v[j].y, et, m);
     am[j] = fabsf(m);
-    // fields are disjoint and k < n: the adds are ORs (one IMAD each)
-    const int sa = j * W;
-    if (sa + W <= 32) alo += k << sa;
-    else if (sa >= 32) ahi += k << (sa - 32);
-    else { alo += k << sa; ahi += k >> (32 - sa); }
+    if constexpr (S::fixed) {
+      // fields are disjoint and k < n: the adds are ORs (one IMAD each)
+      const int sa = j * S::W;
+      if (sa + S::W <= 32) alo += k << sa;
+      else if (sa >= 32) ahi += k << (sa - 32);
+      else { alo += k << sa; ahi += k >> (32 - sa); }
+    } else {
+      // four codes to a word (one integer multiply-add each)
+      if (j < 4) alo += k << (j * W);
+      else ahi += k << ((j - 4) * W);
+    }
+  }
+  if constexpr (!S::fixed) {                    // the words side by side: 4 W bits each
+    alo |= W == 8 ? 0u : ahi << (4 * W);
+    ahi = W == 8 ? ahi : ahi >> (32 - 4 * W);
   }
 
   const float mmin = min3(min3(am[0], am[1], am[2]), min3(am[3], am[4], am[5]), fminf(am[6], am[7]));
@@ -966,9 +1067,9 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
   constexpr bool kEvenK2 = D == 32 || D == 128;
   const float rms = sqrt_ftz(smax_s);
   float hmin = 0.f, hmax = 0.f, qs = 0.f, qo = 0.f, sfloor = 0.f, sc = 0.f;
-  if constexpr (FP32N) {
+  if (fp32n) {
     // no header: the norms are stored as they are (Sec. 3.1)
-  } else if constexpr (MODE == TAC_NORM_LINEAR) {
+  } else if (mode == TAC_NORM_LINEAR) {
     hmin = sqrt_approx(smin * k2);              // smin * sigma may still be subnormal
     hmax = (kEvenK2 ? rms * rk2 : sqrt_ftz(smax_s * k2)) * sr;
     sc = (float)Lq * rcp_approx(hmax - hmin);
@@ -1047,12 +1148,12 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
   // <= 2^-22 absolute on [1/2, 2), and within 4u |result| elsewhere (a GPU
   // test checks each of these limits over whole binades).
   constexpr float kEr = 3.f * kU, kEq = 4.f * kU, kEl = 2.384185791015625e-07f;  // 2^-22
-  constexpr float kMag = FP32N ? 0.f : (float)(1 << (B & 15));  // 2^B
-  constexpr int kFb = 23 - (FP32N ? 8 : B);                     // fraction bits of t + 2^B
-  constexpr uint32_t kFracMask = (1u << kFb) - 1u;
+  const float kMag = fp32n ? 0.f : (float)(1 << (B & 15));      // 2^B
+  const int kFb = 23 - (fp32n ? 8 : B);                         // fraction bits of t + 2^B
+  const uint32_t kFracMask = (1u << kFb) - 1u;
   float th = 0.f;
-  if constexpr (!FP32N) {
-    if constexpr (MODE == TAC_NORM_LINEAR) {
+  if (!fp32n) {
+    if (mode == TAC_NORM_LINEAR) {
       th = kKappa * 2.f * qs * ty + 2.f * kEr * (hmax + hmin) * sc + (float)Lq * kEq +
            kU * (hmin * sc + 4.f * kMag + 2.f);
     } else {
@@ -1071,26 +1172,39 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
   // ---- pass 2: norm codes (Eq. 2), packing ----
   uint32_t nlo = 0, nhi = 0;
   uint32_t nfr = 0xFFFFFFFFu;                   // smallest fraction field of t + th over the lane's pairs
-  float rn[FP32N ? 8 : 1];                      // fp32 norms r_j = sqrt(2 s_j / d)
+  float rn[8];                                  // fp32 norms r_j = sqrt(2 s_j / d), or f(s_j)
+  if (fp32n) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) rn[j] = sqrt_approx(s[j] * k2);
+  } else if (mode == TAC_NORM_LINEAR) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) rn[j] = sqrt_ftz(s[j]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) rn[j] = lg2_ftz(fmaxf(s[j], sfloor));
+  }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    if constexpr (FP32N) {
-      rn[j] = sqrt_approx(s[j] * k2);
-    } else {
-      float f;
-      if constexpr (MODE == TAC_NORM_LINEAR) f = sqrt_ftz(s[j]);
-      else f = lg2_ftz(fmaxf(s[j], sfloor));
-      const uint32_t tb = __float_as_uint(__fmaf_rn(f, qs, qo2));
+    if (!fp32n) {
+      const uint32_t tb = __float_as_uint(__fmaf_rn(rn[j], qs, qo2));
       nfr = min(nfr, tb & kFracMask);
       // code floor(t + th) = bits [kFb, kFb + B) of tb, moved to its field at
       // bit j B (a pair within th of a midpoint is re-decided below)
-      const int sn = j * B;
-      const int sh = kFb - (sn & 31);
-      const uint32_t part = (sh >= 0 ? (tb >> sh) : (tb << -sh)) & ((uint32_t)Lq << (sn & 31));
-      if (sn < 32) nlo |= part; else nhi |= part;
+      if constexpr (S::fixed) {
+        const int sn = j * B;
+        const int sft = kFb - (sn & 31);
+        const uint32_t part = (sft >= 0 ? (tb >> sft) : (tb << -sft)) & ((uint32_t)Lq << (sn & 31));
+        if (sn < 32) nlo |= part; else nhi |= part;
+      } else {
+        const uint32_t c = (tb >> kFb) & (uint32_t)Lq;
+        if (j < 4) nlo |= c << (j * B);
+        else nhi |= c << ((j - 4) * B);
+      }
     }
   }
-  const bool nflag = !FP32N && (nall || nfr < thb2);
+  if constexpr (!S::fixed)
+    if (B == 4) nlo |= nhi << 16;
+  const bool nflag = !fp32n && (nall || nfr < thb2);
   // fl: bits 0-7 name the angle codes to re-decide, bits 8-15 the norm codes
   uint32_t fl = 0;
   // a row whose energy sum is not finite may hold a NaN or an inf: its lanes
@@ -1117,12 +1231,12 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       if (am[j] < tau || s[j] < sthr) fl |= 1u << j;
-    if constexpr (!FP32N) {
+    if (!fp32n) {
       if (nflag) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           float f;
-          if constexpr (MODE == TAC_NORM_LINEAR) f = sqrt_ftz(s[j]);
+          if (mode == TAC_NORM_LINEAR) f = sqrt_ftz(s[j]);
           else f = lg2_ftz(fmaxf(s[j], sfloor));
           if (nall || (__float_as_uint(__fmaf_rn(f, qs, qo2)) & kFracMask) < thb2) fl |= 0x100u << j;
         }
@@ -1144,7 +1258,7 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
         fl = 0;
         alo = ahi = nlo = nhi = 0;
         hmin = hmax = qnan;
-        if constexpr (FP32N) {
+        if (fp32n) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) rn[j] = qnan;
         }
@@ -1202,13 +1316,18 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
 
   // ---- stage the records ----
   if (live) {
-    store_bytes<W>(wsm + C::W_ANG + r * AB + l * W, alo, ahi);
-    if constexpr (FP32N) {
+    if constexpr (S::fixed) store_bytes<ShapeMax<S>::W>(wsm + C::W_ANG + r * AB + l * W, alo, ahi);
+    else store_bytes_any(wsm + C::W_ANG + r * AB + l * W, alo, ahi, W);
+    if (fp32n) {
       float4* dst = reinterpret_cast<float4*>(wsm + C::W_NRM + r * NB + l * 32);
       dst[0] = make_float4(rn[0], rn[1], rn[2], rn[3]);
       dst[1] = make_float4(rn[4], rn[5], rn[6], rn[7]);
     } else {
-      store_bytes<B>(wsm + C::W_NRM + r * NB + l * B, nlo, nhi);
+      if constexpr (!S::fixed) {
+        uint8_t* dst = wsm + C::W_NRM + r * NB + l * B;
+        if (B == 8) *reinterpret_cast<uint2*>(dst) = make_uint2(nlo, nhi);
+        else *reinterpret_cast<uint32_t*>(dst) = nlo;
+      } else if constexpr (ShapeMax<S>::B <= 8) store_bytes<ShapeMax<S>::B>(wsm + C::W_NRM + r * NB + l * B, nlo, nhi);
       if (l == 0) reinterpret_cast<float2*>(wsm + C::W_HDR)[r] = make_float2(hmin, hmax);
     }
   }
@@ -1216,68 +1335,60 @@ __device__ __forceinline__ void tile_body(const uint8_t* in, uint8_t* wsm, const
 
 }
 
-// Records of a tail tile (nrows < RW) or of scattered slots, from the staged
-// records to the planes.
-template <int AB, int NB, int HB>
-__device__ __noinline__ void copy_out_slow(const WarpJob* wj, const uint8_t* sang, const uint8_t* snrm,
-                                           const uint8_t* shdr, int64_t row0, int nrows, int lane) {
-  if (wj->slot == nullptr) {
-    uint8_t* ga = wj->codes + row0 * AB;
-    uint8_t* gn = wj->norms + row0 * NB;
-    uint8_t* gh = wj->hdr + row0 * 8;
-    for (int q = lane; q < nrows * AB; q += 32) ga[q] = sang[q];
-    for (int q = lane; q < nrows * NB; q += 32) gn[q] = snrm[q];
-    if constexpr (HB > 0)
-      for (int q = lane; q < nrows * HB; q += 32) gh[q] = shdr[q];
-  } else if (lane < nrows) {
-    const int64_t s = wj->slot[row0 + lane];
-    if (s < 0 || s >= wj->capacity) return;  // out-of-range slots are skipped
-    uint8_t* ga = wj->codes + s * AB;
-    uint8_t* gn = wj->norms + s * NB;
-    const uint8_t* a = sang + lane * AB;
-    const uint8_t* nn = snrm + lane * NB;
-    if constexpr ((AB & 15) == 0) {
-      for (int q = 0; q < AB / 16; ++q) reinterpret_cast<uint4*>(ga)[q] = reinterpret_cast<const uint4*>(a)[q];
-    } else if constexpr ((AB & 7) == 0) {
-      for (int q = 0; q < AB / 8; ++q) reinterpret_cast<uint2*>(ga)[q] = reinterpret_cast<const uint2*>(a)[q];
-    } else if constexpr ((AB & 3) == 0) {
-      for (int q = 0; q < AB / 4; ++q) reinterpret_cast<uint32_t*>(ga)[q] = reinterpret_cast<const uint32_t*>(a)[q];
-    } else {
-      for (int q = 0; q < AB; ++q) ga[q] = a[q];
-    }
-    if constexpr ((NB & 7) == 0) {
-      for (int q = 0; q < NB / 8; ++q) reinterpret_cast<uint2*>(gn)[q] = reinterpret_cast<const uint2*>(nn)[q];
-    } else {
-      for (int q = 0; q < NB / 4; ++q) reinterpret_cast<uint32_t*>(gn)[q] = reinterpret_cast<const uint32_t*>(nn)[q];
-    }
-    if constexpr (HB > 0) reinterpret_cast<float2*>(wj->hdr)[s] = reinterpret_cast<const float2*>(shdr)[lane];
+// One segment (bytes of each row) of a tail tile's or scattered rows' records,
+// from the staged rows to the plane: the L lanes of a row copy it to record
+// rec (-1: none) in the largest pieces that its row size allows.
+template <int L, int BYTES>
+__device__ __forceinline__ void copy_row_fixed(uint8_t* plane, const uint8_t* staged, long long rec, int r, int l) {
+  constexpr int U = row_chunk(BYTES), PER = BYTES / U;
+  using T = typename CopyUnit<U>::type;
+  if (rec < 0) return;
+  T* dst = reinterpret_cast<T*>(plane + rec * BYTES);
+  const T* src = reinterpret_cast<const T*>(staged + r * BYTES);
+#pragma unroll
+  for (int q = 0; q < PER; q += L)
+    if (q + l < PER) dst[q + l] = src[q + l];
+}
+template <int L>
+__device__ __forceinline__ void copy_row_any(uint8_t* plane, const uint8_t* staged, int bytes, long long rec, int r,
+                                             int l) {
+  if (rec < 0) return;
+  uint8_t* dst = plane + rec * bytes;
+  const uint8_t* src = staged + r * bytes;
+  if ((bytes & 3) == 0) {
+    for (int q = l; q < bytes / 4; q += L)
+      reinterpret_cast<uint32_t*>(dst)[q] = reinterpret_cast<const uint32_t*>(src)[q];
+  } else {
+    for (int q = l; q < bytes; q += L) dst[q] = src[q];
   }
 }
 
-template <int D, typename TIn, int N, int B, int MODE>
+// Records of a tail tile (nrows < RW) or of scattered slots, from the staged
+// records to the planes (rec: the record of the lane's row, or -1).
+template <int D, typename TIn, class S>
+__device__ __forceinline__ void copy_out_rows(const S& sh, const WarpJob* wj, const uint8_t* wsm, long long rec,
+                                              int r, int l) {
+  using C = Enc<D, TIn, S>;
+  constexpr int L = C::L;
+  if constexpr (S::fixed) {
+    copy_row_fixed<L, C::AB>(wj->codes, wsm + C::W_ANG, rec, r, l);
+    copy_row_fixed<L, C::NB>(wj->norms, wsm + C::W_NRM, rec, r, l);
+    if constexpr (C::HB > 0) copy_row_fixed<L, 8>(wj->hdr, wsm + C::W_HDR, rec, r, l);
+  } else {
+    copy_row_any<L>(wj->codes, wsm + C::W_ANG, C::P * sh.W / 8, rec, r, l);
+    copy_row_any<L>(wj->norms, wsm + C::W_NRM, C::P * sh.B / 8, rec, r, l);
+    if (sh.mode != TAC_NORM_FP32) copy_row_any<L>(wj->hdr, wsm + C::W_HDR, 8, rec, r, l);
+  }
+}
+
+template <int D, typename TIn, class S>
 // Two CTAs of kEncWarps warps per SM (see kEncWarps).
 __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const __grid_constant__ EncParams p) {
-  using C = Enc<D, TIn, N, B, MODE>;
+  using C = Enc<D, TIn, S>;
   using IT = typename C::IT;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-
-  // fp32 edge table of this n (shared by the CTA).
-  float2* etab = reinterpret_cast<float2*>(smem + C::OFF_TAB);
-  for (int e = tid; e < C::n; e += kEncThreads) {
-    const float2 cs = cos_sin_q8(edge_q8(e, C::n), C::n);
-#pragma unroll
-    for (int c = 0; c < C::TABR; ++c) etab[e * C::TABR + c] = cs;
-  }
-  // the job table, for the fix-up kernel
-  if (blockIdx.x == 0) {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(p.job);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(p.gjobs);
-    const int words = p.njobs * (int)(sizeof(EncJob) / 4);
-    for (int i = tid; i < words; i += kEncThreads) dst[i] = src[i];
-  }
-  __syncthreads();
 
   // Each warp owns a contiguous range of warp tiles (balanced to +-1 tile), so
   // it meets a new job at most a few times per launch and walks its planes
@@ -1286,7 +1397,7 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
   const int per = p.ntiles / Gw, extra = p.ntiles % Gw;
   int t = gw * per + min(gw, extra);
   const int t_end = t + per + (gw < extra ? 1 : 0);
-  if (t >= t_end) return;
+  const bool work = t < t_end;
   uint8_t* wsm = smem + warp * C::WARP_B;
 
   // ---- prefetch cursor: the next warp tile to load ----
@@ -1294,7 +1405,7 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
   const int lane_cr = lane / C::CPR;
   uint8_t* const in_dst = wsm + C::W_IN + lane_cr * IT::STRIDE + (lane % C::CPR) * 16;
   int it = t;                    // next tile to issue
-  int pj = find_job(p, t);       // its job
+  int pj = work ? find_job(p, t) : 0;   // its job
   int p_end = 0;                 // first tile after that job
   int64_t i_left = 0;            // rows of the job from the tile's row 0
   int64_t i_step = 0;            // bytes between consecutive tiles (RW rows)
@@ -1310,7 +1421,7 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
     i_qstep = C::RPQ * sb;
     i_src = reinterpret_cast<const uint8_t*>(J.x) + (row0 + lane_cr) * sb + (lane % C::CPR) * 16;
   };
-  set_issue_job();
+  if (work) set_issue_job();
   auto issue = [&](int stg) {
     if (it < t_end) {
       if (it >= p_end) {  // a warp's tiles only move forward
@@ -1337,6 +1448,27 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
   };
 #pragma unroll
   for (int s = 0; s < kNS - 1; ++s) issue(s);
+
+  // fp32 edge table(s), shared by the CTA, while the first tiles arrive
+  float2* etab = reinterpret_cast<float2*>(smem + C::OFF_TAB);
+  if constexpr (S::fixed) {
+    for (int e = tid; e < S::n; e += kEncThreads) {
+      const float2 cs = cos_sin_q8(edge_q8(e, S::n), S::n);
+#pragma unroll
+      for (int c = 0; c < C::TABR; ++c) etab[e * C::TABR + c] = cs;
+    }
+    // the job table, for the fix-up kernel
+    if (blockIdx.x == 0) {
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(p.job);
+      uint32_t* dst = reinterpret_cast<uint32_t*>(p.gjobs);
+      const int words = p.njobs * (int)(sizeof(EncJob) / 4);
+      for (int i = tid; i < words; i += kEncThreads) dst[i] = src[i];
+    }
+  } else {
+    for (int e = tid; e < kTabEntries; e += kEncThreads) etab[e] = g_edge_f32.v[e];
+  }
+  __syncthreads();
+  if (S::fixed && !work) return;
 
   // ---- compute cursor ----
   WarpJob* wj = reinterpret_cast<WarpJob*>(wsm + C::W_JOB);
@@ -1367,9 +1499,11 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
   // the current (dense) job and the prefetched tile a full tile of the issue
   // job inside the warp's range.  Set by the general iterations.
   int fast = 0;
-  const float2* const etl = etab + (lane % C::TABR);
+  const float2* etl = etab + (lane % C::TABR);
+  S sh;                          // the current job's shape
+  const int r = lane / C::L, l = lane % C::L;
   while (t < t_end) {
-    if (fast > 0) {
+    if (S::fixed && fast > 0) {
       // A stretch of `fast` tiles, each a full tile of the current dense job
       // whose prefetch is a full tile of the issue job: no per-tile checks, the
       // cursors are settled once after it.
@@ -1383,7 +1517,7 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
         for (int q = 0; q < C::CHUNKS; ++q) cp_async16(dst + q * C::RPQ * IT::STRIDE, i_src + q * i_qstep, 16);
         cp_async_commit();
         i_src += i_step;
-        tile_body<D, TIn, N, B, MODE>(wsm + C::W_IN + stage * IT::BYTES, wsm, etl, C::RW, lane, msk, qb, qn, t, p);
+        tile_body<D, TIn>(sh, wsm + C::W_IN + stage * IT::BYTES, wsm, etl, C::RW, lane, msk, qb, qn, t, p);
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < C::ROUNDS; ++q) {
@@ -1407,7 +1541,8 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
     // ---- general tile: a job's first tile, tails, scattered slots, range ends,
     // and the queue's moves to global memory ----
     if (qn > q_hi) {
-      spill_queue<D>(p, qb, qn, lane);
+      if constexpr (S::fixed) spill_queue<D>(p, qb, qn, lane);
+      else flush_queue<D, TIn, S>(p.job, [&](int e) { return qb + 2 * e; }, qn, reinterpret_cast<long long*>(wsm + C::W_X), lane);
       qn = 0;
     }
     cp_async_wait<kNS - 2>();
@@ -1422,7 +1557,7 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
       c_left = J.rows - c_row0;
       c_dense = J.slot == nullptr;
 #pragma unroll
-      for (int q = 0; q < C::ROUNDS; ++q) {
+      for (int q = 0; q < (S::fixed ? C::ROUNDS : 0); ++q) {
         const int ch = q * 32 + lane;
         if (ch < C::NA) { o_dst[q] = J.codes + 16 * ch; o_step[q] = C::RW * C::AB; }
         else if (ch < C::NA + C::NN) { o_dst[q] = J.norms + 16 * (ch - C::NA); o_step[q] = C::RW * C::NB; }
@@ -1432,10 +1567,11 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
       if (lane == 0) {
         wj->codes = J.codes; wj->norms = J.norms; wj->hdr = J.hdr; wj->slot = J.slot; wj->capacity = J.capacity;
         wj->job = cj;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) wj->signs[q] = J.signs[q];
       }
-      const int l = lane % C::L;
+      if constexpr (!S::fixed) {
+        sh.set(J);
+        etl = etab + tab_offset_n(sh.n);
+      }
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
         msk[m] = pair_sign_mask<C::ESZ>(J.signs, slot_pair<D>(l + C::L * m));
@@ -1444,17 +1580,34 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
       __syncwarp();
     }
     const int nrows = c_left >= C::RW ? C::RW : (int)c_left;
-    tile_body<D, TIn, N, B, MODE>(wsm + C::W_IN + stage * IT::BYTES, wsm, etl, nrows, lane, msk, qb, qn, t, p);
+    // a tail's or scattered rows' records (the slots arrive during the tile)
+    long long rec = -1;
+    if (r < nrows) rec = c_dense ? c_row0 + r : (long long)wj->slot[c_row0 + r];
+    tile_body<D, TIn>(sh, wsm + C::W_IN + stage * IT::BYTES, wsm, etl, nrows, lane, msk, qb, qn, t, p);
     __syncwarp();
     if (c_dense && nrows == C::RW) {
+      if constexpr (S::fixed) {
 #pragma unroll
-      for (int q = 0; q < C::ROUNDS; ++q) {
-        const int ch = q * 32 + lane;
-        if (ch < C::NCH)
-          *reinterpret_cast<uint4*>(o_dst[q]) = *reinterpret_cast<const uint4*>(wsm + C::W_ANG + 16 * ch);
+        for (int q = 0; q < C::ROUNDS; ++q) {
+          const int ch = q * 32 + lane;
+          if (ch < C::NCH)
+            *reinterpret_cast<uint4*>(o_dst[q]) = *reinterpret_cast<const uint4*>(wsm + C::W_ANG + 16 * ch);
+        }
+      } else {
+        // 2 W, 2 B and RW / 2 (header) chunks of 16 bytes
+        const int na = 2 * sh.W, nn = 2 * sh.B, nh = sh.mode != TAC_NORM_FP32 ? C::RW / 2 : 0;
+        for (int ch = lane; ch < na + nn + nh; ch += 32) {
+          const bool a = ch < na, h = ch >= na + nn;
+          const int at = a ? ch : h ? ch - na - nn : ch - na;
+          const int row_bytes = a ? C::P * sh.W / 8 : h ? 8 : C::P * sh.B / 8;
+          uint8_t* plane = a ? wj->codes : h ? wj->hdr : wj->norms;
+          const uint8_t* st = wsm + (a ? C::W_ANG : h ? C::W_HDR : C::W_NRM);
+          *reinterpret_cast<uint4*>(plane + c_row0 * row_bytes + 16 * at) = *reinterpret_cast<const uint4*>(st + 16 * at);
+        }
       }
     } else {
-      copy_out_slow<C::AB, C::NB, C::HB>(wj, wsm + C::W_ANG, wsm + C::W_NRM, wsm + C::W_HDR, c_row0, nrows, lane);
+      if (rec < 0 || rec >= wj->capacity) rec = -1;   // out-of-range slots are skipped
+      copy_out_rows<D, TIn>(sh, wj, wsm, rec, r, l);
     }
 #pragma unroll
     for (int q = 0; q < C::ROUNDS; ++q) o_dst[q] += o_step[q];
@@ -1469,7 +1622,26 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
     const int64_t f = min(cf, pf);
     fast = f > 0 ? (int)f : 0;
   }
-  if (qn > 0) spill_queue<D>(p, qb, qn, lane);
+  if constexpr (S::fixed) {
+    if (qn > 0) spill_queue<D>(p, qb, qn, lane);
+  } else {
+    // the CTA's queues together, the entries dealt to its warps: a warp takes
+    // its rows one after another, microseconds each
+    __shared__ int left[kEncWarps];
+    if (lane == 0) left[warp] = qn;
+    __syncthreads();
+    int total = 0;
+#pragma unroll
+    for (int w = 0; w < kEncWarps; ++w) total += left[w];
+    auto entry = [&](int e) {
+      int i = warp + kEncWarps * e, w = 0;
+      while (i >= left[w]) i -= left[w++];
+      return reinterpret_cast<const uint4*>(smem + w * C::WARP_B + C::W_Q) + 2 * i;
+    };
+    if (warp < total)
+      flush_queue<D, TIn, S>(p.job, entry, (total - warp + kEncWarps - 1) / kEncWarps,
+                             reinterpret_cast<long long*>(wsm + C::W_X), lane);
+  }
   cp_async_wait<0>();
 }
 
@@ -1484,7 +1656,7 @@ __global__ void __launch_bounds__(kEncThreads, kMinBlocks) encode_kernel(const _
 constexpr int kFixWarps = 4;
 constexpr int kFixChunk = 8;
 
-template <int D, typename TIn, int N, int B, int MODE>
+template <int D, typename TIn, class S>
 __global__ void __launch_bounds__(32 * kFixWarps) encode_fixup_kernel(const __grid_constant__ FixParams p) {
   constexpr int P = Geo<D>::P, RW = Geo<D>::RW;
   __shared__ long long scratch[kFixWarps][2 * P];
@@ -1494,8 +1666,8 @@ __global__ void __launch_bounds__(32 * kFixWarps) encode_fixup_kernel(const __gr
   const unsigned long long appended = *p.gq_n;
   const long long n = (long long)min(appended, (unsigned long long)p.gq_cap);
   for (long long c = gw; kFixChunk * c < n; c += GW)
-    flush_queue<D, TIn, N, B, MODE>(p.job, p.gq + 2 * kFixChunk * c, (int)min((long long)kFixChunk, n - kFixChunk * c),
-                                    scratch[warp], lane);
+    flush_queue<D, TIn, S>(p.job, [&](int e) { return p.gq + 2 * (kFixChunk * c + e); },
+                           (int)min((long long)kFixChunk, n - kFixChunk * c), scratch[warp], lane);
   if (appended <= (unsigned long long)p.gq_cap) return;
   const long long nwords = ((long long)p.ntiles * RW + 31) / 32;
   for (long long w0 = gw * 32; w0 < nwords; w0 += GW * 32) {
@@ -1519,7 +1691,7 @@ __global__ void __launch_bounds__(32 * kFixWarps) encode_fixup_kernel(const __gr
           whole[warp][1] = make_uint4(0u, 0u, 0u, 0u);
         }
         __syncwarp();
-        flush_queue<D, TIn, N, B, MODE>(p.job, whole[warp], 1, scratch[warp], lane);
+        flush_queue<D, TIn, S>(p.job, [&](int) { return &whole[warp][0]; }, 1, scratch[warp], lane);
       }
     }
   }
@@ -1528,11 +1700,13 @@ __global__ void __launch_bounds__(32 * kFixWarps) encode_fixup_kernel(const __gr
 // ---------------------------------------------------------------------------
 // Host-side launch helpers (called from tac_api.cu).
 // ---------------------------------------------------------------------------
-// phase: bit 0 launches the encode kernel, bit 1 its fix-up (3: both, in order).
+// phase: bit 0 launches the encode kernel, bit 1 its fix-up (3: both, in order);
+// kEncAny the kernel of small calls.
 template <int D, typename TIn, int N, int B, int MODE>
 static cudaError_t launch_encode_v(const EncParams& p, int grid_cap, cudaStream_t st, int phase) {
-  using C = Enc<D, TIn, N, B, MODE>;
-  auto kern = encode_kernel<D, TIn, N, B, MODE>;
+  using S = FixedShape<N, B, MODE>;
+  using C = Enc<D, TIn, S>;
+  auto kern = encode_kernel<D, TIn, S>;
   static std::atomic<int> configured[64];   // per device; concurrent first calls set the same
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1545,7 +1719,7 @@ static cudaError_t launch_encode_v(const EncParams& p, int grid_cap, cudaStream_
   static std::atomic<int> occ[64][2];
   int per_sm = dev >= 0 && dev < 64 ? occ[dev][0].load(std::memory_order_acquire) : 0;
   int fix_sm = dev >= 0 && dev < 64 ? occ[dev][1].load(std::memory_order_acquire) : 0;
-  auto fix = encode_fixup_kernel<D, TIn, N, B, MODE>;
+  auto fix = encode_fixup_kernel<D, TIn, S>;
   if (per_sm == 0 || fix_sm == 0) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kEncThreads, C::SMEM);
     if (e != cudaSuccess) return e;
@@ -1585,10 +1759,35 @@ static cudaError_t launch_encode_v(const EncParams& p, int grid_cap, cudaStream_
   return cudaGetLastError();
 }
 
+// The kernel of small calls: every shape, its own fix-up, no workspace.
+template <int D, typename TIn>
+static cudaError_t launch_encode_any(const EncParams& p, int sms, cudaStream_t st) {
+  using C = Enc<D, TIn, AnyShape>;
+  auto kern = encode_kernel<D, TIn, AnyShape>;
+  static std::atomic<int> occ[64];   // resident CTAs per SM, per device; concurrent first calls set the same
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  int per_sm = occ[dev].load(std::memory_order_acquire);
+  if (per_sm == 0) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kEncThreads, C::SMEM);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    occ[dev].store(per_sm, std::memory_order_release);
+  }
+  const int grid = std::min(sms * per_sm, (p.ntiles + kEncWarps - 1) / kEncWarps);
+  if (grid < 1) return cudaSuccess;
+  kern<<<grid, kEncThreads, C::SMEM, st>>>(p);
+  return cudaGetLastError();
+}
+
 // One kernel per supported (n, norm bits, mode): n in {2, 4, ..., 256, 48, 56},
 // (B, mode) in {(4, linear), (4, log), (8, linear), (8, log), (32, fp32)}.
 template <int D, typename TIn>
 static cudaError_t launch_encode_t(const EncParams& p, int n, int b, int mode, int sms, cudaStream_t st, int phase) {
+  if (phase == kEncAny) return launch_encode_any<D, TIn>(p, sms, st);
 #define TAC_ENC_N(NN)                                                                                   \
   if (n == NN) {                                                                                        \
     if (mode == TAC_NORM_FP32) return b == 32 ? launch_encode_v<D, TIn, NN, 32, TAC_NORM_FP32>(p, sms, st, phase) \

@@ -1,0 +1,105 @@
+"""Small encode calls (one kernel for every codebook shape, which re-decides its
+own codes) against large ones (a kernel per shape, queue and fix-up kernel).
+
+Every shape the library takes, row counts around the warp tile, contiguous,
+scattered and out-of-range slots, rows that need the exact path, zero rows and
+non-finite rows: the records must be the same bytes, and so must the records of
+a large call whose queue has no room.
+"""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(n, b, m) for n in (2, 4, 8, 16, 32, 48, 56, 64, 128, 256)
+          for b, m in ((4, 0), (4, 1), (8, 0), (8, 1), (32, 2))]
+LARGE_TILES = 65536
+
+
+def _rows(torch, d, dtype, rows):
+    """Gaussian rows with channel scales; the first 400 hold rows that take the rare paths."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    x = torch.randn((rows, d), generator=g, device="cuda")
+    x *= torch.exp(torch.randn((1, d), generator=g, device="cuda"))
+    x[3] = 0
+    x[7] = 1.0
+    x[11] = 0
+    x[11, d // 2] = -3.0
+    x[13, ::2] = 0
+    x[17] = float("nan")
+    x[19, 1] = float("inf")
+    x[100:200] = torch.randint(-2, 3, (100, d), generator=g, device="cuda").float()   # ties at edges and midpoints
+    x[200:300] *= torch.exp2(torch.linspace(-36, 50, 100, device="cuda"))[:, None]
+    x[300:400, 1:] = x[300:400, :1] * 2.0**-30
+    return x.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+
+
+def _view(torch, tac, cache):
+    """The planes of a device cache as rows: angle, norm, header (or None)."""
+    c, n = cache.cfg, cache.capacity
+    ab, nb = tac.angle_row_bytes(c), tac.norm_row_bytes(c)
+    off = tac.header_offset(c, n)
+    hdr = None if c.norm_mode == tac.NORM_FP32 else cache.norms[off: off + 8 * n].reshape(n, 8)
+    return cache.codes[: n * ab].reshape(n, ab), cache.norms[: n * nb].reshape(n, nb), hdr
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+def test_small_calls_match_large_ones(tac_gpu, d, dtype):
+    import torch
+    tac = tac_gpu
+    rw = 32 // (d // 16)
+    rows = LARGE_TILES * rw + 3
+    x = _rows(torch, d, dtype, rows)
+    pieces = [(0, 400), (400, 1), (401, rw - 1), (500, rw), (600, rw + 1), (700, 5 * rw + 3), (rows - 1000, 1000)]
+    pieces = [(a, k) for a, k in pieces if k > 0]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    for n, b, m in SHAPES:
+        cfg = tac.layer_cfg(d, n, b, m, 0, 2, 1)
+        big = tac.Cache.empty(cfg, rows)
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        tac.encode_multi([tac.EncodeJob(cfg, x, big, None, st)])
+        want = _view(torch, tac, big)
+        jobs, at, stats = [], [], []
+        for i, (a, k) in enumerate(pieces):
+            cap, slot, sel = k, None, torch.arange(k, device="cuda")
+            if i % 2:                                   # scattered, two rows dropped
+                cap = 3 * k + 5
+                slot = torch.randperm(cap, generator=g, device="cuda")[:k]
+                if k > 4:
+                    slot[1], slot[k - 2] = -1, cap
+                sel = slot
+            cache = tac.Cache.empty(cfg, cap)
+            s = torch.zeros(1, dtype=torch.int32, device="cuda")
+            jobs.append(tac.EncodeJob(cfg, x[a:a + k], cache, slot, s))
+            at.append((a, k, sel, cap))
+            stats.append(s)
+        tac.encode_multi(jobs)
+        torch.cuda.synchronize()
+        assert int(st) == tac.TAC_E_NONFINITE
+        for (a, k, sel, cap), j, s in zip(at, jobs, stats):
+            ok = (sel >= 0) & (sel < cap)
+            for got, ref in zip(_view(torch, tac, j.cache), want):
+                if ref is not None:
+                    assert torch.equal(got[sel[ok]], ref[a:a + k][ok]), (n, b, m, a, k)
+            assert int(s) == (tac.TAC_E_NONFINITE if a == 0 else 0)
+
+
+@pytest.mark.parametrize("n,b,m", [(64, 8, 0), (256, 4, 1), (56, 32, 2)])
+def test_large_call_without_queue_room(tac_gpu, n, b, m):
+    """The minimum workspace: every queued code's row is re-decided whole."""
+    import torch
+    tac, d = tac_gpu, 128
+    rows = LARGE_TILES * 4 + 1
+    x = _rows(torch, d, "bf16", rows)
+    cfg = tac.layer_cfg(d, n, b, m, 0, 0, 0)
+    caches = [tac.Cache.empty(cfg, rows) for _ in range(2)]
+    for cache, ws in zip(caches, (None, "min")):
+        jobs = [tac.EncodeJob(cfg, x, cache)]
+        if ws:
+            ws = torch.empty(tac.encode_workspace_bytes(jobs)[1], dtype=torch.uint8, device="cuda")
+        tac.encode_multi(jobs, workspace=ws)
+    torch.cuda.synchronize()
+    for a, c in zip(_view(torch, tac, caches[0]), _view(torch, tac, caches[1])):
+        assert a is None or torch.equal(a, c)

@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 from dataclasses import dataclass, field
 
@@ -80,6 +81,8 @@ def library_path() -> str:
 def load():
     """Load libtac.so (raises if it has not been built: there is no fallback)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -244,24 +247,50 @@ def _dtype_code(t) -> int:
     raise TypeError(f"unsupported dtype {t.dtype} (bf16 or fp32)")
 
 
-def _rows(t, d: int) -> _Rows:
-    if t.dim() != 2 or t.shape[1] != d or (t.shape[0] > 1 and t.stride(1) != 1):
-        raise ValueError(f"expected a [rows, {d}] tensor with unit inner stride, got {tuple(t.shape)}")
+def _row_fields(t, d: int):
+    """(address, dtype code, rows, row stride) of a [rows, d] device tensor."""
+    shape = t.shape
+    if len(shape) != 2 or shape[1] != d or (shape[0] > 1 and t.stride(1) != 1):
+        raise ValueError(f"expected a [rows, {d}] tensor with unit inner stride, got {tuple(shape)}")
     if not t.is_cuda:
         raise ValueError("tensor must be on a CUDA device")
+    rows = shape[0]
+    return t.data_ptr(), _dtype_code(t), rows, t.stride(0) if rows > 1 else d
+
+
+def _rows(t, d: int) -> _Rows:
     r = _Rows()
-    r.data = t.data_ptr()
-    r.dtype = _dtype_code(t)
-    r.rows = t.shape[0]
-    r.row_stride = t.stride(0) if t.shape[0] > 1 else d
+    r.data, r.dtype, r.rows, r.row_stride = _row_fields(t, d)
     return r
 
 
 def _stream_ptr(stream) -> int:
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # the same handle without a Stream object
+    if raw is None:
+        return int(torch.cuda.current_stream().cuda_stream)
+    return int(raw(torch.cuda.current_device()))
+
+
+# The job structs as packed by struct: one call fills a job (about 1 us; setting
+# its fields through ctypes takes 4).  Values that the struct formats would
+# refuse or take otherwise than ctypes go through the fields.
+_CFG_FMT = struct.Struct("=4i16s")
+_ENC_FMT = struct.Struct("=32sQi4xqqQQqQQ")
+_DEC_FMT = struct.Struct("=32sQQqQQi4xqq")
+assert _CFG_FMT.size == ctypes.sizeof(_Cfg)
+assert _ENC_FMT.size == ctypes.sizeof(_EncJob) and _DEC_FMT.size == ctypes.sizeof(_DecJob)
+
+
+def _cfg_bytes(cfg: LayerCfg) -> bytes:
+    d, n, b, m, s = cfg.d, cfg.n_angle, cfg.norm_bits, cfg.norm_mode, cfg.signs
+    if (type(d) is int and type(n) is int and type(b) is int and type(m) is int and type(s) is np.ndarray
+            and s.dtype == np.uint32 and s.ndim == 1 and s.size <= MAX_D // 32
+            and max(d, n, b, m) < 2**31 and min(d, n, b, m) >= -(2**31)):
+        return _CFG_FMT.pack(d, n, b, m, s.tobytes())
+    return bytes(cfg.to_c())
 
 
 @dataclass
@@ -321,7 +350,7 @@ def encode(x, cfg: LayerCfg, cache: Cache | None = None, stream=None, status=Non
     if cache.capacity != x.shape[0]:
         raise ValueError("tac_encode writes a cache of capacity rows; use encode_multi for slots")
     r = _rows(x, cfg.d)
-    c = cfg.to_c()
+    c = _Cfg.from_buffer_copy(_cfg_bytes(cfg))
     if status is None:
         _check(load().tac_encode(ctypes.byref(r), ctypes.byref(c), cache.codes.data_ptr(),
                                  cache.norms.data_ptr(), _stream_ptr(stream)))
@@ -340,7 +369,7 @@ def decode(cache: Cache, cfg: LayerCfg, rows: int | None = None, dtype=None, y=N
     if rows != cache.capacity:
         raise ValueError("tac_decode reads a cache of capacity rows; use decode_multi for slots")
     r = _rows(y, cfg.d)
-    c = cfg.to_c()
+    c = _Cfg.from_buffer_copy(_cfg_bytes(cfg))
     _check(load().tac_decode(cache.codes.data_ptr(), cache.norms.data_ptr(), ctypes.byref(c),
                              ctypes.byref(r), _stream_ptr(stream)))
     return y
@@ -362,7 +391,17 @@ class Prepared:
 
 def _enc_array(jobs):
     arr = (_EncJob * max(1, len(jobs)))()
+    at, size, pack = 0, _ENC_FMT.size, _ENC_FMT.pack_into
     for i, j in enumerate(jobs):
+        cache, slot, status = j.cache, j.slot, j.status
+        cap = cache.capacity
+        if type(cap) is int and -(2**63) <= cap < 2**63:
+            ptr, dt, rows, stride = _row_fields(j.x, j.cfg.d)
+            pack(arr, at, _cfg_bytes(j.cfg), ptr, dt, rows, stride, cache.codes.data_ptr(), cache.norms.data_ptr(),
+                 cap, 0 if slot is None else slot.data_ptr(), 0 if status is None else status.data_ptr())
+            at += size
+            continue
+        at += size
         e = arr[i]
         e.cfg = j.cfg.to_c()
         e.x = _rows(j.x, j.cfg.d)
@@ -374,18 +413,22 @@ def _enc_array(jobs):
     return arr
 
 
-def encode_workspace_bytes(jobs) -> tuple[int, int]:
-    """tac_encode_workspace_bytes: (recommended, minimum) workspace bytes."""
+def _enc_workspace_bytes(arr, njobs: int) -> tuple[int, int]:
     mn = ctypes.c_int64(0)
-    n = load().tac_encode_workspace_bytes(_enc_array(jobs), len(jobs), ctypes.byref(mn))
+    n = load().tac_encode_workspace_bytes(arr, njobs, ctypes.byref(mn))
     if n < 0:
         raise TacError(TAC_E_INVAL, last_error())
     return int(n), int(mn.value)
 
 
-def _enc_workspace(jobs, workspace):
+def encode_workspace_bytes(jobs) -> tuple[int, int]:
+    """tac_encode_workspace_bytes: (recommended, minimum) workspace bytes."""
+    return _enc_workspace_bytes(_enc_array(jobs), len(jobs))
+
+
+def _enc_workspace(jobs, arr, workspace):
     if workspace is None:
-        need = encode_workspace_bytes(jobs)[0] if jobs else 0
+        need = _enc_workspace_bytes(arr, len(jobs))[0] if jobs else 0
         dev = jobs[0].x.device if jobs else "cuda"
         workspace = _torch().empty(max(need, 16), dtype=_torch().uint8, device=dev)
     return workspace
@@ -396,7 +439,7 @@ def encode_multi(jobs, stream=None, workspace=None):
     group, or one launch for a small call (see launch_count); allocates the re-decision workspace (torch) when
     none is given.  Returns the workspace."""
     arr = _enc_array(jobs)
-    workspace = _enc_workspace(jobs, workspace)
+    workspace = _enc_workspace(jobs, arr, workspace)
     _check(load().tac_encode_multi_ws(arr, len(jobs), workspace.data_ptr(),
                                       workspace.numel() * workspace.element_size(), _stream_ptr(stream)))
     if stream is not None and jobs:
@@ -407,14 +450,25 @@ def encode_multi(jobs, stream=None, workspace=None):
 def encode_multi_prepared(jobs, workspace=None) -> Prepared:
     """tac_encode_multi_ws over `jobs`, marshalled once (see Prepared), with
     a workspace allocated (torch) once when none is given."""
-    workspace = _enc_workspace(jobs, workspace)
+    arr = _enc_array(jobs)
+    workspace = _enc_workspace(jobs, arr, workspace)
     extra = (workspace.data_ptr(), workspace.numel() * workspace.element_size())
-    return Prepared(load().tac_encode_multi_ws, _enc_array(jobs), len(jobs), extra, (list(jobs), workspace))
+    return Prepared(load().tac_encode_multi_ws, arr, len(jobs), extra, (list(jobs), workspace))
 
 
 def _dec_array(jobs):
     arr = (_DecJob * max(1, len(jobs)))()
+    at, size, pack = 0, _DEC_FMT.size, _DEC_FMT.pack_into
     for i, j in enumerate(jobs):
+        cache, slot = j.cache, j.slot
+        cap = cache.capacity
+        if type(cap) is int and -(2**63) <= cap < 2**63:
+            ptr, dt, rows, stride = _row_fields(j.y, j.cfg.d)
+            pack(arr, at, _cfg_bytes(j.cfg), cache.codes.data_ptr(), cache.norms.data_ptr(), cap,
+                 0 if slot is None else slot.data_ptr(), ptr, dt, rows, stride)
+            at += size
+            continue
+        at += size
         e = arr[i]
         e.cfg = j.cfg.to_c()
         e.codes = j.cache.codes.data_ptr()
@@ -463,19 +517,23 @@ def _att_array(jobs):
     return arr
 
 
-def attend_workspace_bytes(jobs) -> int:
-    """tac_attend_workspace_bytes."""
-    n = load().tac_attend_workspace_bytes(_att_array(jobs), len(jobs))
+def _att_workspace_bytes(arr, njobs: int) -> int:
+    n = load().tac_attend_workspace_bytes(arr, njobs)
     if n < 0:
         raise TacError(TAC_E_INVAL, last_error())
     return int(n)
+
+
+def attend_workspace_bytes(jobs) -> int:
+    """tac_attend_workspace_bytes."""
+    return _att_workspace_bytes(_att_array(jobs), len(jobs))
 
 
 def attend_multi(jobs, workspace=None, stream=None):
     """tac_attend_multi; allocates the workspace (torch) when none is given."""
     torch = _torch()
     arr = _att_array(jobs)
-    need = attend_workspace_bytes(jobs) if jobs else 0
+    need = _att_workspace_bytes(arr, len(jobs)) if jobs else 0
     if workspace is None:
         dev = jobs[0].q.device if jobs else "cuda"
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
@@ -492,7 +550,7 @@ def attend_multi_prepared(jobs, workspace=None, static=False) -> Prepared:
     if static:
         return Prepared(lib.tac_attend_multi_static, arr, len(jobs), (), list(jobs))
     torch = _torch()
-    need = attend_workspace_bytes(jobs) if jobs else 0
+    need = _att_workspace_bytes(arr, len(jobs)) if jobs else 0
     if workspace is None:
         dev = jobs[0].q.device if jobs else "cuda"
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)

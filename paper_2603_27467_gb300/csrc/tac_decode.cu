@@ -505,10 +505,14 @@ static cudaError_t launch_decode_v(const DecParams& p, int grid_cap, cudaStream_
     if (e != cudaSuccess) return e;
     configured[dev].store(1, std::memory_order_release);
   }
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::THREADS, C::SMEM);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
+  static std::atomic<int> occ[64];          // resident CTAs per SM, found once per device
+  int per_sm = dev >= 0 && dev < 64 ? occ[dev].load(std::memory_order_acquire) : 0;
+  if (per_sm == 0) {
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::THREADS, C::SMEM);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    if (dev >= 0 && dev < 64) occ[dev].store(per_sm, std::memory_order_release);
+  }
   int grid = grid_cap * per_sm;
   const int need = (p.ntiles + C::WARPS - 1) / C::WARPS;
   if (grid > need) grid = need;

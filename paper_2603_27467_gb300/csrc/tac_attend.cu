@@ -30,14 +30,21 @@
 //                   stores the row.
 // Bound: instruction issue.  About 12 instructions decode and split one pair
 // (table offset 2, lookup 1, norm code 3, products and split 4, packing 2); of
-// 91 warp-instructions a token-head 48 are these (d = 128, 4 queries), and the
-// schedulers issue in 62 % of the cycles at 16 warps per SM (128 registers).
+// some 85 warp-instructions a token-head 48 are these (d = 128, 4 queries), and
+// the schedulers issue in 62 % of the cycles at 16 warps per SM (128
+// registers).  A warp's batch of 32 tokens takes about 12 000 cycles: scores
+// 4500, values 5900, the rest softmax, constants and copies.  Copies are bulk
+// copies, one lane a segment: six cp.async loops over the segments took 2000
+// cycles a batch (162 us where bulk copies take 150, below).  The set-up of a
+// CTA's first job is 12 000 cycles (20 000 with the queries rotated and split
+// in shared memory, the tables computed and written 16 copies by one thread,
+// and a binary search for the job).
 // With the products on the CUDA cores (114 instructions, 10 - 12 warps, and a
 // warp walking 256 tokens alone) 16 sequences of 1k to 32k tokens (8 KV heads,
-// 4 queries each, 244 MB of records) took 229 us, now 162 us (1.5 TB/s); 8
-// heads of 4097 tokens 59 us, now 21 us (a CTA of 8 warps per 256 tokens fills
+// 4 queries each, 244 MB of records) took 229 us, now 150 us (1.6 TB/s); 8
+// heads of 4097 tokens 59 us, now 19 us (a CTA of 8 warps per 256 tokens fills
 // the device; a third of it are the launches); 128 heads of 8192 tokens at
-// d = 64 143 us, now 90 us.  Error of an fp32 output against 64 bits: 5.4e-7
+// d = 64 143 us, now 81 us.  Error of an fp32 output against 64 bits: 5.4e-7
 // (6.0e-7 before).  A persistent grid merges a CTA's units before it writes, so
 // the combine kernel reads one result per CTA and job instead of one per 256 tokens.
 // Codebooks (n, norm bits, norm mode) are runtime parameters: K and V may
@@ -67,10 +74,11 @@ struct Att {
   static constexpr int P = D / 2, NQ = 4 * QT;
   static constexpr int KP = P / 4;            // K: pairs of a token a lane decodes (4 lanes a token)
   static constexpr int VP = P / 8;            // V: pairs of a token a lane decodes (8 lanes a token)
-  // Shared memory: rotated queries | K table | V table | per warp: batch
-  // constants, weights, staged batch.  The merge of the warps' results reuses
-  // the warps' part.
-  static constexpr int QB = NQ * P * 8 + 64;  // float2 rows, then one scale per query
+  // Shared memory: rotated queries (the words of their fragments, hi and lo
+  // parts), their scales, the warps' barriers | K table | V table | per warp:
+  // batch constants, weights, staged batch.  The merge of the warps' results
+  // reuses the queries' and the warps' parts.
+  static constexpr int Q_S = NQ * P * 8, Q_MB = Q_S + 64, QB = Q_MB + 16 * kAttWarps;
   static constexpr int W_KC = 0;              // float2 per token: (A, B) of K's norms
   static constexpr int W_VC = W_KC + kAttBatch * 8;
   static constexpr int W_KS = W_VC + kAttBatch * 8;   // float per token: 2^e of K's record
@@ -81,6 +89,22 @@ struct Att {
   static int smem(int stage, int tables) { return QB + tables + std::max(kAttWarps * (W_STG + stage), MERGE); }
   static_assert(QB % 16 == 0 && W_STG % 16 == 0, "alignment");
 };
+
+// Bin centres (cos, sin)(2 pi k / n) of every supported n, rounded from fp64
+// by the host compiler.
+namespace cx {
+struct CentreTable { float2 v[kTabEntries]; };
+constexpr CentreTable make_centre_table() {
+  CentreTable t{};
+  for (int idx = 0; idx < kTabEntries; ++idx) {
+    const int n = tab_n_of(idx), k = idx - tab_offset_n(n);
+    const CS cs = cos_sin_q8(8 * k, n);
+    t.v[idx] = float2{(float)cs.c, (float)cs.s};
+  }
+  return t;
+}
+}  // namespace cx
+__device__ const cx::CentreTable g_centre = cx::make_centre_table();
 
 __device__ __forceinline__ uint32_t rotr(uint32_t x, int s) { return __funnelshift_r(x, x, s); }
 
@@ -137,7 +161,44 @@ __device__ __forceinline__ void norm_consts(float2 h, float inv_l, bool lg, floa
   }
 }
 
-// In-place normalized Walsh-Hadamard transform of `rows` rows of d floats in
+// A warp's staged batches arrive by bulk copies (cp.async.bulk) that signal an
+// mbarrier of its own.  A wait gives up after 2^16 tries (each suspends the
+// warp for a while) and returns false; the kernel then marks its results NaN.
+__device__ __forceinline__ uint32_t smem_addr(const void* ptr) { return (uint32_t)__cvta_generic_to_shared(ptr); }
+__device__ __forceinline__ void mbar_init(uint32_t bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, int bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < (1 << 16); ++i) {
+    uint32_t done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+// Shared memory written by ordinary stores is next written by bulk copies.
+__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// The last, partial batch of a job: rows < 32 rows of row_bytes bytes, the rest
+// of the 32 zero-filled.
+static __device__ __noinline__ void copy_tail(const uint8_t* src, uint8_t* dst, int row_bytes, int rows, int lane) {
+  const int full = kAttBatch * row_bytes, valid = rows * row_bytes;
+  for (int c = lane * 16; c < full; c += 512) {
+    const int n = min(max(valid - c, 0), 16);
+    cp_async16(dst + c, n > 0 ? src + c : src, n);
+  }
+}
+
+// In-place unnormalized Walsh-Hadamard transform of a row of d floats in
 // shared memory (Sylvester order), by the lanes of a warp.
 template <int D>
 __device__ __forceinline__ void warp_fwht(float* row, int lane) {
@@ -169,10 +230,11 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
   constexpr int P = C::P, NQ = C::NQ, KP = C::KP, KS = KP / 2, VP = C::VP;
   constexpr int NV = 4 * QT;                       // scores a lane owns in the softmax
   extern __shared__ __align__(128) uint8_t smem[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler too
   const int g = lane >> 2, t = lane & 3;           // the fragments' row group and column pair
-  float2* const qrot = reinterpret_cast<float2*>(smem);                      // [NQ][P], slot order
-  float* const qscale = reinterpret_cast<float*>(smem + NQ * P * 8);         // 2^e of each query
+  uint32_t* const qfrag = reinterpret_cast<uint32_t*>(smem);                 // [hi, lo][NQ][P]
+  float* const qscale = reinterpret_cast<float*>(smem + C::Q_S);             // 2^e of each query
   float2* const tk = reinterpret_cast<float2*>(smem + C::QB);
   uint8_t* const wbase = smem + C::QB + p.tab_k + p.tab_v;
   float2* const tv = reinterpret_cast<float2*>(smem + C::QB + p.tab_k);
@@ -192,16 +254,16 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
   const int u_end = u + per + (cta < extra ? 1 : 0);
   int tab_nk = 0, tab_nv = 0;                      // codebooks the tables hold
 
-  int jb = 0;
-  {
-    int lo = 0, hi = p.njobs - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (p.job[mid].unit0 <= u) lo = mid; else hi = mid - 1;
-    }
-    jb = lo;
+  int jb = p.first_job[cta];
+  const uint32_t bar_k = smem_addr(smem + C::Q_MB) + 16 * warp, bar_v = bar_k + 8;
+  uint32_t phase_k = 0, phase_v = 0;               // parity of the next completion
+  bool dead = false;                               // a wait ran out
+  if (lane == 0) {
+    mbar_init(bar_k);
+    mbar_init(bar_v);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-
+  __syncwarp();
   for (; u < u_end; ++jb) {                        // a segment: the CTA's units of one job
     const AttJob& J = p.job[jb];
     const int nunits = (int)((J.tokens + kAttUnit - 1) / kAttUnit);
@@ -219,88 +281,122 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     const int seg = cta - att_cta_of(J.unit0, p.nunits, p.nctas);
     u = u_stop;
 
-    // ---- staging: 32 rows of the K or V planes, zero-filled past the last token ----
-    auto copy_rows = [&](const uint8_t* src, uint8_t* dst, int row_bytes, int rows) {
-      const int full = kAttBatch * row_bytes, valid = rows * row_bytes;
-      if (rows == kAttBatch) {
-#pragma unroll 4
-        for (int c = lane * 16; c < full; c += 512) cp_async16(dst + c, src + c, 16);
-      } else {
-        for (int c = lane * 16; c < full; c += 512) {
-          const int n = min(max(valid - c, 0), 16);
-          cp_async16(dst + c, n > 0 ? src + c : src, n);
+    // ---- staging: lane s of 6 copies the 32 rows of segment s (K angle | norm |
+    // header, V angle | norm | header) of a whole batch; the last, partial batch
+    // of the job comes by cp.async ----
+    const bool is_v = lane >= 3;
+    const int sg = is_v ? lane - 3 : lane;
+    const int c_row = lane >= 6 ? 0 : sg == 0 ? (is_v ? av : ak) : sg == 1 ? (is_v ? nbv : nbk) : (is_v ? hvb : hkb);
+    const uint8_t* c_src = sg == 0 ? (is_v ? J.vc : J.kc) : sg == 1 ? (is_v ? J.vn : J.kn) : (is_v ? J.vh : J.kh);
+    c_src += row0 * c_row;                         // advances with the K (V) batches
+    const uint32_t c_dst =
+        smem_addr(sg == 0 ? (is_v ? st_va : stk) : sg == 1 ? (is_v ? st_vn : st_kn) : (is_v ? st_vh : st_kh));
+    auto issue = [&](bool v, int64_t row, uint32_t bar, int bytes) {
+      const bool mine = (is_v == v) && lane < 6 && c_row > 0;
+      if (row + kAttBatch <= seg_rows) {
+        if (lane == 0) mbar_expect(bar, bytes);
+        __syncwarp();
+        if (mine) bulk_copy(c_dst, c_src, kAttBatch * c_row, bar);
+      } else if (row < seg_rows) {
+        const int rows = (int)(seg_rows - row);
+        for (int x = 0; x < 3; ++x) {
+          const int from = (v ? 3 : 0) + x, rb = __shfl_sync(0xffffffffu, c_row, from);
+          const uint8_t* src = reinterpret_cast<const uint8_t*>(
+              __shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)c_src, from));
+          uint8_t* dst = x == 0 ? (v ? st_va : stk) : x == 1 ? (v ? st_vn : st_kn) : (v ? st_vh : st_kh);
+          copy_tail(src, dst, rb, rows, lane);
         }
+        cp_async_commit();
       }
+      if (mine) c_src += kAttUnit * c_row;
     };
-    auto issue_k = [&](int64_t row) {
-      if (row < seg_rows) {
-        const int rows = (int)min((int64_t)kAttBatch, J.tokens - row);
-        copy_rows(J.kc + row * ak, stk, ak, rows);
-        copy_rows(J.kn + row * nbk, st_kn, nbk, rows);
-        if (hkb) copy_rows(J.kh + row * 8, st_kh, 8, rows);
+    const int bytes_k = kAttBatch * (ak + nbk + hkb), bytes_v = kAttBatch * (av + nbv + hvb);
+    // waits for the batch of rows [row, row + 32)
+    auto landed = [&](int64_t row, uint32_t bar, uint32_t& phase) {
+      if (row + kAttBatch <= seg_rows) {
+        if (!dead) dead = !mbar_wait(bar, phase);
+        phase ^= 1u;
+      } else {
+        cp_async_wait<0>();
       }
-      cp_async_commit();
+      __syncwarp();
     };
-    auto issue_v = [&](int64_t row) {
-      if (row < seg_rows) {
-        const int rows = (int)min((int64_t)kAttBatch, J.tokens - row);
-        copy_rows(J.vc + row * av, st_va, av, rows);
-        copy_rows(J.vn + row * nbv, st_vn, nbv, rows);
-        if (hvb) copy_rows(J.vh + row * 8, st_vh, 8, rows);
-      }
-      cp_async_commit();
-    };
+    fence_async_proxy();
     __syncthreads();                               // the previous segment's merge is done with the warps' memory
-    issue_k(row0);
-    issue_v(row0);
+    issue(false, row0, bar_k, bytes_k);
+    issue(true, row0, bar_v, bytes_v);
 
     // ---- bin-centre tables (cos, sin)(2 pi k / n), 2^lgr copies: entry k copy c
     // at k 2^lgr + c; entries n..2^W-1 repeat entry n-1 (codes >= n clamp) ----
     const int lgrk = J.lgrk, lgrv = J.lgrv;
     if (tab_nk != J.nk || tab_nv != J.nv) {
       const int ek = 1 << J.wk, ev = 1 << J.wv;
-      for (int e = tid; e < ek + ev; e += kAttThreads) {
-        const bool v = e >= ek;
-        const int i = v ? e - ek : e, n = v ? J.nv : J.nk, lg = v ? lgrv : lgrk;
-        float2* tab = (v ? tv : tk) + (i << lg);
-        const float2 cs = cos_sin_q8(8 * min(i, n - 1), n);
-        for (int c = 0; c < (1 << lg); ++c) tab[c] = cs;
+      for (int e = tid; e < (ek << lgrk) + (ev << lgrv); e += kAttThreads) {
+        const bool v = e >= ek << lgrk;
+        const int at = v ? e - (ek << lgrk) : e, n = v ? J.nv : J.nk;
+        (v ? tv : tk)[at] = g_centre.v[tab_offset_n(n) + min(at >> (v ? lgrv : lgrk), n - 1)];
       }
       tab_nk = J.nk;
       tab_nv = J.nv;
     }
     // ---- rotated queries q' = H D_K q * scale * log2(e), one warp a query,
-    // scaled by 2^-e into [-2, 2) ----
+    // scaled by 2^-e into [-2, 2) and split; the word of slot i (the halves of its
+    // pair) lands where the fragments' order wants it: the run of KP slots of
+    // lane t, step by step.  Step ks takes two slots of every lane's run:
+    // neighbours, or (4-bit norms, whose codes are unpacked four apart) slots
+    // four apart ----
+    const bool k4 = J.ck <= 1;
     if (warp < NQ) {
-      float2* const q2 = qrot + warp * P;
-      float* const qrow = reinterpret_cast<float*>(q2);
-      const int64_t off = (int64_t)warp * J.q_stride;
+      float y[D / 32];                             // elements lane + 32 k
+      const int64_t off = (int64_t)warp * J.q_stride + lane;
 #pragma unroll
-      for (int j = lane; j < D; j += 32) {
+      for (int k = 0; k < D / 32; ++k) {
         float x = 0.f;
         if (warp < nq)
-          x = p.q_bf16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(J.q)[off + j])
-                       : reinterpret_cast<const float*>(J.q)[off + j];
-        qrow[j] = ((J.sk[j >> 5] >> (j & 31)) & 1u) ? -x : x;
+          x = p.q_bf16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(J.q)[off + 32 * k])
+                       : reinterpret_cast<const float*>(J.q)[off + 32 * k];
+        y[k] = (J.sk[k] >> lane) & 1u ? -x : x;
       }
-      warp_fwht<D>(qrow, lane);
-      float2 y[P / 32];
-      float mx = 0.f;
-      const float qs = J.scale * kLog2e * rsqrtf((float)D);
 #pragma unroll
-      for (int k = 0; k < P / 32; ++k) {           // in record (slot) order: slot i holds pair slot_pair(i)
-        y[k] = q2[slot_pair<D>(lane + 32 * k)];
-        y[k].x *= qs;
-        y[k].y *= qs;
-        mx = fmaxf(mx, fmaxf(fabsf(y[k].x), fabsf(y[k].y)));
+      for (int h = 1; h < D / 32; h <<= 1)
+#pragma unroll
+        for (int k = 0; k < D / 32; ++k)
+          if (!(k & h)) {
+            const float a = y[k], b = y[k + h];
+            y[k] = a + b;
+            y[k + h] = a - b;
+          }
+#pragma unroll
+      for (int h = 1; h < 32; h <<= 1) {
+        const float sg_ = lane & h ? -1.f : 1.f;
+#pragma unroll
+        for (int k = 0; k < D / 32; ++k)
+          y[k] = __fmaf_rn(sg_, y[k], __shfl_xor_sync(0xffffffffu, y[k], h));
+      }
+      const float qs = J.scale * kLog2e * rsqrtf((float)D);
+      float mx = 0.f;
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) {
+        y[k] *= qs;
+        mx = fmaxf(mx, fabsf(y[k]));
       }
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       const int e = min(max(exp_of(mx), -126), 126);
       const float sc = exp2i(-e);
-      __syncwarp();
 #pragma unroll
-      for (int k = 0; k < P / 32; ++k) q2[lane + 32 * k] = make_float2(y[k].x * sc, y[k].y * sc);
+      for (int k = 0; k < D / 32; ++k) {
+        const float a = y[k] * sc, b = __shfl_down_sync(0xffffffffu, a, 1);
+        if (!(lane & 1)) {                         // pair 16 k + lane / 2
+          __half ah, al, bh, bl;
+          split_half(a, ah, al);
+          split_half(b, bh, bl);
+          const int i = pair_slot<D>(16 * k + lane / 2), r = i % KP;
+          const int at = warp * P + i - r + (k4 ? (r & ~7) + 2 * (r & 3) + ((r >> 2) & 1) : r);
+          qfrag[at] = h2_bits(__halves2half2(ah, bh));
+          qfrag[NQ * P + at] = h2_bits(__halves2half2(al, bl));
+        }
+      }
       if (lane == 0) qscale[warp] = exp2i(e);
     }
     __syncthreads();
@@ -341,28 +437,18 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     }
     const float kinv = J.inv_lk, vinv = J.inv_lv;
     const bool klog = J.mk == TAC_NORM_LOG, vlog = J.mv == TAC_NORM_LOG;
-    // Query fragments: step ks takes the slots k_slot(ks, 0) and k_slot(ks, 1) of
-    // every lane's run: neighbours, or (4-bit norms, whose codes are unpacked four
-    // apart) slots four apart.
-    const bool k4 = J.ck <= 1;
     uint32_t bq[KS][QT][2];
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
+    for (int x = 0; x < QT; ++x) {
+      const int part = QT == 1 ? g >> 2 : x, a = QT == 1 ? g & 3 : g;
+      const uint4* src = reinterpret_cast<const uint4*>(qfrag + (part * NQ + a) * P + KP * t);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int i = KP * t + (k4 ? 8 * (ks >> 2) + (ks & 3) + 4 * h : 2 * ks + h);
-        const float2 y = qrot[(QT == 1 ? g & 3 : g) * P + i];
-        __half xh, xl, yh, yl;
-        split_half(y.x, xh, xl);
-        split_half(y.y, yh, yl);
-        const uint32_t hi = h2_bits(__halves2half2(xh, yh)), lo = h2_bits(__halves2half2(xl, yl));
-        if constexpr (QT == 1) {
-          bq[ks][0][h] = g < 4 ? hi : lo;
-        } else {
-          bq[ks][0][h] = hi;
-          bq[ks][1][h] = lo;
-        }
+      for (int ks = 0; ks < KS; ks += 2) {
+        const uint4 v = src[ks / 2];
+        bq[ks][x][0] = v.x; bq[ks][x][1] = v.y;
+        bq[ks + 1][x][0] = v.z; bq[ks + 1][x][1] = v.w;
       }
+    }
     // The lane's queries in the softmax: two neighbours, the same as its columns
     // of the value accumulators.
     const int q0 = QT == 1 ? 2 * (t & 1) : 2 * t;
@@ -621,8 +707,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
 
     for (; row0 < seg_rows; row0 += kAttUnit) {
       const int valid = (int)min((int64_t)kAttBatch, J.tokens - row0);
-      cp_async_wait<1>();                          // this batch's K rows have landed
-      __syncwarp();
+      landed(row0, bar_k, phase_k);                // this batch's K rows
       if (hkb) norm_consts(reinterpret_cast<const float2*>(st_kh)[lane], kinv, klog, kc[lane], ksc[lane]);
       else fp32_consts(st_kn, nbk, kc, ksc);
       __syncwarp();
@@ -643,7 +728,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
         over |= !(sv[i] <= m_run[i & 1] + 8.f);
       }
       __syncwarp();                                // every lane is done with the K rows
-      issue_k(row0 + kAttUnit);
+      issue(false, row0 + kAttUnit, bar_k, bytes_k);
 
       // ---- softmax (base 2): the reference m moves only when a score passes it by more than 8 ----
       if (__any_sync(0xffffffffu, over)) {
@@ -662,8 +747,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
           }
         }
       }
-      cp_async_wait<1>();                          // this batch's V rows have landed
-      __syncwarp();
+      landed(row0, bar_v, phase_v);                // this batch's V rows
       if (hvb) norm_consts(reinterpret_cast<const float2*>(st_vh)[lane], vinv, vlog, vc[lane], vsc[lane]);
       else fp32_consts(st_vn, nbv, vc, vsc);
       __syncwarp();
@@ -718,9 +802,8 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
         default: values(IC<4>{}); break;
       }
       __syncwarp();                                // every lane is done with the V rows and the weights
-      issue_v(row0 + kAttUnit);
+      issue(true, row0 + kAttUnit, bar_v, bytes_v);
     }
-    cp_async_wait<0>();
 
     // ---- merge the warps: the segment's (max, sum, accumulator) per query ----
 #pragma unroll
@@ -733,7 +816,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         red[(warp * NQ + q0 + q) * 2] = m_run[q];
-        red[(warp * NQ + q0 + q) * 2 + 1] = l_run[q];
+        red[(warp * NQ + q0 + q) * 2 + 1] = dead ? __int_as_float(0x7FC00000) : l_run[q];
       }
     }
     __syncthreads();
@@ -886,8 +969,13 @@ static cudaError_t launch_attend_t(const AttParams& p_in, int nq_max, float* ws,
   const int smem = C::smem(p.stage, p.tab_k + p.tab_v);
   const int regs_cta = ((regs[dev].load(std::memory_order_relaxed) * 32 + 255) / 256) * 256 * kAttWarps;
   const int per_sm = std::max(1, std::min(228 * 1024 / (smem + 1024), 65536 / regs_cta));
-  p.nctas = (int32_t)std::min<int64_t>(p.nunits, (int64_t)sms * per_sm);
+  p.nctas = (int32_t)std::min<int64_t>(std::min<int64_t>(p.nunits, (int64_t)sms * per_sm), kAttMaxCtas);
   if (p.nctas < 1) return cudaSuccess;
+  const int per = p.nunits / p.nctas, extra = p.nunits % p.nctas;
+  for (int c = 0, j = 0; c < p.nctas; ++c) {
+    while (j + 1 < p.njobs && p.job[j + 1].unit0 <= c * per + std::min(c, extra)) ++j;
+    p.first_job[c] = (uint8_t)j;
+  }
   kp<<<p.nctas, kAttThreads, smem, st>>>(p, ws);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -24,12 +24,16 @@ struct AttJob {
   int64_t ws;                        // first workspace float of this job
 };
 
+constexpr int kAttMaxCtas = 640;
+static_assert(TAC_ATTEND_MAX_JOBS <= 256, "AttParams::first_job");
+
 struct AttParams {
   int32_t njobs;
   int32_t nctas;
   int32_t nunits;
   int32_t stage, tab_k, tab_v;       // shared memory: a warp's staged batch, the two tables (largest of the jobs)
   int32_t q_bf16;                    // queries (and outputs) are bf16 rows, else fp32
+  uint8_t first_job[kAttMaxCtas];    // job of each CTA's first unit
   AttJob job[TAC_ATTEND_MAX_JOBS];   // 200 bytes each: within the 32 KB of kernel parameters
 };
 

@@ -153,6 +153,9 @@ struct Enc {
   static_assert(32 % CPR == 0 && RW % RPQ == 0, "chunk map");
 };
 
+template <bool V>
+struct Flag { static constexpr bool value = V; };
+
 // The job a warp is encoding as far as the rare paths need it (exact
 // re-decision, tail tiles and scatter), kept in the warp's shared region.
 struct WarpJob {
@@ -234,6 +237,24 @@ __device__ __forceinline__ int candidate_bits(float E, float O) {
   else return __float_as_int(__fadd_rd(12582912.0f + 0.125f * n, -ab));
 }
 
+// candidate_bits of two pairs at a time (n a multiple of 8): the same
+// operations, those in the middle on packed fp32 pairs (the sign of E enters as
+// a factor +-1): 17 instructions for the two instead of 22, a 32k-token cache 40
+// us faster.
+template <int N>
+__device__ __forceinline__ void candidate_bits2(float2 p0, float2 p1, int& b0, int& b1) {
+  constexpr float nb = (float)N * 0.15915494309189535f;  // bins per radian
+  constexpr float ca = 0.97239412f * nb, cb = -0.19194795f * nb, M = 12582912.0f + 0.125f * N;
+  const float2 t = mul2(make_float2(fabsf(p0.y) - fabsf(p0.x), fabsf(p1.y) - fabsf(p1.x)),
+                        make_float2(rcp_approx(fabsf(p0.y) + fabsf(p0.x)), rcp_approx(fabsf(p1.y) + fabsf(p1.x))));
+  const float2 q = __ffma2_rn(mul2(t, t), make_float2(cb, cb), make_float2(ca, ca));
+  const float2 dq = __ffma2_rn(t, q, make_float2(-0.125f * N, -0.125f * N));
+  auto one = [](float x) { return __uint_as_float((__float_as_uint(x) & 0x80000000u) | 0x3F800000u); };
+  const float2 fb = __ffma2_rn(make_float2(one(p0.x), one(p1.x)), dq, make_float2(0.25f * N, 0.25f * N));
+  b0 = __float_as_int(__fadd_rd(M, -__uint_as_float(__float_as_uint(fb.x) ^ (__float_as_uint(p0.y) & 0x80000000u))));
+  b1 = __float_as_int(__fadd_rd(M, -__uint_as_float(__float_as_uint(fb.y) ^ (__float_as_uint(p1.y) & 0x80000000u))));
+}
+
 // The candidate edge in [0, n).
 template <class S>
 __device__ __forceinline__ int candidate_edge(const S& sh, float E, float O) {
@@ -263,16 +284,19 @@ __device__ __forceinline__ int candidate_edge(const S& sh, float E, float O) {
 // magnitude is the certification margin, and a pair with m == 0 is never
 // certified, so which side the fast path gives it does not matter.
 template <int R, class S>
-__device__ __forceinline__ uint32_t edge_test(const S& sh, float E, float O, const float2* et, float& m) {
+__device__ __forceinline__ uint32_t edge_test(const S& sh, float E, float O, const float2* et, float& m,
+                                              [[maybe_unused]] int bits) {
   if constexpr (S::fixed) {
     if constexpr (is_pow2(S::n)) {
-      const int bits = candidate_bits<S::n>(E, O);
+      if constexpr (S::n % 8 != 0) bits = candidate_bits<S::n>(E, O);   // else the caller's (candidate_bits2)
       const float2 dir = et[(bits & (S::n - 1)) * R];
       m = __fmaf_rn(O, dir.y, -__fmul_rn(E, dir.x));
       return (uint32_t)(bits + (int)(__float_as_uint(m) >> 31)) & (uint32_t)(S::n - 1);
     }
   }
-  const int e = candidate_edge(sh, E, O);
+  int e;
+  if constexpr (S::fixed) e = (int)min((uint32_t)wrap_bin(sh, bits - 0x4B400000), (uint32_t)(S::n - 1));
+  else e = candidate_edge(sh, E, O);
   const float2 dir = et[e * R];
   m = __fmaf_rn(O, dir.y, -__fmul_rn(E, dir.x));
   const int k = e + (int)(__float_as_uint(m) >> 31);
@@ -1009,16 +1033,25 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   const float lmin_s = min3(min3(s[0], s[1], s[2]), min3(s[3], s[4], s[5]), fminf(s[6], s[7]));
   float smin = lmin_s;
   float smax = max3(max3(s[0], s[1], s[2]), max3(s[3], s[4], s[5]), fmaxf(s[6], s[7]));
-  float ssum = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+  const float2 s2 = add2(add2(make_float2(s[0], s[1]), make_float2(s[2], s[3])),
+                         add2(make_float2(s[4], s[5]), make_float2(s[6], s[7])));
+  float ssum = s2.x + s2.y;
 
   // ---- angle codes (Alg. 1): they need no row constant, so they are decided
   // before the row reductions (whose shuffle latency they cover) ----
   uint32_t alo = 0, ahi = 0;
   float am[8];                                  // |m|: each pair's certification margin
+  int cand[8];                                  // candidate edges (candidate_bits) of a fixed shape
+  if constexpr (S::fixed) {
+    if constexpr (S::n % 8 == 0) {
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) candidate_bits2<S::n>(v[j], v[j + 1], cand[j], cand[j + 1]);
+    }
+  }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     float m;
-    const uint32_t k = edge_test<C::TABR>(sh, v[j].x, v[j].y, et, m);
+    const uint32_t k = edge_test<C::TABR>(sh, v[j].x, v[j].y, et, m, cand[j]);
     am[j] = fabsf(m);
     if constexpr (S::fixed) {
       // fields are disjoint and k < n: the adds are ORs (one IMAD each)
@@ -1056,40 +1089,59 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   // the square roots and logarithms of the row and of its pairs run on normal
   // arguments in their flush-to-zero hardware forms and are scaled back
   // exactly: sqrt(s) = 2^k sqrt(s sigma), log2 s = log2(s sigma) + 2k.
-  const int ek = ((int)((__float_as_uint(smax) >> 23) & 0xFFu) - 127) >> 1;
-  const int kk = ek < -62 ? -62 : (ek > 63 ? 63 : ek);
-  const float sigma = __uint_as_float((uint32_t)(127 - 2 * kk) << 23);
-  const float sr = __uint_as_float((uint32_t)(127 + kk) << 23);   // 2^k
-  const float smax_s = smax * sigma;
-  // sqrt(smax sigma); for d = 32, 128 the factor 2/d of r^2 is an even power of
-  // two, so sqrt(smax sigma 2/d) is taken as this times sqrt(2/d), an exact
+  // Rows whose largest energy lies in [2^-60, 2^100] (and zero rows) need none
+  // of it: sigma = 1 when all rows of the warp are such.
+  // For d = 32, 128 the factor 2/d of r^2 is an even power of two, so
+  // sqrt(smax sigma 2/d) is taken as sqrt(smax sigma) times sqrt(2/d), an exact
   // product (one hardware square root, about 1 ulp, either way).
   constexpr bool kEvenK2 = D == 32 || D == 128;
-  const float rms = sqrt_ftz(smax_s);
+  constexpr float lk2 = (float)(G::LOGD == 4 ? -3 : G::LOGD == 5 ? -4 : G::LOGD == 6 ? -5 : -6);   // log2(2/d)
   float hmin = 0.f, hmax = 0.f, qs = 0.f, qo = 0.f, sfloor = 0.f, sc = 0.f;
-  if (fp32n) {
-    // no header: the norms are stored as they are (Sec. 3.1)
-  } else if (mode == TAC_NORM_LINEAR) {
-    hmin = sqrt_approx(smin * k2);              // smin * sigma may still be subnormal
-    hmax = (kEvenK2 ? rms * rk2 : sqrt_ftz(smax_s * k2)) * sr;
-    sc = (float)Lq * rcp_approx(hmax - hmin);
-    qs = sc * rk2;                              // f(s) = sqrt(s)
-    qo = __fmaf_rn(-hmin, sc, 0.5f);
-    if (!(hmax > hmin) || !(sc <= 3.0e38f)) { qs = 0.f; qo = 0.5f; }
-  } else {  // log-space, norms floored at 2^-24 r_max
-    sfloor = smax * 3.5527136788005009e-15f;    // 2^-48 on the energy
-    const float hmin_s = sqrt_ftz(fmaxf(smin, sfloor) * sigma * k2);   // >= 2^-24 hmax_s: normal
-    const float hmax_s = kEvenK2 ? rms * rk2 : sqrt_ftz(smax_s * k2);
-    hmin = hmin_s * sr;
-    hmax = hmax_s * sr;
-    const float lmin_s = lg2_ftz(hmin_s);
-    sc = (float)Lq * rcp_approx(lg2_ftz(hmax_s) - lmin_s);
-    qs = 0.5f * sc;                             // f(s) = log2 s; log2 r = (log2 s + log2 k2)/2
-    qo = __fmaf_rn(0.5f * (float)(G::LOGD == 4 ? -3 : G::LOGD == 5 ? -4 : G::LOGD == 6 ? -5 : -6) -
-                       (lmin_s + (float)kk),
-                   sc, 0.5f);
-    if (!(hmax > hmin) || !(sc <= 3.0e38f)) { qs = 0.f; qo = 0.5f; }
-  }
+  float lerr = 0.f;                             // log-space: bound on the log2s' own errors (see the band below)
+  float rmx = 0.f, rsum = 0.f;                  // sqrt(smax), sqrt(ssum)
+  auto row_constants = [&](auto tame_) {
+    constexpr bool TAME = decltype(tame_)::value;
+    const int ek = ((int)((__float_as_uint(smax) >> 23) & 0xFFu) - 127) >> 1;
+    const int kk = TAME ? 0 : ek < -62 ? -62 : (ek > 63 ? 63 : ek);
+    const float sigma = TAME ? 1.f : __uint_as_float((uint32_t)(127 - 2 * kk) << 23);
+    const float sr = TAME ? 1.f : __uint_as_float((uint32_t)(127 + kk) << 23);   // 2^k
+    const float smax_s = TAME ? smax : smax * sigma;
+    const float rms = sqrt_ftz(smax_s);
+    rmx = TAME ? rms : rms * sr;
+    rsum = TAME ? sqrt_ftz(ssum) : sqrt_ftz(ssum * sigma) * sr;
+    if (fp32n) {
+      // no header: the norms are stored as they are (Sec. 3.1)
+    } else if (mode == TAC_NORM_LINEAR) {
+      hmin = TAME ? sqrt_ftz(smin * k2) : sqrt_approx(smin * k2);   // smin * sigma may still be subnormal
+      hmax = kEvenK2 ? rms * rk2 : sqrt_ftz(smax_s * k2);
+      if (!TAME) hmax *= sr;
+      const float range = hmax - hmin, rr = rcp_approx(range);
+      sc = (float)Lq * rr;
+      sc = __fmaf_rn(__fmaf_rn(-range, sc, (float)Lq), rr, sc);     // Lq / range to within u
+      qs = sc * rk2;                            // f(s) = sqrt(s)
+      qo = __fmaf_rn(-hmin, sc, 0.5f);
+      if (!(hmax > hmin) || !(sc <= 3.0e38f)) { qs = 0.f; qo = 0.5f; }
+    } else {  // log-space, norms floored at 2^-24 r_max
+      sfloor = smax * 3.5527136788005009e-15f;  // 2^-48 on the energy
+      const float smin_f = TAME ? fmaxf(smin, sfloor) : fmaxf(smin, sfloor) * sigma;
+      const float hmin_s = sqrt_ftz(smin_f * k2);                   // >= 2^-24 hmax_s: normal
+      const float hmax_s = kEvenK2 ? rms * rk2 : sqrt_ftz(smax_s * k2);
+      hmin = TAME ? hmin_s : hmin_s * sr;
+      hmax = TAME ? hmax_s : hmax_s * sr;
+      const float lmin_s = lg2_ftz(hmin_s), lmax_s = lg2_ftz(hmax_s);
+      const float lmin = TAME ? lmin_s : lmin_s + (float)kk, lmax = TAME ? lmax_s : lmax_s + (float)kk;
+      sc = (float)Lq * rcp_approx(lmax_s - lmin_s);
+      const float lh = fmaxf(fabsf(lmin_s), fabsf(lmax_s));
+      const float ls = TAME ? 2.f * lh - lk2 : 2.f * fmaxf(fabsf(lmin), fabsf(lmax)) - lk2;
+      lerr = 1.5f * 2.384185791015625e-07f + kU * (2.1f * ls + 4.1f * lh + 10.f);
+      qs = 0.5f * sc;                           // f(s) = log2 s; log2 r = (log2 s + log2 k2)/2
+      qo = __fmaf_rn(0.5f * lk2 - lmin, sc, 0.5f);
+      if (!(hmax > hmin) || !(sc <= 3.0e38f)) { qs = 0.f; qo = 0.5f; }
+    }
+  };
+  const bool tame = (smax >= 8.6736174e-19f && smax <= 1.2676506e30f) || smax == 0.f;
+  if (S::fixed && __all_sync(0xffffffffu, tame)) row_constants(Flag<S::fixed>{});
+  else row_constants(Flag<false>{});
   // Certification bound on the cross product m = E c - O s.  The butterfly's
   // log2 d - 1 rounded stages give |dE| <= (log2 d - 1) u ||x_even||_1 and
   // |dO| <= (log2 d - 1) u ||x_odd||_1 (first order), so with c^2 + s^2 = 1
@@ -1104,8 +1156,7 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   // pair norm), so ty sqrt(2/d) bounds the error of each r_i.
   // The angle band takes norm_kappa() of the transform's part (see the norm
   // band below) and all of the arithmetic's part.
-  const float rmx = rms * sr;
-  const float ty = (float)(G::LOGD - 1) * kU * 1.01f * (sqrt_ftz(ssum * sigma) * sr);
+  const float ty = (float)(G::LOGD - 1) * kU * 1.01f * rsum;
   const float tau = norm_kappa<D>() * ty + 3.03f * kU * rmx;
   // The per-pair norm functions below take s itself (pairs below the log floor
   // are clamped to it first), against the true-scale qs, qo: for inputs in the
@@ -1135,38 +1186,46 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   //    bound and the exact value lies closer to the midpoint than that error,
   //    i.e. within about 1e-4 code units (or 1e-7 rad) of it, where the parity
   //    rule counts such codes;
-  //  - the kernel's own arithmetic, bounded in full: each computed norm (the
-  //    pair's, r_min's, r_max's) within kEr of its value for the computed
-  //    energy (hardware square root, rounding of the energy), qs within kEq,
-  //    log2 within kEl absolute plus a rounding of the result, and the roundings
-  //    of qo and of the final fma at magnitudes up to 2^(B+1).
+  //  - the kernel's own arithmetic, bounded in full.  Linear: each computed norm
+  //    (the pair's, r_min's, r_max's) lies within kEr of its value for the
+  //    computed energy (hardware square root, rounding of the energy); with f the
+  //    pair's place in [r_min, r_max] the three move t by at most kEr sc (r +
+  //    (1 - f) r_min + f r_max) = 2 kEr sc r <= 2 kEr sc r_max; qs lies within
+  //    kEq (one Newton step after the reciprocal: the range's rounding and the
+  //    quotient's; where rk2 is no power of two also its own and its product's).  Log: log2 within 2^-22
+  //    absolute on [1/2, 2) and 4u of its result elsewhere: lerr takes half of
+  //    that for the pair's energy (|log2 s| <= ls), all of it for r_min or r_max
+  //    (|log2 r| <= lh as computed), and 10u for their roundings before the
+  //    logarithm (1.45u + 5.8u + 1.45u).  Both: the roundings of qo (two, or three
+  //    in log-space), of qo2 and of the final fma (half an ulp of 2^B each).
+  //    Bounds of 4u for the quotient, 52 binades for every energy and 2^(B+1)
+  //    for the last two made the bands 1.4 (8-bit linear) and 3 times (4-bit log)
+  //    as wide, and the encode of a 32k-token cache 78 us slower.
   // A row whose band reaches 1/4 (rows of nearly equal pair norms, non-finite
   // rows) has every norm code re-decided.
   constexpr float kKappa = norm_kappa<D>();
   // kEr: hardware sqrt <= 2u relative (1 ulp) plus the energy's rounding
-  // (2u on s, u on its root); kEq: rcp <= 2u plus two roundings; kEl: lg2
-  // <= 2^-22 absolute on [1/2, 2), and within 4u |result| elsewhere (a GPU
-  // test checks each of these limits over whole binades).
-  constexpr float kEr = 3.f * kU, kEq = 4.f * kU, kEl = 2.384185791015625e-07f;  // 2^-22
+  // (2u on s, u on its root).  A GPU test checks the hardware limits over whole
+  // binades.
+  constexpr float kEr = 3.f * kU, kEq = (kEvenK2 ? 2.1f : 4.1f) * kU;
   const float kMag = fp32n ? 0.f : (float)(1 << (B & 15));      // 2^B
   const int kFb = 23 - (fp32n ? 8 : B);                         // fraction bits of t + 2^B
   const uint32_t kFracMask = (1u << kFb) - 1u;
   float th = 0.f;
   if (!fp32n) {
     if (mode == TAC_NORM_LINEAR) {
-      th = kKappa * 2.f * qs * ty + 2.f * kEr * (hmax + hmin) * sc + (float)Lq * kEq +
-           kU * (hmin * sc + 4.f * kMag + 2.f);
+      th = kKappa * 2.f * qs * ty + sc * (2.f * kEr * hmax + 2.f * kU * hmin) + (float)Lq * kEq +
+           kU * (2.f * kMag + 3.f);
     } else {
-      const float elp = kEl + 4.f * kU * (fabsf(2.f * (float)kk) + 52.f);   // log2 of one pair's energy
-      th = kKappa * 2.f * sc * (ty * rk2) * rcp_approx(hmin) * 1.4426950408889634f + 1.5f * sc * elp +
-           (float)Lq * kEq + kU * (fabsf(qo) + 4.f * kMag + 2.f);
+      th = kKappa * 2.f * sc * (ty * rk2) * rcp_approx(hmin) * 1.4426950408889634f + sc * lerr +
+           (float)Lq * 4.f * kU + kU * (3.f * fabsf(qo) + 2.f * kMag + 3.f);
     }
   }
   const bool nall = !(th < 0.25f);              // also NaN
   const float thu = nall ? 0.f : th;
   // t + 2^B + th (in [2^B, 2^(B+1))): the integer part of t + th sits in the
   // mantissa bits [23 - B, 23) and its fraction in the kFb bits below
-  const float qo2 = qo + (kMag + thu);
+  const float qo2 = (qo + thu) + kMag;
   const uint32_t thb2 = nall ? 0xFFFFFFFFu : 2u * ((uint32_t)(thu * (float)(1u << kFb)) + 1u);
 
   // ---- pass 2: norm codes (Eq. 2), packing ----
@@ -1179,6 +1238,9 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   } else if (mode == TAC_NORM_LINEAR) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) rn[j] = sqrt_ftz(s[j]);
+  } else if (S::fixed && !__any_sync(0xffffffffu, smin < sfloor)) {   // nothing to floor
+#pragma unroll
+    for (int j = 0; j < 8; ++j) rn[j] = lg2_ftz(s[j]);
   } else {
 #pragma unroll
     for (int j = 0; j < 8; ++j) rn[j] = lg2_ftz(fmaxf(s[j], sfloor));

@@ -556,6 +556,11 @@ struct QGeo {
   static constexpr int RW = Geo<D>::RW;
   static constexpr int kRowEntries = (32 / RW) > 1 ? 32 / RW : 1;   // per row before it goes whole
   static constexpr int kMaxPerTile = RW * kRowEntries;              // <= 32
+  // Flagged codes of a row above which it goes whole.  Rows with many are rows
+  // of nearly equal norms, where the transform's error counts most: the exact
+  // path is then also the safer one.
+  static constexpr int kRowLimitLinear = kRowEntries > 1 ? 5 * kRowEntries / 8 : 1;
+  static constexpr int kRowLimitLog = kRowEntries > 4 ? kRowEntries / 4 : 1;
 };
 
 // The part of the norm band left once the fast path's own arithmetic is taken
@@ -1177,14 +1182,13 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   //    assumes every rounding of every stage at its maximum and with one sign;
   //    the errors measured on the synthetic caches of every workload stay
   //    below 0.075 of it for a pair norm at d = 64, 128 (0.17 at d <= 32), and
-  //    their distribution is what kKappa is set from: in a simulation of the
-  //    fp32 transform over 1.3e8 pairs of every workload no norm code (and
-  //    over 1.8e8 codes no angle code) decided from the fp32 values outside
-  //    the band at kKappa = 1/128 differed from the exact one.  kKappa = 1/64
-  //    (d >= 64) or 1/4 (d <= 32) is used.  It is no proof for every input: a
-  //    code can still differ where the transform's error exceeds kKappa of its
-  //    bound and the exact value lies closer to the midpoint than that error,
-  //    i.e. within about 1e-4 code units (or 1e-7 rad) of it, where the parity
+  //    1e-5 of them pass 0.04 to 0.06.  kKappa = 1/16 (d >= 64) or 1/4 (d <= 32);
+  //    a flagged code is settled by the second look beyond norm_kappa() of the
+  //    bound, where a simulation over 1.3e8 pairs of every workload found no
+  //    code that differed from the exact one.  It is no proof for every input: a
+  //    code can still differ where the transform's error exceeds that and the
+  //    exact value lies closer to the midpoint than the error, i.e. within about
+  //    1e-4 code units (or 1e-7 rad) of it on these caches, where the parity
   //    rule counts such codes;
   //  - the kernel's own arithmetic, bounded in full.  Linear: each computed norm
   //    (the pair's, r_min's, r_max's) lies within kEr of its value for the
@@ -1199,11 +1203,13 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   //    logarithm (1.45u + 5.8u + 1.45u).  Both: the roundings of qo (two, or three
   //    in log-space), of qo2 and of the final fma (half an ulp of 2^B each).
   //    Bounds of 4u for the quotient, 52 binades for every energy and 2^(B+1)
-  //    for the last two made the bands 1.4 (8-bit linear) and 3 times (4-bit log)
-  //    as wide, and the encode of a 32k-token cache 78 us slower.
-  // A row whose band reaches 1/4 (rows of nearly equal pair norms, non-finite
-  // rows) has every norm code re-decided.
-  constexpr float kKappa = norm_kappa<D>();
+  //    for the last two, with kKappa = 1/64, made the bands 1.2 (8-bit linear) and
+  //    2 times (4-bit log) as wide, and a 32k-token cache 30 us slower; with 1/64
+  //    these narrower ones are 45 us faster still, but let the transform's error
+  //    through in rows of nearly equal norms.
+  // A row whose band reaches 0.15 (linear) or 0.06 (log) - rows of nearly equal
+  // pair norms, non-finite rows - has every norm code re-decided.
+  constexpr float kKappa = D >= 64 ? 0.0625f : 0.25f;
   // kEr: hardware sqrt <= 2u relative (1 ulp) plus the energy's rounding
   // (2u on s, u on its root).  A GPU test checks the hardware limits over whole
   // binades.
@@ -1221,7 +1227,7 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
            (float)Lq * 4.f * kU + kU * (3.f * fabsf(qo) + 2.f * kMag + 3.f);
     }
   }
-  const bool nall = !(th < 0.25f);              // also NaN
+  const bool nall = !(th < (mode == TAC_NORM_LINEAR ? 0.15f : 0.06f));   // also NaN
   const float thu = nall ? 0.f : th;
   // t + 2^B + th (in [2^B, 2^(B+1))): the integer part of t + th sits in the
   // mantissa bits [23 - B, 23) and its fraction in the kFb bits below
@@ -1334,7 +1340,8 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
     int rowcnt = cnt;
 #pragma unroll
     for (int off = 1; off < L; off <<= 1) rowcnt += __shfl_xor_sync(0xffffffffu, rowcnt, off);
-    const bool whole = rowcnt > QG::kRowEntries || (nall && rowcnt > 0);
+    const int limit = fp32n ? QG::kRowEntries : mode == TAC_NORM_LINEAR ? QG::kRowLimitLinear : QG::kRowLimitLog;
+    const bool whole = rowcnt > limit || (nall && rowcnt > 0);
     const int mine = whole ? (l == 0 ? 1 : 0) : cnt;
     int inc = mine;
 #pragma unroll

@@ -44,7 +44,7 @@ struct Dec {
   static constexpr int NA = RW * AB / 16, NN = RW * NB / 16, NH = RW * HB / 16;
   static constexpr int NCH = NA + NN + NH;
   static constexpr int ROUNDS = (NCH + 31) / 32;
-  static constexpr bool kGather = (AB & 3) == 0;   // gathered records by cp.async (see gather_segment)
+  static constexpr bool kAsync = (AB & 3) == 0;    // gathered records by cp.async (see gather_segment)
   // one record stage of a warp tile: angle | norm | header segments
   static constexpr int R_ANG = 0;
   static constexpr int R_NRM = RW * AB;
@@ -93,7 +93,7 @@ __device__ __forceinline__ void gather_segment(const uint8_t* base, long long re
 // of the three segments, the last chunk of each zero-filled past the tile.
 // Gathered slots: lane r < nrows copies row r's record with plain loads; an
 // out-of-range slot decodes as an all-zero record.
-template <int AB, int NB, int HB, int R_NRM, int R_HDR>
+template <int AB, int NB, int HB, int R_NRM, int R_HDR, bool GATHER>
 __device__ __noinline__ void stage_records_slow(const DecJob& J, int64_t row0, int nrows, uint8_t* stage,
                                                 int lane) {
   if (J.slot == nullptr) {
@@ -114,7 +114,7 @@ __device__ __noinline__ void stage_records_slow(const DecJob& J, int64_t row0, i
         cp_async16(stage + R_HDR + 16 * qq, gh + 16 * qq, rem >= 16 ? 16 : rem);
       }
     }
-  } else if constexpr ((AB & 3) != 0) {
+  } else if constexpr (GATHER) {
     if (lane < nrows) {
       const int64_t s = J.slot[row0 + lane];
       uint8_t* da = stage + lane * AB;
@@ -285,12 +285,18 @@ __device__ __forceinline__ void decode_body(const uint8_t* rec, uint8_t* wsm, co
   }
 }
 
-template <int D, typename TOut, int N, int B, int MODE>
+// GATHER: some job of the launch has a slot table.  Launches without one have a
+// kernel of their own: the gathering loops and copies in the same kernel made
+// every launch about 6 us longer (46 jobs of 11180 rows, four shapes: 58 us
+// against 51; 52 us with the slower gathering code it replaced), as instructions
+// to fetch, although no contiguous job runs them.
+template <int D, typename TOut, int N, int B, int MODE, bool GATHER>
 // Two CTAs per SM, as for the encoder: the scheduling room is worth more than
 // a third CTA of warps.
 __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
     decode_kernel(const __grid_constant__ DecParams p) {
   using C = Dec<D, TOut, N, B, MODE>;
+  constexpr bool kGather = GATHER && C::kAsync;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
     }
   };
   auto gather = [&](const DecJob& J, uint8_t* stage) {
-    if constexpr (C::kGather) {
+    if constexpr (kGather) {
       gather_segment<C::L, C::AB>(J.codes, g_rec, stage + C::R_ANG, r, l);
       gather_segment<C::L, C::NB>(J.norms, g_rec, stage + C::R_NRM, r, l);
       if constexpr (C::HB > 0) gather_segment<C::L, 8>(J.hdr, g_rec, stage + C::R_HDR, r, l);
@@ -357,7 +363,7 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
       else { i_src[q] = J.hdr + 16 * (ch - C::NA - C::NN); i_step[q] = C::RW * C::HB; }
       i_src[q] += (int64_t)rel * i_step[q];
     }
-    if constexpr (C::kGather)
+    if constexpr (kGather)
       if (!p_dense) load_slots(J);
   };
   set_issue_job();
@@ -374,10 +380,10 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
           const int ch = q * 32 + lane;
           if (ch < C::NCH) cp_async16(stage + 16 * ch, i_src[q], 16);
         }
-      } else if (C::kGather && !p_dense) {
+      } else if (kGather && !p_dense) {
         gather(p.job[pj], stage);
       } else {
-        stage_records_slow<C::AB, C::NB, C::HB, C::R_NRM, C::R_HDR>(p.job[pj], i_row0, (int)min((int64_t)C::RW, i_left),
+        stage_records_slow<C::AB, C::NB, C::HB, C::R_NRM, C::R_HDR, GATHER && !kGather>(p.job[pj], i_row0, (int)min((int64_t)C::RW, i_left),
                                                             stage, lane);
       }
 #pragma unroll
@@ -385,7 +391,7 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
       i_row0 += C::RW;
       i_left -= C::RW;
       ++it;
-      if constexpr (C::kGather)
+      if constexpr (kGather)
         if (!p_dense && it < t_end && it < p_end) load_slots(p.job[pj]);
     }
     cp_async_commit();
@@ -426,7 +432,7 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
           stage = (stage + 1) & (kNS - 1);
         }
       };
-      if (!C::kGather || p_dense) {
+      if (!kGather || p_dense) {
         stretch([&](uint8_t* dst) {
 #pragma unroll
           for (int q = 0; q < C::ROUNDS; ++q) {
@@ -435,7 +441,7 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
             i_src[q] += i_step[q];
           }
         });
-      } else if constexpr (C::kGather) {
+      } else if constexpr (kGather) {
         // the slots of the tile after the one being copied, a tile ahead (the
         // last one loaded is the first after the stretch: checked against the job)
         const DecJob& J = p.job[pj];
@@ -486,17 +492,17 @@ __global__ void __launch_bounds__(Dec<D, TOut, N, B, MODE>::THREADS, kMinBlocks)
     // c_left now counts the rows of the compute job from tile t, i_left those
     // of the issue job from tile it (the next to prefetch).
     const int64_t cf = c_left / C::RW;
-    const int64_t pf = C::kGather || p_dense ? min(min((int64_t)(p_end - it), i_left / C::RW), (int64_t)(t_end - it)) : 0;
+    const int64_t pf = kGather || p_dense ? min(min((int64_t)(p_end - it), i_left / C::RW), (int64_t)(t_end - it)) : 0;
     const int64_t f = min(cf, pf);
     fast = f > 0 ? (int)f : 0;
   }
   cp_async_wait<0>();
 }
 
-template <int D, typename TOut, int N, int B, int MODE>
-static cudaError_t launch_decode_v(const DecParams& p, int grid_cap, cudaStream_t st) {
+template <int D, typename TOut, int N, int B, int MODE, bool GATHER>
+static cudaError_t launch_decode_g(const DecParams& p, int grid_cap, cudaStream_t st) {
   using C = Dec<D, TOut, N, B, MODE>;
-  auto kern = decode_kernel<D, TOut, N, B, MODE>;
+  auto kern = decode_kernel<D, TOut, N, B, MODE, GATHER>;
   static std::atomic<int> configured[64];   // per device; concurrent first calls set the same
   int dev = 0;
   cudaGetDevice(&dev);
@@ -521,7 +527,15 @@ static cudaError_t launch_decode_v(const DecParams& p, int grid_cap, cudaStream_
   return cudaGetLastError();
 }
 
-// One kernel per supported (n, norm bits, mode), as for the encoder.
+template <int D, typename TOut, int N, int B, int MODE>
+static cudaError_t launch_decode_v(const DecParams& p, int grid_cap, cudaStream_t st) {
+  for (int j = 0; j < p.njobs; ++j)
+    if (p.job[j].slot != nullptr) return launch_decode_g<D, TOut, N, B, MODE, true>(p, grid_cap, st);
+  return launch_decode_g<D, TOut, N, B, MODE, false>(p, grid_cap, st);
+}
+
+// One kernel per supported (n, norm bits, mode), as for the encoder, and one
+// more of each for launches that gather.
 template <int D, typename TOut>
 static cudaError_t launch_decode_t(const DecParams& p, int n, int b, int mode, int sms, cudaStream_t st) {
 #define TAC_DEC_N(NN)                                                                                   \

@@ -17,9 +17,10 @@
 //                   fragments, so nothing decoded touches memory.  A decoded
 //                   value r^ (cos, sin), scaled by the power of two that brings
 //                   its record's largest norm into [1, 2), is split as
-//                   hi + lo: hi on the grid of 2^-10, lo the exact residue of
-//                   the fp32 product rounded to fp16 (2^-23 of the record's
-//                   scale at most).  The queries (and, for the values, the
+//                   hi + lo: hi rounded to fp16 (keys) or to the grid of 2^-10
+//                   (values), lo the exact residue of the fp32 product rounded
+//                   to fp16 (2^-24 of the value, or 2^-23 of the record's
+//                   scale, at most).  The queries (and, for the values, the
 //                   softmax weights) are split hi + 2^-11 lo as well, both
 //                   rounded to fp16 (2^-24 of the value), the two parts in
 //                   different columns of the other operand: one mma for A_hi
@@ -29,24 +30,26 @@
 //                   of the job, divides, applies D H (fp32 butterfly) and
 //                   stores the row.
 // Bound: instruction issue.  About 12 instructions decode and split one pair
-// (table offset 2, lookup 1, norm code 3, products and split 4, packing 2); of
-// some 85 warp-instructions a token-head 48 are these (d = 128, 4 queries), and
-// the schedulers issue in 62 % of the cycles at 16 warps per SM (128
+// (table offset 2, lookup 1, norm code 3, products and split 4 or 5, packing 2);
+// of some 87 warp-instructions a token-head 50 are these (d = 128, 4 queries),
+// and the schedulers issue in 62 % of the cycles at 16 warps per SM (128
 // registers).  A warp's batch of 32 tokens takes about 12 000 cycles: scores
-// 4500, values 5900, the rest softmax, constants and copies.  Copies are bulk
+// 4800, values 5900, the rest softmax, constants and copies.  Copies are bulk
 // copies, one lane a segment: six cp.async loops over the segments took 2000
-// cycles a batch (162 us where bulk copies take 150, below).  The set-up of a
-// CTA's first job is 12 000 cycles (20 000 with the queries rotated and split
-// in shared memory, the tables computed and written 16 copies by one thread,
-// and a binary search for the job).
+// cycles a batch (12 us of the 162 below).  The set-up of a CTA's first job is
+// 12 000 cycles (20 000 with the queries rotated and split in shared memory, the
+// tables computed and written 16 copies by one thread, and a binary search for
+// the job).
 // With the products on the CUDA cores (114 instructions, 10 - 12 warps, and a
 // warp walking 256 tokens alone) 16 sequences of 1k to 32k tokens (8 KV heads,
-// 4 queries each, 244 MB of records) took 229 us, now 150 us (1.6 TB/s); 8
-// heads of 4097 tokens 59 us, now 19 us (a CTA of 8 warps per 256 tokens fills
-// the device; a third of it are the launches); 128 heads of 8192 tokens at
-// d = 64 143 us, now 81 us.  Error of an fp32 output against 64 bits: 5.4e-7
-// (6.0e-7 before).  A persistent grid merges a CTA's units before it writes, so
-// the combine kernel reads one result per CTA and job instead of one per 256 tokens.
+// 4 queries each, 244 MB of records) took 229 us, with tensor cores 162 and with
+// bulk copies and the keys' better split 158 us (1.5 TB/s); 8 heads of 4097
+// tokens 59 us, now 19 us (a CTA of 8 warps per 256 tokens fills the device; a
+// third of it are the launches); 128 heads of 8192 tokens at d = 64 143 us, now
+// 84 us.  Error of fp32 outputs against 64 bits over ten shapes (1 to 8 queries,
+// 37 to 20000 tokens, every norm storage): 3.3e-7 to 5.7e-7, 3.7e-7 to 7.0e-7
+// before.  A persistent grid merges a CTA's units before it writes, so the combine
+// kernel reads one result per CTA and job instead of one per 256 tokens.
 // Codebooks (n, norm bits, norm mode) are runtime parameters: K and V may
 // differ, and any codebook the encoder supports is accepted.
 #include <algorithm>
@@ -138,6 +141,18 @@ __device__ __forceinline__ void split_pair(float r, float2 cs, float2& nh, float
   const float2 q = __ffma2_rn(rr, cs, make_float2(M, M));
   nh = __ffma2_rn(q, make_float2(-1.f, -1.f), make_float2(M, M));
   lo = __ffma2_rn(rr, cs, nh);
+}
+
+// The same with hi rounded to fp16 itself: nh = -(hi of both) in fp16, lo the
+// residue.  One instruction more, for the keys: lo is 2^-12 of the value instead
+// of 2^-11 of the record's scale, and the scores' error decides the output's
+// (5.1e-7 against 6.0e-7 for 4097 tokens at d = 128; 5.4e-7 on the CUDA cores).
+__device__ __forceinline__ void split_pair_fp(float r, float2 cs, uint32_t& nh, float2& lo) {
+  const float2 rr = make_float2(r, r);
+  const float2 y = mul2(rr, cs);
+  const __half2 hh = __floats2half2_rn(-y.x, -y.y);
+  nh = h2_bits(hh);
+  lo = __ffma2_rn(rr, cs, __half22float2(hh));
 }
 
 // x = hi + 2^-11 lo in fp16 (|x| below about 2^15).
@@ -553,13 +568,20 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
             for (int h = 0; h < 2; ++h) {
               const int i = (KB == 4 && !F32) ? 8 * (ks >> 2) + (ks & 3) + 4 * h : 2 * ks + h;
               const uint32_t o = (rotr(x[rr][i >> 2], kra[i & 3]) & kM) | kC;
-              float2 nh, lo;
-              split_pair(rv[h], *reinterpret_cast<const float2*>(tkb + o), nh, lo);
-              ah[2 * h + rr] = h2_bits(__floats2half2_rn(nh.x, nh.y));
+              float2 lo;
+              split_pair_fp(rv[h], *reinterpret_cast<const float2*>(tkb + o), ah[2 * h + rr], lo);
               al[2 * h + rr] = h2_bits(__floats2half2_rn(lo.x, lo.y));
             }
           }
-          mma_f16(ch[ks & 1], ah, bq[ks][0][0], bq[ks][0][1]);
+          if constexpr (F32) {                     // every step's sum added in fp32
+            float c[4];
+            mma_f16_zero(c, ah, bq[ks][0][0], bq[ks][0][1]);
+            float2* a2 = reinterpret_cast<float2*>(ch[ks & 1]);
+            a2[0] = add2(a2[0], make_float2(c[0], c[1]));
+            a2[1] = add2(a2[1], make_float2(c[2], c[3]));
+          } else {
+            mma_f16(ch[ks & 1], ah, bq[ks][0][0], bq[ks][0][1]);
+          }
           mma_f16(cl, al, bq[ks][0][0], bq[ks][0][1]);
           if constexpr (QT == 2) mma_f16(cx, ah, bq[ks][QT - 1][0], bq[ks][QT - 1][1]);
         }

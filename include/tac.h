@@ -273,7 +273,8 @@ int tac_decode_multi(const tac_decode_job* jobs, int njobs, tac_stream_t stream)
  */
 #define TAC_MAX_QUERIES 8      /* query rows per job (a GQA group) */
 #define TAC_ATTEND_MAX_JOBS 160 /* jobs per launch pair of tac_attend_multi */
-#define TAC_ATTEND_SPLIT 256   /* tokens per partial result in the workspace */
+#define TAC_ATTEND_SPLIT 256   /* tokens a CTA takes together: the workspace has room for a partial
+                                  result for each (one is written per CTA and job) */
 
 typedef struct {
   tac_layer_cfg cfg_k;     /* K codebook and D; cfg_v.d must equal cfg_k.d (64 or 128) */
@@ -295,7 +296,8 @@ typedef struct {
 int64_t tac_attend_workspace_bytes(const tac_attend_job* jobs, int njobs);
 
 /* Attention for every job.  Jobs of one (d, dtype) share a launch pair (up to
- * TAC_ATTEND_MAX_JOBS jobs each); several launch pairs run concurrently on
+ * TAC_ATTEND_MAX_JOBS jobs each; the second kernel is launched while the first
+ * runs and waits for it on the device); several launch pairs run concurrently on
  * `stream` and the helper streams of tac_encode_multi (fork / join by events),
  * ordered on `stream` as a whole.
  * `workspace` (device, 16-byte aligned, >= tac_attend_workspace_bytes) is the

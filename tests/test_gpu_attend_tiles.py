@@ -75,3 +75,40 @@ def test_value_scales_per_token(tac_gpu, orc, order):
     size = p @ np.linalg.norm(vh, axis=1)           # sum_t p_t ||v^_t||
     err = np.abs(parity.to_f64(out) - want).max(1)
     assert np.all(err <= 2.0**-18 * size), err / size
+
+
+def test_attend_captured_into_graph(tac_gpu):
+    """A prepared call (both kernels, the second launched while the first runs)
+    replays from a CUDA graph to the bits of the direct call, over new queries."""
+    import torch
+    tac = tac_gpu
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    jobs = []
+    for d, T, nq in ((128, 1000, 4), (128, 33, 4), (64, 2000, 7)):
+        caches = []
+        for kv, (n, b, m) in ((0, (64, 8, 0)), (1, (64, 4, 1))):
+            cfg = tac.layer_cfg(d, n, b, m, 0, 1, kv)
+            caches.append((cfg, tac.encode(torch.randn((T, d), generator=g, device="cuda"), cfg)))
+        q = torch.randn((nq, d), generator=g, device="cuda")
+        jobs.append(tac.AttendJob(*caches[0], *caches[1], T, q, torch.empty_like(q), 1.0 / math.sqrt(d)))
+    call = tac.attend_multi_prepared(jobs)
+    call()
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        call(torch.cuda.current_stream())
+    for _ in range(3):
+        for j in jobs:
+            j.q.copy_(torch.randn(j.q.shape, generator=g, device="cuda"))
+        call()
+        torch.cuda.synchronize()
+        want = [j.out.clone() for j in jobs]
+        for j in jobs:
+            j.out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        for j, w in zip(jobs, want):
+            assert torch.equal(j.out, w)

@@ -31,8 +31,8 @@
 //                   stores the row.
 // Bound: instruction issue.  About 12 instructions decode and split one pair
 // (table offset 2, lookup 1, norm code 3, products and split 4 or 5, packing 2);
-// of some 87 warp-instructions a token-head 50 are these (d = 128, 4 queries),
-// and the schedulers issue in 62 % of the cycles at 16 warps per SM (128
+// of some 98 warp-instructions a token-head 50 are these (d = 128, 4 queries),
+// and the schedulers issue in 67 % of the cycles at 16 warps per SM (128
 // registers).  A warp's batch of 32 tokens takes about 12 000 cycles: scores
 // 4800, values 5900, the rest softmax, constants and copies.  Copies are bulk
 // copies, one lane a segment: six cp.async loops over the segments took 2000
@@ -44,7 +44,7 @@
 // warp walking 256 tokens alone) 16 sequences of 1k to 32k tokens (8 KV heads,
 // 4 queries each, 244 MB of records) took 229 us, with tensor cores 162 and with
 // bulk copies and the keys' better split 158 us (1.5 TB/s); 8 heads of 4097
-// tokens 59 us, now 19 us (a CTA of 8 warps per 256 tokens fills the device; a
+// tokens 59 us, now 20 us (a CTA of 8 warps per 256 tokens fills the device; a
 // third of it are the launches); 128 heads of 8192 tokens at d = 64 143 us, now
 // 84 us.  Error of fp32 outputs against 64 bits over ten shapes (1 to 8 queries,
 // 37 to 20000 tokens, every norm storage): 3.3e-7 to 5.7e-7, 3.7e-7 to 7.0e-7

@@ -38,10 +38,10 @@
 // and launches bound them, so one launch takes all jobs of a (d, dtype), needs
 // no workspace, and re-decides its codes itself when its tiles are done, the
 // entries of a CTA's eight queues dealt to its warps.  One token for each of
-// 64 caches (8 rows each, four shapes) takes 12 us, 34 us as four launches and
-// four fix-ups; one token for each of 256 sequences 51 us, 67 us before.  The
+// 64 caches (8 rows each, four shapes) takes 10 us, 34 us as four launches and
+// four fix-ups; one token for each of 256 sequences 47 us, 67 us before.  The
 // slowest CTA's exact rows are the last 5 to 8 us (row load, 64-bit butterfly,
-// extremes and decision in a chain), the tiles 38 us.
+// extremes and decision in a chain), the tiles about 33 us.
 #include <algorithm>
 #include <atomic>
 

@@ -43,8 +43,8 @@ FALLBACK_HBM_GBS = 6800.0
 # so its traffic is this figure times its rows.  Each figure holds only for the
 # kernel sources it was measured on; after any change to them it reads null.
 MEASURED_TRAFFIC = {
-    "encode": {"sources": ("tac_common.cuh", "tac_encode.cu"), "sha256_16": "dace7d0d44c2467c",
-               "bytes_per_row": 337.948},
+    "encode": {"sources": ("tac_common.cuh", "tac_encode.cu"), "sha256_16": "e224be8193223fa7",
+               "bytes_per_row": 338.784},
     "decode": {"sources": ("tac_common.cuh", "tac_decode.cu"), "sha256_16": "7e243c787a12fa2b",
                "bytes_per_row": 305.417},
     "attend": {"sources": ("tac_common.cuh", "tac_attend.cuh", "tac_attend.cu"), "sha256_16": "602fd2051d6e7948",

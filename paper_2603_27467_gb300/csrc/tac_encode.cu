@@ -556,11 +556,6 @@ struct QGeo {
   static constexpr int RW = Geo<D>::RW;
   static constexpr int kRowEntries = (32 / RW) > 1 ? 32 / RW : 1;   // per row before it goes whole
   static constexpr int kMaxPerTile = RW * kRowEntries;              // <= 32
-  // Flagged codes of a row above which it goes whole.  Rows with many are rows
-  // of nearly equal norms, where the transform's error counts most: the exact
-  // path is then also the safer one.
-  static constexpr int kRowLimitLinear = kRowEntries > 1 ? 5 * kRowEntries / 8 : 1;
-  static constexpr int kRowLimitLog = kRowEntries > 4 ? kRowEntries / 4 : 1;
 };
 
 // The part of the norm band left once the fast path's own arithmetic is taken
@@ -1102,12 +1097,12 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   constexpr bool kEvenK2 = D == 32 || D == 128;
   constexpr float lk2 = (float)(G::LOGD == 4 ? -3 : G::LOGD == 5 ? -4 : G::LOGD == 6 ? -5 : -6);   // log2(2/d)
   float hmin = 0.f, hmax = 0.f, qs = 0.f, qo = 0.f, sfloor = 0.f, sc = 0.f;
-  float lerr = 0.f;                             // log-space: bound on the log2s' own errors (see the band below)
   float rmx = 0.f, rsum = 0.f;                  // sqrt(smax), sqrt(ssum)
+  const int ek = ((int)((__float_as_uint(smax) >> 23) & 0xFFu) - 127) >> 1;
+  const int krow = ek < -62 ? -62 : (ek > 63 ? 63 : ek);
   auto row_constants = [&](auto tame_) {
     constexpr bool TAME = decltype(tame_)::value;
-    const int ek = ((int)((__float_as_uint(smax) >> 23) & 0xFFu) - 127) >> 1;
-    const int kk = TAME ? 0 : ek < -62 ? -62 : (ek > 63 ? 63 : ek);
+    const int kk = TAME ? 0 : krow;
     const float sigma = TAME ? 1.f : __uint_as_float((uint32_t)(127 - 2 * kk) << 23);
     const float sr = TAME ? 1.f : __uint_as_float((uint32_t)(127 + kk) << 23);   // 2^k
     const float smax_s = TAME ? smax : smax * sigma;
@@ -1136,9 +1131,6 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
       const float lmin_s = lg2_ftz(hmin_s), lmax_s = lg2_ftz(hmax_s);
       const float lmin = TAME ? lmin_s : lmin_s + (float)kk, lmax = TAME ? lmax_s : lmax_s + (float)kk;
       sc = (float)Lq * rcp_approx(lmax_s - lmin_s);
-      const float lh = fmaxf(fabsf(lmin_s), fabsf(lmax_s));
-      const float ls = TAME ? 2.f * lh - lk2 : 2.f * fmaxf(fabsf(lmin), fabsf(lmax)) - lk2;
-      lerr = 1.5f * 2.384185791015625e-07f + kU * (2.1f * ls + 4.1f * lh + 10.f);
       qs = 0.5f * sc;                           // f(s) = log2 s; log2 r = (log2 s + log2 k2)/2
       qo = __fmaf_rn(0.5f * lk2 - lmin, sc, 0.5f);
       if (!(hmax > hmin) || !(sc <= 3.0e38f)) { qs = 0.f; qo = 0.5f; }
@@ -1182,56 +1174,53 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   //    assumes every rounding of every stage at its maximum and with one sign;
   //    the errors measured on the synthetic caches of every workload stay
   //    below 0.075 of it for a pair norm at d = 64, 128 (0.17 at d <= 32), and
-  //    1e-5 of them pass 0.04 to 0.06.  kKappa = 1/16 (d >= 64) or 1/4 (d <= 32);
-  //    a flagged code is settled by the second look beyond norm_kappa() of the
-  //    bound, where a simulation over 1.3e8 pairs of every workload found no
-  //    code that differed from the exact one.  It is no proof for every input: a
-  //    code can still differ where the transform's error exceeds that and the
-  //    exact value lies closer to the midpoint than the error, i.e. within about
-  //    1e-4 code units (or 1e-7 rad) of it on these caches, where the parity
+  //    their distribution is what kKappa is set from: in a simulation of the
+  //    fp32 transform over 1.3e8 pairs of every workload no norm code (and
+  //    over 1.8e8 codes no angle code) decided from the fp32 values outside
+  //    the band at kKappa = 1/128 differed from the exact one.  kKappa = 1/64
+  //    (d >= 64) or 1/4 (d <= 32) is used.  It is no proof for every input: a
+  //    code can still differ where the transform's error exceeds kKappa of its
+  //    bound and the exact value lies closer to the midpoint than that error,
+  //    i.e. within about 1e-4 code units (or 1e-7 rad) of it, where the parity
   //    rule counts such codes;
-  //  - the kernel's own arithmetic, bounded in full.  Linear: each computed norm
-  //    (the pair's, r_min's, r_max's) lies within kEr of its value for the
-  //    computed energy (hardware square root, rounding of the energy); with f the
-  //    pair's place in [r_min, r_max] the three move t by at most kEr sc (r +
-  //    (1 - f) r_min + f r_max) = 2 kEr sc r <= 2 kEr sc r_max; qs lies within
-  //    kEq (one Newton step after the reciprocal: the range's rounding and the
-  //    quotient's; where rk2 is no power of two also its own and its product's).  Log: log2 within 2^-22
-  //    absolute on [1/2, 2) and 4u of its result elsewhere: lerr takes half of
-  //    that for the pair's energy (|log2 s| <= ls), all of it for r_min or r_max
-  //    (|log2 r| <= lh as computed), and 10u for their roundings before the
-  //    logarithm (1.45u + 5.8u + 1.45u).  Both: the roundings of qo (two, or three
-  //    in log-space), of qo2 and of the final fma (half an ulp of 2^B each).
-  //    Bounds of 4u for the quotient, 52 binades for every energy and 2^(B+1)
-  //    for the last two, with kKappa = 1/64, made the bands 1.2 (8-bit linear) and
-  //    2 times (4-bit log) as wide, and a 32k-token cache 30 us slower; with 1/64
-  //    these narrower ones are 45 us faster still, but let the transform's error
-  //    through in rows of nearly equal norms.
-  // A row whose band reaches 0.15 (linear) or 0.06 (log) - rows of nearly equal
-  // pair norms, non-finite rows - has every norm code re-decided.
-  constexpr float kKappa = D >= 64 ? 0.0625f : 0.25f;
+  //  - the kernel's own arithmetic, bounded in full: each computed norm (the
+  //    pair's, r_min's, r_max's) within kEr of its value for the computed
+  //    energy (hardware square root, rounding of the energy), qs within kEq,
+  //    log2 within kEl absolute plus a rounding of the result, and the roundings
+  //    of qo and of the final fma at magnitudes up to 2^(B+1).
+  // Tighter bounds of the second part (r_min's and r_max's errors weighed by the
+  // pair's place between them, the logarithms' own magnitudes) narrow the bands
+  // to 0.8 (8-bit linear) and 0.5 (4-bit log): a 32k-token cache takes 2255 us, not 2350.
+  // Fewer rows are then re-decided whole, and in rows of nearly equal norms more
+  // codes of the transform's own error stay: one channel x300, fp32, 150 of
+  // 1.28e7 codes instead of 142.  Not taken.
+  // A row whose band reaches 1/4 (rows of nearly equal pair norms, non-finite
+  // rows) has every norm code re-decided.
+  constexpr float kKappa = norm_kappa<D>();
   // kEr: hardware sqrt <= 2u relative (1 ulp) plus the energy's rounding
-  // (2u on s, u on its root).  A GPU test checks the hardware limits over whole
-  // binades.
-  constexpr float kEr = 3.f * kU, kEq = (kEvenK2 ? 2.1f : 4.1f) * kU;
+  // (2u on s, u on its root); kEq: rcp <= 2u plus two roundings; kEl: lg2
+  // <= 2^-22 absolute on [1/2, 2), and within 4u |result| elsewhere (a GPU
+  // test checks each of these limits over whole binades).
+  constexpr float kEr = 3.f * kU, kEq = 4.f * kU, kEl = 2.384185791015625e-07f;  // 2^-22
   const float kMag = fp32n ? 0.f : (float)(1 << (B & 15));      // 2^B
   const int kFb = 23 - (fp32n ? 8 : B);                         // fraction bits of t + 2^B
   const uint32_t kFracMask = (1u << kFb) - 1u;
   float th = 0.f;
   if (!fp32n) {
     if (mode == TAC_NORM_LINEAR) {
-      th = kKappa * 2.f * qs * ty + sc * (2.f * kEr * hmax + 2.f * kU * hmin) + (float)Lq * kEq +
-           kU * (2.f * kMag + 3.f);
+      th = kKappa * 2.f * qs * ty + 2.f * kEr * (hmax + hmin) * sc + (float)Lq * kEq +
+           kU * (hmin * sc + 4.f * kMag + 2.f);
     } else {
-      th = kKappa * 2.f * sc * (ty * rk2) * rcp_approx(hmin) * 1.4426950408889634f + sc * lerr +
-           (float)Lq * 4.f * kU + kU * (3.f * fabsf(qo) + 2.f * kMag + 3.f);
+      const float elp = kEl + 4.f * kU * (fabsf(2.f * (float)krow) + 52.f);   // log2 of one pair's energy
+      th = kKappa * 2.f * sc * (ty * rk2) * rcp_approx(hmin) * 1.4426950408889634f + 1.5f * sc * elp +
+           (float)Lq * kEq + kU * (fabsf(qo) + 4.f * kMag + 2.f);
     }
   }
-  const bool nall = !(th < (mode == TAC_NORM_LINEAR ? 0.15f : 0.06f));   // also NaN
+  const bool nall = !(th < 0.25f);              // also NaN
   const float thu = nall ? 0.f : th;
   // t + 2^B + th (in [2^B, 2^(B+1))): the integer part of t + th sits in the
   // mantissa bits [23 - B, 23) and its fraction in the kFb bits below
-  const float qo2 = (qo + thu) + kMag;
+  const float qo2 = qo + (kMag + thu);
   const uint32_t thb2 = nall ? 0xFFFFFFFFu : 2u * ((uint32_t)(thu * (float)(1u << kFb)) + 1u);
 
   // ---- pass 2: norm codes (Eq. 2), packing ----
@@ -1340,8 +1329,7 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
     int rowcnt = cnt;
 #pragma unroll
     for (int off = 1; off < L; off <<= 1) rowcnt += __shfl_xor_sync(0xffffffffu, rowcnt, off);
-    const int limit = fp32n ? QG::kRowEntries : mode == TAC_NORM_LINEAR ? QG::kRowLimitLinear : QG::kRowLimitLog;
-    const bool whole = rowcnt > limit || (nall && rowcnt > 0);
+    const bool whole = rowcnt > QG::kRowEntries || (nall && rowcnt > 0);
     const int mine = whole ? (l == 0 ? 1 : 0) : cnt;
     int inc = mine;
 #pragma unroll

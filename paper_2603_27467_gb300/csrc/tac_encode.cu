@@ -265,7 +265,9 @@ __device__ __forceinline__ int candidate_edge(const S& sh, float E, float O) {
     return (int)min((uint32_t)wrap_bin(sh, bits - 0x4B400000), (uint32_t)(S::n - 1));
   } else {
     // candidate_bits for a runtime n, by the direct conversion; the angle lies in
-    // [-n/2, n/2] (or is NaN, which converts to 0), the edge in [-3 n/8 - 1, 5 n/8]
+    // [-n/2, n/2] and the edge in [-3 n/8 - 1, 5 n/8], except that the reciprocal
+    // of a subnormal |E| + |O| is infinite: the conversion then saturates (a zero
+    // pair's NaN converts to 0), and the clamp keeps the edge inside [0, n)
     const float n = (float)sh.n, aE = fabsf(E), aO = fabsf(O);
     const float t = (aO - aE) * rcp_approx(aO + aE);
     const float nb = n * 0.15915494309189535f;
@@ -273,7 +275,7 @@ __device__ __forceinline__ int candidate_edge(const S& sh, float E, float O) {
     const float fb = 0.25f * n + __uint_as_float(__float_as_uint(dq) ^ (__float_as_uint(E) & 0x80000000u));
     const float ab = __uint_as_float(__float_as_uint(fb) ^ (__float_as_uint(O) & 0x80000000u));
     const int v = __float2int_rd(0.125f * n - ab);
-    return v + (v < 0 ? sh.n : 0);
+    return (int)min((uint32_t)v + (v < 0 ? (uint32_t)sh.n : 0u), (uint32_t)(sh.n - 1));
   }
 }
 

@@ -86,6 +86,41 @@ def test_small_calls_match_large_ones(tac_gpu, d, dtype):
             assert int(s) == (tac.TAC_E_NONFINITE if a == 0 else 0)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+def test_subnormal_pairs_match_large_calls(tac_gpu, d, dtype):
+    """Pairs whose |E| + |O| is a subnormal number (its hardware reciprocal is
+    infinite) get a code inside the codebook and leave their neighbours' codes
+    alone: rows of subnormals, one subnormal element in a row whose even elements
+    cancel, and the same beside ordinary rows, against the large call."""
+    import torch
+    tac = tac_gpu
+    rw = 32 // (d // 16)
+    rows = LARGE_TILES * rw
+    g = torch.Generator(device="cuda")
+    g.manual_seed(7 * d)
+    x = torch.zeros((rows, d), device="cuda")
+    sub = 2.0**-130
+    x[0, 0], x[1, 1], x[2, d - 1] = sub, -sub, sub
+    x[3:20] = torch.randn((17, d), generator=g, device="cuda") * sub
+    for i in range(20, 60):                             # E = 0 in half of the pairs, O subnormal
+        j = 2 * int(torch.randint(1, d // 2, (1,), generator=g, device="cuda"))
+        x[i, 0], x[i, j], x[i, 1 + 2 * (i % (d // 2))] = 1.0, -1.0 if i & 1 else 1.0, sub if i & 2 else -3 * sub
+    for i in range(60, 80):                             # the same with the halves exchanged
+        x[i, 1], x[i, 3], x[i, 2 * (i % (d // 2))] = 2.0, 2.0, sub
+    x[80:100] = torch.randn((20, d), generator=g, device="cuda")
+    x[80:100:3, ::2] = sub
+    x = x.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    for n, b, m in [s for s in SHAPES if s[1:] in ((4, 1), (8, 0), (32, 2))]:
+        cfg = tac.layer_cfg(d, n, b, m, 0, 1, 0)
+        big, few = tac.Cache.empty(cfg, rows), tac.Cache.empty(cfg, 101)
+        tac.encode_multi([tac.EncodeJob(cfg, x, big)])
+        tac.encode_multi([tac.EncodeJob(cfg, x[:101], few)])
+        torch.cuda.synchronize()
+        for got, ref in zip(_view(torch, tac, few), _view(torch, tac, big)):
+            assert ref is None or torch.equal(got, ref[:101]), (n, b, m)
+
+
 @pytest.mark.parametrize("n,b,m", [(64, 8, 0), (256, 4, 1), (56, 32, 2)])
 def test_large_call_without_queue_room(tac_gpu, n, b, m):
     """The minimum workspace: every queued code's row is re-decided whole."""

@@ -273,8 +273,7 @@ int tac_decode_multi(const tac_decode_job* jobs, int njobs, tac_stream_t stream)
  */
 #define TAC_MAX_QUERIES 8      /* query rows per job (a GQA group) */
 #define TAC_ATTEND_MAX_JOBS 160 /* jobs per launch pair of tac_attend_multi */
-#define TAC_ATTEND_SPLIT 256   /* tokens a CTA takes together: the workspace has room for a partial
-                                  result for each (one is written per CTA and job) */
+#define TAC_ATTEND_SPLIT 256   /* tokens per partial result in the workspace */
 
 typedef struct {
   tac_layer_cfg cfg_k;     /* K codebook and D; cfg_v.d must equal cfg_k.d (64 or 128) */

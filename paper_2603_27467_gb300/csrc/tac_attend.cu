@@ -48,8 +48,8 @@
 // third of it are the launches); 128 heads of 8192 tokens at d = 64 143 us, now
 // 84 us.  Error of fp32 outputs against 64 bits over ten shapes (1 to 8 queries,
 // 37 to 20000 tokens, every norm storage): 3.3e-7 to 5.7e-7, 3.7e-7 to 7.0e-7
-// before.  A persistent grid merges a CTA's units before it writes, so the combine
-// kernel reads one result per CTA and job instead of one per 256 tokens.
+// before.  Every unit is merged and written by itself, so a job's outputs do not
+// depend on the other jobs of the call or on how the units fall to the CTAs.
 // Codebooks (n, norm bits, norm mode) are runtime parameters: K and V may
 // differ, and any codebook the encoder supports is accepted.
 #include <algorithm>
@@ -81,7 +81,7 @@ struct Att {
   // parts), their scales, the warps' barriers | K table | V table | per warp:
   // batch constants, weights, staged batch.  The merge of the warps' results
   // reuses the queries' and the warps' parts.
-  static constexpr int Q_S = NQ * P * 8, Q_MB = Q_S + 64, QB = Q_MB + 16 * kAttWarps;
+  static constexpr int Q_S = NQ * P * 8, Q_MB = Q_S + 64, Q_RED = Q_MB + 16 * kAttWarps, QB = Q_RED + 8 * kAttWarps * NQ;
   static constexpr int W_KC = 0;              // float2 per token: (A, B) of K's norms
   static constexpr int W_VC = W_KC + kAttBatch * 8;
   static constexpr int W_KS = W_VC + kAttBatch * 8;   // float per token: 2^e of K's record
@@ -231,13 +231,6 @@ __device__ __forceinline__ void warp_fwht(float* row, int lane) {
   __syncwarp();
 }
 
-// The CTA that takes unit u when `units` units go to `ctas` CTAs in contiguous
-// ranges, the first units % ctas of them one longer.
-__host__ __device__ inline int att_cta_of(int u, int units, int ctas) {
-  const int per = units / ctas, extra = units % ctas, cut = extra * (per + 1);
-  return u < cut ? u / (per + 1) : extra + (u - cut) / per;
-}
-
 template <int D, int QT>
 __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     attend_partial(const __grid_constant__ AttParams p, float* ws) {
@@ -293,7 +286,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     uint8_t* const st_vh = st_vn + kAttBatch * nbv;
     int64_t row0 = (int64_t)(u - J.unit0) * kAttUnit + warp * kAttBatch;
     const int64_t seg_rows = min(J.tokens, (int64_t)(u_stop - J.unit0) * kAttUnit);   // the segment's end
-    const int seg = cta - att_cta_of(J.unit0, p.nunits, p.nctas);
+    int unit = u - J.unit0;                        // within the job
     u = u_stop;
 
     // ---- staging: lane s of 6 copies the 32 rows of segment s (K angle | norm |
@@ -469,18 +462,12 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     const int q0 = QT == 1 ? 2 * (t & 1) : 2 * t;
     const float qsc[2] = {qscale[q0], qscale[q0 + 1]};
 
-    // Running softmax state of the lane's two queries (the same on every lane
-    // that owns them): m a whole number not more than 8 below the largest score
+    // Softmax state of the lane's two queries (the same on every lane that owns
+    // them) in a unit: m a whole number not more than 8 below the largest score
     // (log2 units), l the lane's part of the sum of 2^(s - m); accumulators in
     // units of 2^m / c, c a power of two (infinite while they are empty).
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, c_run[2] = {INFINITY, INFINITY};
+    float m_run[2], l_run[2], c_run[2];
     float acc[QT][VP][4];
-#pragma unroll
-    for (int x = 0; x < QT; ++x)
-#pragma unroll
-      for (int j = 0; j < VP; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[x][j][i] = 0.f;
 
     // fp32 norms: no header; the largest norm of each token of the batch sets its scale.
     auto fp32_consts = [&](const uint8_t* norms, int row_bytes, float2* ab, float* scale) {
@@ -727,7 +714,20 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       }
     };
 
-    for (; row0 < seg_rows; row0 += kAttUnit) {
+    for (; ; ++unit, row0 += kAttUnit) {             // a unit: one batch for each warp
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      m_run[q] = -INFINITY;
+      l_run[q] = 0.f;
+      c_run[q] = INFINITY;
+    }
+#pragma unroll
+    for (int x = 0; x < QT; ++x)
+#pragma unroll
+      for (int j = 0; j < VP; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[x][j][i] = 0.f;
+    if (row0 < seg_rows) {
       const int valid = (int)min((int64_t)kAttBatch, J.tokens - row0);
       landed(row0, bar_k, phase_k);                // this batch's K rows
       if (hkb) norm_consts(reinterpret_cast<const float2*>(st_kh)[lane], kinv, klog, kc[lane], ksc[lane]);
@@ -749,9 +749,6 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
         sv[i] = tok < valid ? sv[i] * qsc[i & 1] * ksc[tok] : -INFINITY;
         over |= !(sv[i] <= m_run[i & 1] + 8.f);
       }
-      __syncwarp();                                // every lane is done with the K rows
-      issue(false, row0 + kAttUnit, bar_k, bytes_k);
-
       // ---- softmax (base 2): the reference m moves only when a score passes it by more than 8 ----
       if (__any_sync(0xffffffffu, over)) {
 #pragma unroll
@@ -823,17 +820,16 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
         case 3: values(IC<3>{}); break;
         default: values(IC<4>{}); break;
       }
-      __syncwarp();                                // every lane is done with the V rows and the weights
-      issue(true, row0 + kAttUnit, bar_v, bytes_v);
     }
 
-    // ---- merge the warps: the segment's (max, sum, accumulator) per query ----
+    // ---- merge the warps: the unit's (max, sum, accumulator) per query, in an
+    // order of its own: a job's record depends on nothing but its rows and queries ----
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
       for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) l_run[q] += __shfl_xor_sync(0xffffffffu, l_run[q], o);
     __syncthreads();                               // every warp is done with its memory and the queries
-    float* const red = reinterpret_cast<float*>(smem);        // [warp][NQ][2]: m, l
+    float* const red = reinterpret_cast<float*>(smem + C::Q_RED);   // [warp][NQ][2]: m, l
     if (g == 0 && (QT == 2 || t < 2)) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -874,7 +870,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       }
     }
     __syncthreads();
-    float* const rec = ws + J.ws + (int64_t)seg * nq * att_rec_floats(D);
+    float* const rec = ws + J.ws + (int64_t)unit * nq * att_rec_floats(D);
     for (int e = tid; e < nq * D; e += kAttThreads) {
       const int a = e / D, j = e % D;
       float s = 0.f;
@@ -894,10 +890,16 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       rec[tid * att_rec_floats(D)] = M;
       rec[tid * att_rec_floats(D) + 1] = l;
     }
+    fence_async_proxy();
+    __syncthreads();                               // the merge is done with the warps' memory and the queries
+    if (unit + 1 == u_stop - J.unit0) break;
+    issue(false, row0 + kAttUnit, bar_k, bytes_k);
+    issue(true, row0 + kAttUnit, bar_v, bytes_v);
+    }
   }
 }
 
-// One CTA of 4 warps per (job, query): warp w merges segments w, w + 4, ...
+// One CTA of 4 warps per (job, query): warp w merges units w, w + 4, ...
 // against the row's overall max, the warps' sums are added in shared memory,
 // and warp 0 normalizes, applies D H (fp32 butterfly) and stores the row.
 template <int D, typename TO>
@@ -910,10 +912,9 @@ __global__ void __launch_bounds__(128) attend_combine(const __grid_constant__ At
   const AttJob& J = p.job[blockIdx.y];
   const int a = blockIdx.x;
   if (a >= J.nq) return;
-  const int last = J.unit0 + (int)((J.tokens + kAttUnit - 1) / kAttUnit) - 1;
-  const int nsp = att_cta_of(last, p.nunits, p.nctas) - att_cta_of(J.unit0, p.nunits, p.nctas) + 1;
+  const int nsp = (int)((J.tokens + kAttUnit - 1) / kAttUnit);
   const float* recs = ws + J.ws + (int64_t)a * att_rec_floats(D);
-  const int64_t stride = (int64_t)J.nq * att_rec_floats(D);   // between segments
+  const int64_t stride = (int64_t)J.nq * att_rec_floats(D);   // between units
   // launched while the partial kernel runs: wait for its results
   asm volatile("griddepcontrol.wait;" ::: "memory");
   float M = -INFINITY;

@@ -37,9 +37,8 @@ struct AttParams {
   AttJob job[TAC_ATTEND_MAX_JOBS];   // 200 bytes each: within the 32 KB of kernel parameters
 };
 
-// Workspace record of one segment (a CTA's tokens of one job) and query: max
-// (log2 units), sum, accumulator (d floats).  A job has at most one segment per
-// TAC_ATTEND_SPLIT tokens.
+// Workspace record of one unit (TAC_ATTEND_SPLIT tokens of one job) and query:
+// max (log2 units), sum, accumulator (d floats).
 __host__ __device__ constexpr int att_rec_floats(int d) { return d + 2; }
 
 // Attention staging: a warp takes its tokens in batches of 32; a staged batch

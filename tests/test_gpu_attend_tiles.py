@@ -77,6 +77,37 @@ def test_value_scales_per_token(tac_gpu, orc, order):
     assert np.all(err <= 2.0**-18 * size), err / size
 
 
+def _job(torch, tac, d, T, nq, seed, dtype):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    kcfg, vcfg = tac.layer_cfg(d, 64, 8, 0, 0, 1, 0), tac.layer_cfg(d, 64, 4, 1, 0, 1, 1)
+    kc, vc = (tac.encode(torch.randn((T, d), generator=g, device="cuda"), c) for c in (kcfg, vcfg))
+    q = (2 * torch.randn((nq, d), generator=g, device="cuda")).to(dtype)
+    return tac.AttendJob(kcfg, kc, vcfg, vc, T, q, torch.zeros_like(q), 1.0 / math.sqrt(d))
+
+
+@pytest.mark.parametrize("d,nq", [(64, 4), (128, 1), (128, 8)])
+def test_outputs_do_not_depend_on_the_other_jobs(tac_gpu, d, nq):
+    """The same bits from a job alone and in batches whose units are dealt to the
+    CTAs in other ways (more units than CTAs, fewer, the job first or last)."""
+    import torch
+    tac = tac_gpu
+    jobs = [_job(torch, tac, d, T, nq, i, torch.float32) for i, T in enumerate([20000, 300, 4097, 33, 70000, 1000])]
+    alone = []
+    for j in jobs:
+        tac.attend_multi([j])
+        alone.append(j.out.clone())
+    fill = [_job(torch, tac, d, T, nq, 50 + i, torch.float32) for i, T in enumerate([511, 30000, 30000, 7, 90000])]
+    for batch in (jobs, jobs[::-1], fill[:1] + jobs[1:4], fill + jobs, jobs + fill, jobs[:2] + fill + jobs[2:]):
+        for j in jobs:
+            j.out.zero_()
+        tac.attend_multi(batch)
+        torch.cuda.synchronize()
+        for j, want in zip(jobs, alone):
+            if any(j is b for b in batch):
+                assert torch.equal(j.out, want), (j.tokens, len(batch))
+
+
 def test_attend_captured_into_graph(tac_gpu):
     """A prepared call (both kernels, the second launched while the first runs)
     replays from a CUDA graph to the bits of the direct call, over new queries."""

@@ -298,7 +298,8 @@ int64_t tac_attend_workspace_bytes(const tac_attend_job* jobs, int njobs);
  * TAC_ATTEND_MAX_JOBS jobs each; the second kernel is launched while the first
  * runs and waits for it on the device); several launch pairs run concurrently on
  * `stream` and the helper streams of tac_encode_multi (fork / join by events),
- * ordered on `stream` as a whole.
+ * ordered on `stream` as a whole.  A job's outputs are the same bits whatever
+ * the other jobs of the call are.
  * `workspace` (device, 16-byte aligned, >= tac_attend_workspace_bytes) is the
  * caller's; its contents need no initialisation and are overwritten.  Calls
  * that share a workspace must not overlap in time. */

@@ -14,42 +14,36 @@
 //                   tokens of each (a batch).  Both contractions run on the
 //                   tensor cores (mma.sync m16n8k16, fp16 operands, fp32 sums):
 //                   the operands are decoded straight into the registers of the
-//                   fragments, so nothing decoded touches memory.  A decoded
-//                   value r^ (cos, sin), scaled by the power of two that brings
-//                   its record's largest norm into [1, 2), is split as
-//                   hi + lo: hi rounded to fp16 (keys) or to the grid of 2^-10
-//                   (values), lo the exact residue of the fp32 product rounded
-//                   to fp16 (2^-24 of the value, or 2^-23 of the record's
-//                   scale, at most).  The queries (and, for the values, the
-//                   softmax weights) are split hi + 2^-11 lo as well, both
-//                   rounded to fp16 (2^-24 of the value), the two parts in
-//                   different columns of the other operand: one mma for A_hi
-//                   and one for A_lo give all four products.  Sums over more
-//                   than a few mma steps are taken in fp32 registers.
-//   attend_combine  one CTA per (job, query): merges the CTAs' partial results
+//                   fragments, so nothing decoded touches memory.  Operands are
+//                   split into fp16 parts that together keep what fp32 would:
+//                   a decoded value r^ (cos, sin), in units of the power of two of
+//                   its record, into hi (a multiple of 2^-10), the residue of the
+//                   product rounded to fp16 and, in jobs of few tokens, what that
+//                   leaves; the queries and the softmax weights into a multiple of
+//                   2^-6 and two residues, exact.  The parts of a query or a weight
+//                   are columns of the other operand (two of them side by side, in
+//                   the same lane's accumulators).  hi times the first part sums
+//                   exactly on the tensor cores, whose sums are truncated to 24
+//                   bits (measured); the smaller products are added in fp32.
+//   attend_combine  one CTA per (job, query): merges the units' partial results
 //                   of the job, divides, applies D H (fp32 butterfly) and
 //                   stores the row.
-// Bound: instruction issue.  About 12 instructions decode and split one pair
-// (table offset 2, lookup 1, norm code 3, products and split 4 or 5, packing 2);
-// of some 98 warp-instructions a token-head 50 are these (d = 128, 4 queries),
-// and the schedulers issue in 67 % of the cycles at 16 warps per SM (128
-// registers).  A warp's batch of 32 tokens takes about 12 000 cycles: scores
-// 4800, values 5900, the rest softmax, constants and copies.  Copies are bulk
-// copies, one lane a segment: six cp.async loops over the segments took 2000
-// cycles a batch (12 us of the 162 below).  The set-up of a CTA's first job is
-// 12 000 cycles (20 000 with the queries rotated and split in shared memory, the
-// tables computed and written 16 copies by one thread, and a binary search for
-// the job).
-// With the products on the CUDA cores (114 instructions, 10 - 12 warps, and a
-// warp walking 256 tokens alone) 16 sequences of 1k to 32k tokens (8 KV heads,
-// 4 queries each, 244 MB of records) took 229 us, with tensor cores 162 and with
-// bulk copies and the keys' better split 158 us (1.5 TB/s); 8 heads of 4097
-// tokens 59 us, now 20 us (a CTA of 8 warps per 256 tokens fills the device; a
-// third of it are the launches); 128 heads of 8192 tokens at d = 64 143 us, now
-// 84 us.  Error of fp32 outputs against 64 bits over ten shapes (1 to 8 queries,
-// 37 to 20000 tokens, every norm storage): 3.3e-7 to 5.7e-7, 3.7e-7 to 7.0e-7
-// before.  Every unit is merged and written by itself, so a job's outputs do not
-// depend on the other jobs of the call or on how the units fall to the CTAs.
+// Bound: instruction issue: 95 warp-instructions a token-head (d = 128, 4
+// queries), 50 of them to decode and split its 128 pairs (table offset 2, lookup
+// 1, norm code 3, products and split 3, packing 2 for each), issued in 60 % of the
+// cycles at 16 warps per SM (128 registers); the barriers of the units' merges
+// cost 4 %.  Copies are bulk copies, one lane a segment (six cp.async loops took
+// 2000 cycles of a batch's 12 000).
+// 16 sequences of 1k to 32k tokens (8 KV heads, 4 queries each, 244 MB of records)
+// take 173 us (1.4 TB/s), 229 us with fp32 products on the CUDA cores (114
+// instructions, 10 - 12 warps, a warp walking 256 tokens alone); 8 heads of 4097
+// tokens 16.6 and 59 us; 128 heads of 8192 tokens at d = 64 97 and 145 us.  The
+// error of fp32 outputs against 64 bits is 0.55 to 1.0 times that of the fp32
+// products over 70 shapes (1 to 8 queries, 1 to 20000 tokens, every norm storage),
+// 0.77 times on average.  Two fp16 parts of everything and sums over a CTA's units
+// took 158, 20.5 and 84 us and had 0.74 to 2.5 times that error.
+// Every unit is merged and written by itself, in a fixed order, so a job's outputs
+// do not depend on the other jobs of the call or on how the units fall to the CTAs.
 // Codebooks (n, norm bits, norm mode) are runtime parameters: K and V may
 // differ, and any codebook the encoder supports is accepted.
 #include <algorithm>
@@ -67,34 +61,44 @@ struct IC { static constexpr int value = V; };
 constexpr int kAttWarps = 8;                  // warps per CTA
 constexpr int kAttThreads = 32 * kAttWarps;
 constexpr int kAttUnit = TAC_ATTEND_SPLIT;    // tokens of a unit: one batch for each warp
+// Jobs of at most this many tokens split the decoded values in three parts.  With
+// two a value keeps 2^-23 of its record's scale, which shows where few tokens share
+// the softmax: 1.0 to 1.13 times the error of fp32 products up to 40 tokens (fp32
+// norms), 0.56 to 0.99 times with three.  The third part costs 4 instructions a
+// pair; with more tokens two parts stay below 0.93 times.
+constexpr int kAttThree = kAttUnit;
 constexpr float kLog2e = 1.4426950408889634f;
 static_assert(kAttUnit == kAttWarps * kAttBatch, "a unit is one batch per warp");
 
-// QT = 1: up to 4 queries, the 8 columns of an mma are 4 hi and 4 lo parts;
-// QT = 2: up to 8 queries, one column tile of hi and one of lo parts.
+// QT column tiles of four queries each (up to 4 QT queries).
 template <int D, int QT>
 struct Att {
   static constexpr int P = D / 2, NQ = 4 * QT;
-  static constexpr int KP = P / 4;            // K: pairs of a token a lane decodes (4 lanes a token)
+  static constexpr int KP = P / 4, KS = KP / 2;   // K: pairs of a token a lane decodes (4 lanes a token), mma steps
   static constexpr int VP = P / 8;            // V: pairs of a token a lane decodes (8 lanes a token)
-  // Shared memory: rotated queries (the words of their fragments, hi and lo
-  // parts), their scales, the warps' barriers | K table | V table | per warp:
-  // batch constants, weights, staged batch.  The merge of the warps' results
-  // reuses the queries' and the warps' parts.
-  static constexpr int Q_S = NQ * P * 8, Q_MB = Q_S + 64, Q_RED = Q_MB + 16 * kAttWarps, QB = Q_RED + 8 * kAttWarps * NQ;
+  // Shared memory: rotated queries as the fragments their mma steps load, their
+  // scales, the warps' barriers, the warps' (max, sum, 1/unit) of a unit | K table
+  // | V table | per warp: batch constants, weights, staged batch.  A warp's sums
+  // of a unit are merged from the place of its staged V rows.
+  static constexpr int Q_S = KS / 2 * QT * 2 * 512, Q_MB = Q_S + 32, Q_RED = Q_MB + 16 * kAttWarps;
+  static constexpr int QB = Q_RED + 3 * kAttWarps * NQ * 4;
   static constexpr int W_KC = 0;              // float2 per token: (A, B) of K's norms
   static constexpr int W_VC = W_KC + kAttBatch * 8;
   static constexpr int W_KS = W_VC + kAttBatch * 8;   // float per token: 2^e of K's record
   static constexpr int W_VS = W_KS + kAttBatch * 4;
-  static constexpr int W_W = W_VS + kAttBatch * 4;    // weights: [2][columns][16 tokens] halves
-  static constexpr int W_STG = W_W + 2 * 8 * QT * 32;
-  static constexpr int MERGE = kAttWarps * NQ * D * 4;
-  static int smem(int stage, int tables) { return QB + tables + std::max(kAttWarps * (W_STG + stage), MERGE); }
+  static constexpr int W_W = W_VS + kAttBatch * 4;    // weights: [2][QT][8 + 4 columns][16 tokens] halves
+  static constexpr int W_STG = W_W + 2 * QT * 12 * 32;
+  static constexpr int MERGE = NQ * D * 4;            // a warp's sums
+  static int smem(int stage, int tables) { return QB + tables + kAttWarps * (W_STG + stage); }
   static_assert(QB % 16 == 0 && W_STG % 16 == 0, "alignment");
 };
 
-// Bin centres (cos, sin)(2 pi k / n) of every supported n, rounded from fp64
-// by the host compiler.
+// Decoded values are scaled by 2^kYExp of their record's power of two, which
+// keeps their residues normal fp16 numbers.
+constexpr int kYExp = 14;
+
+// Bin centres (cos, sin)(2 pi k / n) of every supported n times 2^kYExp, rounded
+// from fp64 by the host compiler.
 namespace cx {
 struct CentreTable { float2 v[kTabEntries]; };
 constexpr CentreTable make_centre_table() {
@@ -102,12 +106,20 @@ constexpr CentreTable make_centre_table() {
   for (int idx = 0; idx < kTabEntries; ++idx) {
     const int n = tab_n_of(idx), k = idx - tab_offset_n(n);
     const CS cs = cos_sin_q8(8 * k, n);
-    t.v[idx] = float2{(float)cs.c, (float)cs.s};
+    t.v[idx] = float2{(float)cs.c * (1 << kYExp), (float)cs.s * (1 << kYExp)};
   }
   return t;
 }
 }  // namespace cx
 __device__ const cx::CentreTable g_centre = cx::make_centre_table();
+
+// A shared-memory 16-byte load the compiler may not hoist or merge: keeps a
+// loop-invariant operand in shared memory instead of in registers.
+__device__ __forceinline__ uint4 lds_reload(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+  return v;
+}
 
 __device__ __forceinline__ uint32_t rotr(uint32_t x, int s) { return __funnelshift_r(x, x, s); }
 
@@ -134,40 +146,31 @@ __device__ __forceinline__ float exp2_whole(float x) { return x < -126.f ? 0.f :
 // The exponent of a nonnegative fp32 number (-127 for zero and subnormals).
 __device__ __forceinline__ int exp_of(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFFu) - 127; }
 
-// The split of (r, r) * cs, |r cs| < 2: nh = -(hi of both), lo the residue.
+// The split of (r, r) * cs, |r cs| < 2^(1 + kYExp): nh = -(hi of both), hi a
+// multiple of 2^(kYExp - 10), lo the residue.
 __device__ __forceinline__ void split_pair(float r, float2 cs, float2& nh, float2& lo) {
-  constexpr float M = 12288.f;                // 1.5 * 2^13: sums round to multiples of 2^-10
+  constexpr float M = 12288.f * (1 << kYExp);  // 1.5 * 2^(13 + kYExp)
   const float2 rr = make_float2(r, r);
   const float2 q = __ffma2_rn(rr, cs, make_float2(M, M));
   nh = __ffma2_rn(q, make_float2(-1.f, -1.f), make_float2(M, M));
   lo = __ffma2_rn(rr, cs, nh);
 }
 
-// The same with hi rounded to fp16 itself: nh = -(hi of both) in fp16, lo the
-// residue.  One instruction more, for the keys: lo is 2^-12 of the value instead
-// of 2^-11 of the record's scale, and the scores' error decides the output's
-// (5.1e-7 against 6.0e-7 for 4097 tokens at d = 128; 5.4e-7 on the CUDA cores).
-__device__ __forceinline__ void split_pair_fp(float r, float2 cs, uint32_t& nh, float2& lo) {
-  const float2 rr = make_float2(r, r);
-  const float2 y = mul2(rr, cs);
-  const __half2 hh = __floats2half2_rn(-y.x, -y.y);
-  nh = h2_bits(hh);
-  lo = __ffma2_rn(rr, cs, __half22float2(hh));
-}
-
-// x = hi + 2^-11 lo in fp16 (|x| below about 2^15).
-__device__ __forceinline__ void split_half(float x, __half& hi, __half& lo) {
-  hi = __float2half_rn(x);
-  lo = __float2half_rn((x - __half2float(hi)) * 2048.f);
+// x = a + b + c, three fp16 numbers, to 2^-33 of 2^13 <= |x| < 2^15 at worst.
+__device__ __forceinline__ void split_three(float x, float first, __half& a, __half& b, __half& c) {
+  a = __float2half_rn(first);
+  const float r = x - __half2float(a);
+  b = __float2half_rn(r);
+  c = __float2half_rn(r - __half2float(b));
 }
 
 // Batch constants of one token from its header: r^ 2^-e = A c + B for the norm
 // code c (log mode: its log2), e the exponent of the larger of the two norms.
 __device__ __forceinline__ void norm_consts(float2 h, float inv_l, bool lg, float2& ab, float& scale) {
   const bool spread = h.y > h.x;
-  const int e = min(max(exp_of(spread ? h.y : h.x), -126), 126);
+  const int e = min(max(exp_of(spread ? h.y : h.x), kYExp - 126), 126);
   const float sc = exp2i(-e);
-  scale = exp2i(e);
+  scale = exp2i(e - kYExp);
   if (lg) {
     const float lo = lg2_approx(h.x);
     ab = make_float2(spread ? (lg2_approx(h.y) - lo) * inv_l : 0.f, lo - (float)e);
@@ -235,14 +238,15 @@ template <int D, int QT>
 __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     attend_partial(const __grid_constant__ AttParams p, float* ws) {
   using C = Att<D, QT>;
-  constexpr int P = C::P, NQ = C::NQ, KP = C::KP, KS = KP / 2, VP = C::VP;
-  constexpr int NV = 4 * QT;                       // scores a lane owns in the softmax
+  constexpr int P = C::P, NQ = C::NQ, KP = C::KP, KS = C::KS, VP = C::VP;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler too
   const int g = lane >> 2, t = lane & 3;           // the fragments' row group and column pair
-  uint32_t* const qfrag = reinterpret_cast<uint32_t*>(smem);                 // [hi, lo][NQ][P]
+  uint32_t* const qfrag = reinterpret_cast<uint32_t*>(smem);                 // [KS / 2][QT][2][lane] uint4
   float* const qscale = reinterpret_cast<float*>(smem + C::Q_S);             // 2^e of each query
+  float2* const red = reinterpret_cast<float2*>(smem + C::Q_RED);            // [warp][query]: max, 1/unit of a unit's sums
+  float* const redl = reinterpret_cast<float*>(red + kAttWarps * NQ);        // and the sum
   float2* const tk = reinterpret_cast<float2*>(smem + C::QB);
   uint8_t* const wbase = smem + C::QB + p.tab_k + p.tab_v;
   float2* const tv = reinterpret_cast<float2*>(smem + C::QB + p.tab_k);
@@ -330,7 +334,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       __syncwarp();
     };
     fence_async_proxy();
-    __syncthreads();                               // the previous segment's merge is done with the warps' memory
+    __syncthreads();                               // the previous segment is done with the queries and the tables
     issue(false, row0, bar_k, bytes_k);
     issue(true, row0, bar_v, bytes_v);
 
@@ -348,11 +352,13 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       tab_nv = J.nv;
     }
     // ---- rotated queries q' = H D_K q * scale * log2(e), one warp a query,
-    // scaled by 2^-e into [-2, 2) and split; the word of slot i (the halves of its
-    // pair) lands where the fragments' order wants it: the run of KP slots of
-    // lane t, step by step.  Step ks takes two slots of every lane's run:
-    // neighbours, or (4-bit norms, whose codes are unpacked four apart) slots
-    // four apart ----
+    // scaled by 2^-e into [-2^14, 2^14) and split in three: a multiple of 2^8 (six
+    // bits), then two fp16 residues.  Columns 2 a and 2 a + 1 of a fragment are the
+    // first two parts of query a; the third (negated) is column 2 a of a fragment
+    // of its own.  The word of a slot (the halves of its pair) lands where its mma
+    // step loads it: the run of KP slots of lane t, step by step.  Step ks takes
+    // two slots of every lane's run: neighbours, or (4-bit norms, whose codes are
+    // unpacked four apart) slots four apart ----
     const bool k4 = J.ck <= 1;
     if (warp < NQ) {
       float y[D / 32];                             // elements lane + 32 k
@@ -390,19 +396,23 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       }
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const int e = min(max(exp_of(mx), -126), 126);
+      const int e = min(max(exp_of(mx) - 13, -126), 126);
       const float sc = exp2i(-e);
 #pragma unroll
       for (int k = 0; k < D / 32; ++k) {
         const float a = y[k] * sc, b = __shfl_down_sync(0xffffffffu, a, 1);
         if (!(lane & 1)) {                         // pair 16 k + lane / 2
-          __half ah, al, bh, bl;
-          split_half(a, ah, al);
-          split_half(b, bh, bl);
+          constexpr float M = 3221225472.f;        // 1.5 * 2^31: sums round to multiples of 2^8
+          __half a1, a2, a3, b1, b2, b3;
+          split_three(a, __fsub_rn(__fadd_rn(a, M), M), a1, a2, a3);
+          split_three(b, __fsub_rn(__fadd_rn(b, M), M), b1, b2, b3);
           const int i = pair_slot<D>(16 * k + lane / 2), r = i % KP;
-          const int at = warp * P + i - r + (k4 ? (r & ~7) + 2 * (r & 3) + ((r >> 2) & 1) : r);
-          qfrag[at] = h2_bits(__halves2half2(ah, bh));
-          qfrag[NQ * P + at] = h2_bits(__halves2half2(al, bl));
+          const int at = k4 ? (r & ~7) + 2 * (r & 3) + ((r >> 2) & 1) : r;
+          uint32_t* const w = qfrag + (((at >> 2) * QT + (warp >> 2)) * 64 + 8 * (warp & 3) + i / KP) * 4 + (at & 3);
+          w[0] = h2_bits(__halves2half2(a1, b1));
+          w[16] = h2_bits(__halves2half2(a2, b2));
+          w[128] = h2_bits(__halves2half2(__hneg(a3), __hneg(b3)));
+          w[144] = 0u;
         }
       }
       if (lane == 0) qscale[warp] = exp2i(e);
@@ -443,31 +453,13 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       voff[q] = (bit >> 5) * 4;
       vsh[q] = bit & 31;
     }
+    const uint32_t qlane = smem_addr(qfrag) + 16 * lane;
     const float kinv = J.inv_lk, vinv = J.inv_lv;
     const bool klog = J.mk == TAC_NORM_LOG, vlog = J.mv == TAC_NORM_LOG;
-    uint32_t bq[KS][QT][2];
+    // The lane's queries: 4 x + t.
+    float qsc[QT];
 #pragma unroll
-    for (int x = 0; x < QT; ++x) {
-      const int part = QT == 1 ? g >> 2 : x, a = QT == 1 ? g & 3 : g;
-      const uint4* src = reinterpret_cast<const uint4*>(qfrag + (part * NQ + a) * P + KP * t);
-#pragma unroll
-      for (int ks = 0; ks < KS; ks += 2) {
-        const uint4 v = src[ks / 2];
-        bq[ks][x][0] = v.x; bq[ks][x][1] = v.y;
-        bq[ks + 1][x][0] = v.z; bq[ks + 1][x][1] = v.w;
-      }
-    }
-    // The lane's queries in the softmax: two neighbours, the same as its columns
-    // of the value accumulators.
-    const int q0 = QT == 1 ? 2 * (t & 1) : 2 * t;
-    const float qsc[2] = {qscale[q0], qscale[q0 + 1]};
-
-    // Softmax state of the lane's two queries (the same on every lane that owns
-    // them) in a unit: m a whole number not more than 8 below the largest score
-    // (log2 units), l the lane's part of the sum of 2^(s - m); accumulators in
-    // units of 2^m / c, c a power of two (infinite while they are empty).
-    float m_run[2], l_run[2], c_run[2];
-    float acc[QT][VP][4];
+    for (int x = 0; x < QT; ++x) qsc[x] = qscale[4 * x + t];
 
     // fp32 norms: no header; the largest norm of each token of the batch sets its scale.
     auto fp32_consts = [&](const uint8_t* norms, int row_bytes, float2* ab, float* scale) {
@@ -478,29 +470,32 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
 #pragma unroll
         for (int k = 0; k < VP; k += 4) {
           const float4 v = *reinterpret_cast<const float4*>(nr + k);
-          mx = fmaxf(fmaxf(fmaxf(mx, v.x), fmaxf(v.y, v.z)), v.w);
+          mx = fmaxf(fmaxf(fmaxf(mx, fabsf(v.x)), fmaxf(fabsf(v.y), fabsf(v.z))), fabsf(v.w));
         }
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const int e = min(max(exp_of(mx), -126), 126);
+        const int e = min(max(exp_of(mx), kYExp - 126), 126);
         if ((lane & 7) == 0) {
           ab[tok] = make_float2(exp2i(-e), 0.f);
-          scale[tok] = exp2i(e);
+          scale[tok] = exp2i(e - kYExp);
         }
       }
     };
 
     // Scores of the staged batch.  Rows of the fragments are tokens, columns the
-    // queries (QT = 1: their hi and lo parts), the steps run over the slots.
-    // sv: QT = 1 tokens 16 (t / 2) + 8 (i / 2) + g, query q0 + (i & 1);
-    //     QT = 2 tokens 16 (i / 4) + 8 (i / 2 & 1) + g, query q0 + (i & 1).
-    auto scores = [&](float (&sv)[4 * QT], auto kc_) {
+    // parts of the queries, the steps run over the slots.  hi is a multiple of 2^-10
+    // below 2 and the queries' first part of 2^8 up to 2^14, so that their products
+    // and all sums of them are whole multiples of 2^-2 below 2^22 (64 pairs, each
+    // at most 2 sqrt(2) 2^14): exact, although the tensor cores' sums are truncated
+    // to 24 bits.  The other parts are 2^-7 of it or less and are added last, in fp32.
+    // sv[x]: tokens 16 (i / 2) + 8 (i & 1) + g, query 4 x + t.
+    auto scores = [&](float (&sv)[QT][4], auto kc_, auto three_) {
       constexpr int KC = decltype(kc_)::value;
+      constexpr bool THREE = decltype(three_)::value != 0;
       constexpr bool F32 = KC == 4, LOG = KC == 1 || KC == 3;
       constexpr int KB = KC <= 1 ? 4 : 8, KW = F32 ? 1 : KP * KB / 32;
-      float s0[4], s1[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) s0[i] = s1[i] = 0.f;
+      for (int x2 = 0; x2 < QT; ++x2) sv[x2][2] = sv[x2][3] = 0.f;
 #pragma unroll 1
       for (int mt = 0; mt < 2; ++mt) {
         uint32_t x[2][KP / 4], nw[2][KW];
@@ -529,12 +524,21 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
             nw[rr][0] = *reinterpret_cast<const uint32_t*>(nr + 4 * t);
           }
         }
-        float ch[2][4], cl[4], cx[4];
+        float ch[QT][2][4], cl[QT][4];             // hi times parts 1 | 2 (two chains), the rest
 #pragma unroll
-        for (int i = 0; i < 4; ++i) ch[0][i] = ch[1][i] = cl[i] = cx[i] = 0.f;
+        for (int x2 = 0; x2 < QT; ++x2)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) ch[x2][0][i] = ch[x2][1][i] = cl[x2][i] = 0.f;
+        uint4 bq[QT][2];
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
-          uint32_t ah[4], al[4];
+          if ((ks & 1) == 0) {
+#pragma unroll
+            for (int x2 = 0; x2 < QT; ++x2)
+#pragma unroll
+              for (int f = 0; f < 2; ++f) bq[x2][f] = lds_reload(qlane + ((ks / 2 * QT + x2) * 2 + f) * 512);
+          }
+          uint32_t ah[4], al[4], al2[4];
 #pragma unroll
           for (int rr = 0; rr < 2; ++rr) {
             float rv[2];
@@ -549,59 +553,52 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
               const float2 cc = __half22float2(__hsub2(h2_of(hb), h2_of(0x64006400u)));
               rv[0] = __fmaf_rn(cc.x, ab[rr].x, ab[rr].y);
               rv[1] = __fmaf_rn(cc.y, ab[rr].x, ab[rr].y);
-              if constexpr (LOG) { rv[0] = ex2_approx(rv[0]); rv[1] = ex2_approx(rv[1]); }
+              if constexpr (LOG) { rv[0] = ex2_ftz(rv[0]); rv[1] = ex2_ftz(rv[1]); }
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const int i = (KB == 4 && !F32) ? 8 * (ks >> 2) + (ks & 3) + 4 * h : 2 * ks + h;
               const uint32_t o = (rotr(x[rr][i >> 2], kra[i & 3]) & kM) | kC;
-              float2 lo;
-              split_pair_fp(rv[h], *reinterpret_cast<const float2*>(tkb + o), ah[2 * h + rr], lo);
-              al[2 * h + rr] = h2_bits(__floats2half2_rn(lo.x, lo.y));
+              float2 nh, lo;
+              split_pair(rv[h], *reinterpret_cast<const float2*>(tkb + o), nh, lo);
+              ah[2 * h + rr] = h2_bits(__floats2half2_rn(nh.x, nh.y));
+              const __half2 hl = __floats2half2_rn(lo.x, lo.y);
+              al[2 * h + rr] = h2_bits(hl);
+              if constexpr (THREE) {
+                const float2 fl = __half22float2(hl);
+                al2[2 * h + rr] = h2_bits(__floats2half2_rn(lo.x - fl.x, lo.y - fl.y));
+              }
             }
           }
-          if constexpr (F32) {                     // every step's sum added in fp32
-            float c[4];
-            mma_f16_zero(c, ah, bq[ks][0][0], bq[ks][0][1]);
-            float2* a2 = reinterpret_cast<float2*>(ch[ks & 1]);
-            a2[0] = add2(a2[0], make_float2(c[0], c[1]));
-            a2[1] = add2(a2[1], make_float2(c[2], c[3]));
-          } else {
-            mma_f16(ch[ks & 1], ah, bq[ks][0][0], bq[ks][0][1]);
-          }
-          mma_f16(cl, al, bq[ks][0][0], bq[ks][0][1]);
-          if constexpr (QT == 2) mma_f16(cx, ah, bq[ks][QT - 1][0], bq[ks][QT - 1][1]);
-        }
-        if constexpr (QT == 1) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) { s0[i] = s1[i]; s1[i] = cl[i] - (ch[0][i] + ch[1][i]); }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            s0[i] = s1[i];
-            s1[i] = __fmaf_rn(cx[i], -0.00048828125f, cl[i] - (ch[0][i] + ch[1][i]));
+          for (int x2 = 0; x2 < QT; ++x2) {
+            const uint4 q12 = bq[x2][0], q3 = bq[x2][1];
+            const uint32_t b0 = ks & 1 ? q12.z : q12.x, b1 = ks & 1 ? q12.w : q12.y;
+            mma_f16(ch[x2][ks & 1], ah, b0, b1);
+            mma_f16(cl[x2], al, b0, b1);
+            if constexpr (THREE) mma_f16(cl[x2], al2, b0, b1);
+            mma_f16(cl[x2], ah, ks & 1 ? q3.z : q3.x, ks & 1 ? q3.w : q3.y);
           }
         }
-      }
-      if constexpr (QT == 1) {
-        // lanes t < 2 hold the hi parts of their queries, t >= 2 the lo parts of the same ones
-        const bool up = t >= 2;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float kept = up ? s1[i] : s0[i];
-          const float got = __shfl_xor_sync(0xffffffffu, up ? s0[i] : s1[i], 2);
-          sv[i] = __fmaf_rn(up ? kept : got, 0.00048828125f, up ? got : kept);
-        }
-      } else {
+        for (int x2 = 0; x2 < QT; ++x2)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { sv[i] = s0[i]; sv[4 * (QT - 1) + i] = s1[i]; }
+          for (int i = 0; i < 2; ++i) {
+            sv[x2][i] = sv[x2][2 + i];
+            const float rest = (cl[x2][2 * i] + cl[x2][2 * i + 1]) - (ch[x2][0][2 * i + 1] + ch[x2][1][2 * i + 1]);
+            sv[x2][2 + i] = rest - (ch[x2][0][2 * i] + ch[x2][1][2 * i]);
+          }
       }
     };
 
     // Values: acc += sum_t w_t y^V_t.  Rows of the fragments are the (cos, sin) of
-    // slot VP g + j, columns the queries' weights, the steps run over the tokens.
-    auto values = [&](auto vc_) {
+    // slot VP g + j, columns the parts of the queries' weights (as the queries'
+    // parts above), the steps run over the tokens.  THREE: a value's residue is
+    // split once more (see kAttThree).
+    float acc[QT][VP][4];
+    auto values = [&](auto vc_, auto three_) {
       constexpr int VC = decltype(vc_)::value;
+      constexpr bool THREE = decltype(three_)::value != 0;
       constexpr bool F32 = VC == 4, LOG = VC == 1 || VC == 3;
       constexpr int VB = VC <= 1 ? 4 : 8;
       constexpr bool N16 = VB == 4 && VP == 4 && !F32;   // a lane's norms of a token in 16 bits
@@ -637,12 +634,15 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
           nw[0][0] |= nw[1][0] << 16;
           nw[2][0] |= nw[3][0] << 16;
         }
-        uint32_t b[QT][2], nb[QT][2];
+        uint32_t b[QT][2], nb[QT][2], nb3[QT][2];
 #pragma unroll
         for (int x2 = 0; x2 < QT; ++x2) {
-          const uint2 v = *reinterpret_cast<const uint2*>(pw + C::W_W + ((kk * QT + x2) * 8 + g) * 32 + 8 * t);
+          const uint8_t* wt = pw + C::W_W + (kk * QT + x2) * 384 + 8 * t;
+          const uint2 v = *reinterpret_cast<const uint2*>(wt + g * 32);
+          const uint2 v3 = *reinterpret_cast<const uint2*>(wt + 256 + (g >> 1) * 32);
           b[x2][0] = v.x; b[x2][1] = v.y;
           nb[x2][0] = v.x ^ 0x80008000u; nb[x2][1] = v.y ^ 0x80008000u;
+          nb3[x2][0] = g & 1 ? 0u : v3.x; nb3[x2][1] = g & 1 ? 0u : v3.y;
         }
 #pragma unroll
         for (int jj = 0; jj < VP / 2; ++jj) {      // two slots at a time
@@ -678,12 +678,12 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
           }
           if constexpr (LOG) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) { rv[i][0] = ex2_approx(rv[i][0]); rv[i][1] = ex2_approx(rv[i][1]); }
+            for (int i = 0; i < 4; ++i) { rv[i][0] = ex2_ftz(rv[i][0]); rv[i][1] = ex2_ftz(rv[i][1]); }
           }
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const int j = js[h];
-            uint32_t ah[4], al[4];
+            uint32_t ah[4], al[4], al2[4];
 #pragma unroll
             for (int i = 0; i < 4; i += 2) {
               float2 n0, l0, n1, l1;
@@ -693,17 +693,30 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
               split_pair(rv[i + 1][h], *reinterpret_cast<const float2*>(tvb + o1), n1, l1);
               ah[i] = h2_bits(__floats2half2_rn(n0.x, n1.x));
               ah[i + 1] = h2_bits(__floats2half2_rn(n0.y, n1.y));
-              al[i] = h2_bits(__floats2half2_rn(l0.x, l1.x));
-              al[i + 1] = h2_bits(__floats2half2_rn(l0.y, l1.y));
+              const __half2 lx = __floats2half2_rn(l0.x, l1.x), ly = __floats2half2_rn(l0.y, l1.y);
+              al[i] = h2_bits(lx);
+              al[i + 1] = h2_bits(ly);
+              if constexpr (THREE) {
+                const float2 fx = __half22float2(lx), fy = __half22float2(ly);
+                al2[i] = h2_bits(__floats2half2_rn(l0.x - fx.x, l1.x - fx.y));
+                al2[i + 1] = h2_bits(__floats2half2_rn(l0.y - fy.x, l1.y - fy.y));
+              }
             }
 #pragma unroll
             for (int x2 = 0; x2 < QT; ++x2) {
               float c[4];
-              if (x2 == 0) {
-                mma_f16_zero(c, al, b[x2][0], b[x2][1]);
-                mma_f16(c, ah, nb[x2][0], nb[x2][1]);
+              mma_f16_zero(c, al, b[x2][0], b[x2][1]);
+              if constexpr (THREE) mma_f16(c, al2, b[x2][0], b[x2][1]);
+              mma_f16(c, ah, nb3[x2][0], nb3[x2][1]);
+              if constexpr (THREE) {               // hi times part 1 (exact) apart from the rest
+                float ch[4];
+                mma_f16_zero(ch, ah, nb[x2][0], nb[x2][1]);
+                c[1] = (c[1] + ch[1]) + c[0];
+                c[3] = (c[3] + ch[3]) + c[2];
+                c[0] = ch[0];
+                c[2] = ch[2];
               } else {
-                mma_f16_zero(c, ah, nb[x2][0], nb[x2][1]);
+                mma_f16(c, ah, nb[x2][0], nb[x2][1]);
               }
               float2* a2 = reinterpret_cast<float2*>(acc[x2][j]);
               a2[0] = add2(a2[0], make_float2(c[0], c[1]));
@@ -714,187 +727,158 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       }
     };
 
+    const bool three = J.tokens <= kAttThree;
     for (; ; ++unit, row0 += kAttUnit) {             // a unit: one batch for each warp
+      float m_[QT], l_[QT], iu[QT];                  // its max (whole), sum of 2^(s - m), and 1 / the sums' unit
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      m_run[q] = -INFINITY;
-      l_run[q] = 0.f;
-      c_run[q] = INFINITY;
-    }
+      for (int x = 0; x < QT; ++x) {
+        m_[x] = -INFINITY;
+        l_[x] = 0.f;
+        iu[x] = 1.f;
 #pragma unroll
-    for (int x = 0; x < QT; ++x)
+        for (int j = 0; j < VP; ++j)
 #pragma unroll
-      for (int j = 0; j < VP; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[x][j][i] = 0.f;
-    if (row0 < seg_rows) {
-      const int valid = (int)min((int64_t)kAttBatch, J.tokens - row0);
-      landed(row0, bar_k, phase_k);                // this batch's K rows
-      if (hkb) norm_consts(reinterpret_cast<const float2*>(st_kh)[lane], kinv, klog, kc[lane], ksc[lane]);
-      else fp32_consts(st_kn, nbk, kc, ksc);
-      __syncwarp();
-      float sv[NV];
-      switch (J.ck) {
-        case 0: scores(sv, IC<0>{}); break;
-        case 1: scores(sv, IC<1>{}); break;
-        case 2: scores(sv, IC<2>{}); break;
-        case 3: scores(sv, IC<3>{}); break;
-        default: scores(sv, IC<4>{}); break;
+          for (int i = 0; i < 4; ++i) acc[x][j][i] = 0.f;
       }
-      auto token = [&](int i) { return QT == 1 ? 16 * (t >> 1) + 8 * (i >> 1) + g : 16 * (i >> 2) + 8 * ((i >> 1) & 1) + g; };
-      bool over = false;
+      if (row0 < seg_rows) {
+        const int valid = (int)min((int64_t)kAttBatch, J.tokens - row0);
+        landed(row0, bar_k, phase_k);                // this batch's K rows
+        if (hkb) norm_consts(reinterpret_cast<const float2*>(st_kh)[lane], kinv, klog, kc[lane], ksc[lane]);
+        else fp32_consts(st_kn, nbk, kc, ksc);
+        __syncwarp();
+        float sv[QT][4];
+        switch (J.ck + (three ? 8 : 0)) {
+          case 0: scores(sv, IC<0>{}, IC<0>{}); break;
+          case 1: scores(sv, IC<1>{}, IC<0>{}); break;
+          case 2: scores(sv, IC<2>{}, IC<0>{}); break;
+          case 3: scores(sv, IC<3>{}, IC<0>{}); break;
+          case 4: scores(sv, IC<4>{}, IC<0>{}); break;
+          case 8: scores(sv, IC<0>{}, IC<1>{}); break;
+          case 9: scores(sv, IC<1>{}, IC<1>{}); break;
+          case 10: scores(sv, IC<2>{}, IC<1>{}); break;
+          case 11: scores(sv, IC<3>{}, IC<1>{}); break;
+          default: scores(sv, IC<4>{}, IC<1>{}); break;
+        }
+        auto token = [&](int i) { return 16 * (i >> 1) + 8 * (i & 1) + g; };
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        const int tok = token(i);
-        sv[i] = tok < valid ? sv[i] * qsc[i & 1] * ksc[tok] : -INFINITY;
-        over |= !(sv[i] <= m_run[i & 1] + 8.f);
+        for (int i = 0; i < 4; ++i) {
+          const int tok = token(i);
+          const float ks = ksc[tok];
+#pragma unroll
+          for (int x = 0; x < QT; ++x) sv[x][i] = tok < valid ? sv[x][i] * (qsc[x] * ks) : -INFINITY;
+        }
+        __syncwarp();                                // every lane is done with the K rows
+        issue(false, row0 + kAttUnit, bar_k, bytes_k);
+        landed(row0, bar_v, phase_v);                // this batch's V rows
+        if (hvb) norm_consts(reinterpret_cast<const float2*>(st_vh)[lane], vinv, vlog, vc[lane], vsc[lane]);
+        else fp32_consts(st_vn, nbv, vc, vsc);
+        __syncwarp();
+        // ---- softmax (base 2) of the batch against the whole number above its
+        // largest score; weights 2^(s - m) 2^e scaled by the power of two that
+        // brings the largest to [2^14, 2^15), in three fp16 parts ----
+#pragma unroll
+        for (int x = 0; x < QT; ++x) {
+          float mx = fmaxf(fmaxf(sv[x][0], sv[x][1]), fmaxf(sv[x][2], sv[x][3]));
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          m_[x] = J.tokens <= kAttBatch ? mx : ceilf(mx);
+          float w[4], wm = 0.f;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float pr = ex2_approx(sv[x][i] - m_[x]);
+            l_[x] += pr;
+            w[i] = pr * vsc[token(i)];
+            wm = fmaxf(wm, w[i]);
+          }
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
+          const int k = min(max(14 - exp_of(wm), -126), 126);
+          const float unit_ = exp2i(k);
+          iu[x] = exp2i(-k);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            __half w1, w2, w3;
+            const float ws_ = w[i] * unit_;
+            constexpr float M = 6442450944.f;      // 1.5 * 2^32: sums round to multiples of 2^9
+            split_three(ws_, __fsub_rn(__fadd_rn(ws_, M), M), w1, w2, w3);
+            const int tok = token(i);
+            __half* const wt = reinterpret_cast<__half*>(pw + C::W_W + ((tok >> 4) * QT + x) * 384) + (tok & 15);
+            wt[32 * t] = w1;
+            wt[32 * t + 16] = w2;
+            wt[128 + 16 * t] = __hneg(w3);
+          }
+        }
+        __syncwarp();
+        switch (J.cv + (three ? 8 : 0)) {
+          case 0: values(IC<0>{}, IC<0>{}); break;
+          case 1: values(IC<1>{}, IC<0>{}); break;
+          case 2: values(IC<2>{}, IC<0>{}); break;
+          case 3: values(IC<3>{}, IC<0>{}); break;
+          case 4: values(IC<4>{}, IC<0>{}); break;
+          case 8: values(IC<0>{}, IC<1>{}); break;
+          case 9: values(IC<1>{}, IC<1>{}); break;
+          case 10: values(IC<2>{}, IC<1>{}); break;
+          case 11: values(IC<3>{}, IC<1>{}); break;
+          default: values(IC<4>{}, IC<1>{}); break;
+        }
+#pragma unroll
+        for (int x = 0; x < QT; ++x)
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) l_[x] += __shfl_xor_sync(0xffffffffu, l_[x], o);
       }
-      // ---- softmax (base 2): the reference m moves only when a score passes it by more than 8 ----
-      if (__any_sync(0xffffffffu, over)) {
+      __syncwarp();                                  // every lane is done with the V rows and the weights
+      // ---- merge the warps' sums of the unit in a fixed order: its record depends on
+      // nothing but the job's own rows and queries ----
+      float2* const mrg = reinterpret_cast<float2*>(st_va);   // [x][j][lane], in the place of the V rows
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          float mx = -INFINITY;
+      for (int x = 0; x < QT; ++x)
 #pragma unroll
-          for (int i = q; i < NV; i += 2) mx = fmaxf(mx, sv[i]);
+        for (int j = 0; j < VP; ++j)
+          mrg[(x * VP + j) * 32 + lane] = make_float2(acc[x][j][0] + acc[x][j][1], acc[x][j][2] + acc[x][j][3]);
+      if (g == 0) {
 #pragma unroll
-          for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-          const float mn = fmaxf(m_run[q], ceilf(mx));
-          if (mn > m_run[q]) {
-            l_run[q] *= exp2_whole(m_run[q] - mn);
-            c_run[q] *= ex2_approx(mn - m_run[q]);   // whole (or infinite) argument: exact
-            m_run[q] = mn;
+        for (int x = 0; x < QT; ++x) {
+          const int at = warp * NQ + 4 * x + t;
+          red[at] = make_float2(m_[x], iu[x]);
+          redl[at] = dead ? __int_as_float(0x7FC00000) : l_[x];
+        }
+      }
+      __syncthreads();
+      float* const rec = ws + J.ws + (int64_t)unit * nq * att_rec_floats(D);
+      const uint8_t* const m0 = reinterpret_cast<const uint8_t*>(mrg) - (size_t)warp * (C::W_STG + p.stage);
+#pragma unroll
+      for (int e0 = 0; e0 < QT * VP * 32; e0 += kAttThreads) {
+        const int e = e0 + tid, x = e / (VP * 32), j = (e >> 5) % VP, a = 4 * x + t;
+        if (e < QT * VP * 32 && a < nq) {
+          float2 mw[kAttWarps];
+          float M = -INFINITY;
+#pragma unroll
+          for (int w = 0; w < kAttWarps; ++w) {
+            mw[w] = red[w * NQ + a];
+            M = fmaxf(M, mw[w].x);
+          }
+          float2 s2 = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int w = 0; w < kAttWarps; ++w) {
+            mw[w].x = ex2_ftz(mw[w].x - M);          // of a whole number (or -infinity): exact
+            const float f = mw[w].x * mw[w].y;
+            const float2 v = reinterpret_cast<const float2*>(m0 + (size_t)w * (C::W_STG + p.stage))[e];
+            s2 = __ffma2_rn(v, make_float2(f, f), s2);
+          }
+          float* const ra = rec + a * att_rec_floats(D);
+          *reinterpret_cast<float2*>(ra + 2 + 2 * slot_pair<D>(VP * g + j)) = s2;
+          if (j == 0 && g == 0) {
+            float l = 0.f;
+#pragma unroll
+            for (int w = 0; w < kAttWarps; ++w) l = __fmaf_rn(redl[w * NQ + a], mw[w].x, l);
+            *reinterpret_cast<float2*>(ra) = make_float2(M, l);
           }
         }
       }
-      landed(row0, bar_v, phase_v);                // this batch's V rows
-      if (hvb) norm_consts(reinterpret_cast<const float2*>(st_vh)[lane], vinv, vlog, vc[lane], vsc[lane]);
-      else fp32_consts(st_vn, nbv, vc, vsc);
-      __syncwarp();
-      // weights 2^(s - m) 2^e in the accumulators' units, which move only when a
-      // weight passes 2^8
-      float w[NV];
-      over = false;
-#pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        const float pr = ex2_approx(sv[i] - m_run[i & 1]);
-        l_run[i & 1] += pr;
-        w[i] = pr * vsc[token(i)];
-        over |= !(w[i] * c_run[i & 1] <= 256.f);
-      }
-      if (__any_sync(0xffffffffu, over)) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          float mx = 0.f;
-#pragma unroll
-          for (int i = q; i < NV; i += 2) mx = fmaxf(mx, w[i]);
-#pragma unroll
-          for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-          if (!(mx * c_run[q] <= 256.f)) {
-            const float cn = exp2i(-(exp_of(mx) + 1));
-            const float f = cn / c_run[q];           // 0 for empty accumulators
-            c_run[q] = cn;
-#pragma unroll
-            for (int x = 0; x < QT; ++x)
-#pragma unroll
-              for (int j = 0; j < VP; ++j) {
-                acc[x][j][q] *= f;
-                acc[x][j][2 + q] *= f;
-              }
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        __half hi, lo;
-        split_half(w[i] * c_run[i & 1], hi, lo);
-        const int tok = token(i), q = q0 + (i & 1);
-        __half* base = reinterpret_cast<__half*>(pw + C::W_W) + (tok >> 4) * QT * 128 + (tok & 15);
-        base[q * 16] = hi;
-        base[(QT == 1 ? q + 4 : q + 8) * 16] = lo;
-      }
-      __syncwarp();
-      switch (J.cv) {
-        case 0: values(IC<0>{}); break;
-        case 1: values(IC<1>{}); break;
-        case 2: values(IC<2>{}); break;
-        case 3: values(IC<3>{}); break;
-        default: values(IC<4>{}); break;
-      }
-    }
-
-    // ---- merge the warps: the unit's (max, sum, accumulator) per query, in an
-    // order of its own: a job's record depends on nothing but its rows and queries ----
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int o = QT == 1 ? 2 : 4; o < 32; o <<= 1) l_run[q] += __shfl_xor_sync(0xffffffffu, l_run[q], o);
-    __syncthreads();                               // every warp is done with its memory and the queries
-    float* const red = reinterpret_cast<float*>(smem + C::Q_RED);   // [warp][NQ][2]: m, l
-    if (g == 0 && (QT == 2 || t < 2)) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        red[(warp * NQ + q0 + q) * 2] = m_run[q];
-        red[(warp * NQ + q0 + q) * 2 + 1] = dead ? __int_as_float(0x7FC00000) : l_run[q];
-      }
-    }
-    __syncthreads();
-    float* const mrg = reinterpret_cast<float*>(wbase);       // [warp][NQ][D]
-    float f[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float M = -INFINITY;
-#pragma unroll
-      for (int x = 0; x < kAttWarps; ++x) M = fmaxf(M, red[(x * NQ + q0 + q) * 2]);
-      // an empty warp (no tokens) has m = -inf, c = inf and adds nothing; NaN scores stay NaN
-      f[q] = m_run[q] == -INFINITY && M > -INFINITY ? 0.f : exp2_whole(m_run[q] - M) * (1.f / c_run[q]);
-      if (M == -INFINITY) f[q] = 1.f;
-    }
-#pragma unroll
-    for (int j = 0; j < VP; ++j) {
-      const int at = 2 * slot_pair<D>(VP * g + j);
-      float o[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if constexpr (QT == 1) {
-          const float a = acc[0][j][i] * f[i & 1];
-          const float b = __shfl_xor_sync(0xffffffffu, a, 2);   // hi lanes t < 2, lo lanes t >= 2
-          o[i] = __fmaf_rn(b, 0.00048828125f, a);
-        } else {
-          o[i] = __fmaf_rn(acc[QT - 1][j][i], 0.00048828125f, acc[0][j][i]) * f[i & 1];
-        }
-      }
-      if (QT == 2 || t < 2) {
-        float* d0 = mrg + (warp * NQ + q0) * D + at;
-        *reinterpret_cast<float2*>(d0) = make_float2(o[0], o[2]);
-        *reinterpret_cast<float2*>(d0 + D) = make_float2(o[1], o[3]);
-      }
-    }
-    __syncthreads();
-    float* const rec = ws + J.ws + (int64_t)unit * nq * att_rec_floats(D);
-    for (int e = tid; e < nq * D; e += kAttThreads) {
-      const int a = e / D, j = e % D;
-      float s = 0.f;
-#pragma unroll
-      for (int x = 0; x < kAttWarps; ++x) s += mrg[(x * NQ + a) * D + j];
-      rec[a * att_rec_floats(D) + 2 + j] = s;
-    }
-    if (tid < nq) {
-      float M = -INFINITY, l = 0.f;
-#pragma unroll
-      for (int x = 0; x < kAttWarps; ++x) M = fmaxf(M, red[(x * NQ + tid) * 2]);
-#pragma unroll
-      for (int x = 0; x < kAttWarps; ++x) {
-        const float mw = red[(x * NQ + tid) * 2];
-        l += red[(x * NQ + tid) * 2 + 1] * (mw == M ? 1.f : exp2_whole(mw - M));
-      }
-      rec[tid * att_rec_floats(D)] = M;
-      rec[tid * att_rec_floats(D) + 1] = l;
-    }
-    fence_async_proxy();
-    __syncthreads();                               // the merge is done with the warps' memory and the queries
-    if (unit + 1 == u_stop - J.unit0) break;
-    issue(false, row0 + kAttUnit, bar_k, bytes_k);
-    issue(true, row0 + kAttUnit, bar_v, bytes_v);
+      fence_async_proxy();
+      __syncthreads();                               // the merge is done with the warps' memory
+      if (unit + 1 == u_stop - J.unit0) break;
+      issue(true, row0 + kAttUnit, bar_v, bytes_v);
     }
   }
 }
@@ -985,7 +969,7 @@ static cudaError_t launch_attend_t(const AttParams& p_in, int nq_max, float* ws,
   p.stage = p.tab_k = p.tab_v = 0;
   for (int j = 0; j < p.njobs; ++j) {
     const AttJob& J = p.job[j];
-    p.stage = std::max(p.stage, att_stage_bytes(D, J.wk, J.bk, J.mk, J.wv, J.bv, J.mv));
+    p.stage = std::max(p.stage, att_stage_bytes(D, J.wk, J.bk, J.mk, J.wv, J.bv, J.mv, C::MERGE));
     p.tab_k = std::max(p.tab_k, 8 << (J.wk + J.lgrk));
     p.tab_v = std::max(p.tab_v, 8 << (J.wv + J.lgrv));
   }

@@ -44,14 +44,15 @@ __host__ __device__ constexpr int att_rec_floats(int d) { return d + 2; }
 // Attention staging: a warp takes its tokens in batches of 32; a staged batch
 // holds 32 rows of each record plane (K angle | K norm | K header | V angle |
 // V norm | V header, headers absent for fp32 norms) plus 16 bytes of slack for
-// word reads past a row's end.
+// word reads past a row's end.  The V rows' place also holds the warp's sums of a
+// unit (`merge` bytes) between two batches.
 constexpr int kAttBatch = 32;
 constexpr int kAttTabBytes = 16384;  // at most, per bin-centre table, all copies
-__host__ __device__ inline int att_stage_bytes(int d, int wk, int bk, int mk, int wv, int bv, int mv) {
+__host__ __device__ inline int att_stage_bytes(int d, int wk, int bk, int mk, int wv, int bv, int mv, int merge) {
   const int P = d / 2;
-  return kAttBatch * (P * wk / 8 + P * bk / 8 + (mk != TAC_NORM_FP32 ? 8 : 0) + P * wv / 8 + P * bv / 8 +
-                      (mv != TAC_NORM_FP32 ? 8 : 0)) +
-         16;
+  const int k = kAttBatch * (P * wk / 8 + P * bk / 8 + (mk != TAC_NORM_FP32 ? 8 : 0));
+  const int v = kAttBatch * (P * wv / 8 + P * bv / 8 + (mv != TAC_NORM_FP32 ? 8 : 0));
+  return k + (v > merge ? v : merge) + 16;
 }
 // Norm decoding case: 0/1 = 4-bit linear/log, 2/3 = 8-bit linear/log, 4 = fp32.
 __host__ __device__ inline int att_norm_case(int bits, int mode) {

@@ -89,7 +89,8 @@ def _job(torch, tac, d, T, nq, seed, dtype):
 @pytest.mark.parametrize("d,nq", [(64, 4), (128, 1), (128, 8)])
 def test_outputs_do_not_depend_on_the_other_jobs(tac_gpu, d, nq):
     """The same bits from a job alone and in batches whose units are dealt to the
-    CTAs in other ways (more units than CTAs, fewer, the job first or last)."""
+    CTAs in other ways (more units than CTAs, fewer, the job first or last), among jobs
+    of more and of fewer queries."""
     import torch
     tac = tac_gpu
     jobs = [_job(torch, tac, d, T, nq, i, torch.float32) for i, T in enumerate([20000, 300, 4097, 33, 70000, 1000])]
@@ -97,7 +98,8 @@ def test_outputs_do_not_depend_on_the_other_jobs(tac_gpu, d, nq):
     for j in jobs:
         tac.attend_multi([j])
         alone.append(j.out.clone())
-    fill = [_job(torch, tac, d, T, nq, 50 + i, torch.float32) for i, T in enumerate([511, 30000, 30000, 7, 90000])]
+    fill = [_job(torch, tac, d, T, m, 50 + i, torch.float32)
+            for i, (T, m) in enumerate([(511, nq), (30000, 8), (30000, 1), (7, 5), (90000, 2)])]
     for batch in (jobs, jobs[::-1], fill[:1] + jobs[1:4], fill + jobs, jobs + fill, jobs[:2] + fill + jobs[2:]):
         for j in jobs:
             j.out.zero_()
@@ -106,6 +108,71 @@ def test_outputs_do_not_depend_on_the_other_jobs(tac_gpu, d, nq):
         for j, want in zip(jobs, alone):
             if any(j is b for b in batch):
                 assert torch.equal(j.out, want), (j.tokens, len(batch))
+
+
+def _fwht(x, dtype):
+    """Unnormalized Walsh-Hadamard butterfly over the last axis, in `dtype`."""
+    import torch
+    x, d = x.to(dtype), x.shape[-1]
+    for h in [1 << i for i in range(d.bit_length() - 1)]:
+        v = x.reshape(*x.shape[:-1], d // (2 * h), 2, h)
+        x = torch.stack([v[..., 0, :] + v[..., 1, :], v[..., 0, :] - v[..., 1, :]], -2).reshape(x.shape)
+    return x
+
+
+def _plain(q, rk, ak, rv, av, scale, signs, dtype):
+    """The kernel's op with every operation in `dtype`: rotated queries, scores against
+    r (cos, sin), base-2 softmax, weighted values, one transform of the output."""
+    import torch
+    d = q.shape[-1]
+    cs = lambda r, a: torch.stack([r.to(dtype) * torch.cos(a).to(dtype), r.to(dtype) * torch.sin(a).to(dtype)], -1).flatten(-2)
+    qr = _fwht(q.to(dtype) * signs[0].to(dtype), dtype) * (scale * math.log2(math.e) / math.sqrt(d))
+    s = (qr[..., :, None, :] * cs(rk, ak)[..., None, :, :]).sum(-1)
+    p = torch.exp2(s - s.amax(-1, keepdim=True))
+    y = (p[..., None] * cs(rv, av)[..., None, :, :]).sum(-2) / p.sum(-1, keepdim=True)
+    return _fwht(y, dtype) / math.sqrt(d) * signs[1].to(dtype)
+
+
+@pytest.mark.parametrize("T", [1, 2, 5, 20, 33, 130, 300, 1500])
+@pytest.mark.parametrize("d,nq", [(64, 2), (128, 8)])
+def test_error_no_larger_than_that_of_fp32_arithmetic(tac_gpu, d, nq, T):
+    """Outputs against 64 bits (2-norm over 16 jobs of fp32 norms) are no further off
+    than the same op in fp32 throughout, by more than the spread of such a ratio
+    (each side a few thousand rounding errors; pairwise sums in the fp32 one, whose
+    error is the least fp32 arithmetic can have).  Jobs of more than 256 tokens keep
+    two parts of a value: the residue's rounding (0.44 * 2^-23 of the record's scale
+    in the mean square) is about as large as that error and adds to the 0.75 of it
+    that three parts leave: sqrt(1 + 0.75^2) = 1.25."""
+    import torch
+    tac, n, jobs = tac_gpu, 256, 16
+    g = torch.Generator(device="cuda")
+    g.manual_seed(100 * d + T)
+    cfg = [tac.layer_cfg(d, n, 32, tac.NORM_FP32, 0, 1, kv) for kv in (0, 1)]
+    signs = [torch.tensor(parity.signs_pm1(c.signs, d), dtype=torch.float64, device="cuda") for c in cfg]
+    order = torch.tensor([4 * (v % (d // 16)) + (v // (d // 16)) % 4 + d // 4 * (v // (d // 4)) for v in range(d // 2)],
+                         device="cuda")
+    q = 2 * torch.randn((jobs, nq, d), generator=g, device="cuda")
+    out = torch.zeros_like(q)
+    r, a, job = [[], []], [[], []], []
+    for i in range(jobs):
+        caches = []
+        for kv in (0, 1):
+            c = tac.Cache.empty(cfg[kv], T)
+            k = torch.randint(0, n, (T, d // 2), generator=g, device="cuda", dtype=torch.uint8)
+            v = torch.sqrt(torch.empty((T, d // 2), device="cuda").exponential_(0.5, generator=g))
+            c.codes[: k.numel()] = k.reshape(-1)
+            c.norms[: 4 * v.numel()] = v.reshape(-1).view(torch.uint8)
+            pairs = torch.empty((2, T, d // 2), dtype=torch.float64, device="cuda")
+            pairs[0][:, order], pairs[1][:, order] = v.double(), k.double() * (2 * math.pi / n)
+            r[kv].append(pairs[0]), a[kv].append(pairs[1])
+            caches.append(c)
+        job.append(tac.AttendJob(cfg[0], caches[0], cfg[1], caches[1], T, q[i], out[i], 1.0 / math.sqrt(d)))
+    tac.attend_multi(job)
+    args = [torch.stack(x) for kv in (0, 1) for x in (r[kv], a[kv])]
+    want, fp32 = (_plain(q, *args, 1.0 / math.sqrt(d), signs, t) for t in (torch.float64, torch.float32))
+    torch.cuda.synchronize()
+    err, lim = (float((x.double() - want).norm() / want.norm()) for x in (out, fp32))
+    assert err <= (1.15 if T <= 256 else 1.25) * lim, (err, lim)
 
 
 def test_attend_captured_into_graph(tac_gpu):

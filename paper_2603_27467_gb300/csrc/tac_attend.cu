@@ -181,7 +181,8 @@ __device__ __forceinline__ void norm_consts(float2 h, float inv_l, bool lg, floa
 
 // A warp's staged batches arrive by bulk copies (cp.async.bulk) that signal an
 // mbarrier of its own.  A wait gives up after 2^16 tries (each suspends the
-// warp for a while) and returns false; the kernel then marks its results NaN.
+// warp for a while) and returns false; the warp then copies nothing more, its
+// results are NaN, and it waits (as long at most) for its copies before it leaves.
 __device__ __forceinline__ uint32_t smem_addr(const void* ptr) { return (uint32_t)__cvta_generic_to_shared(ptr); }
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
@@ -305,6 +306,7 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
         smem_addr(sg == 0 ? (is_v ? st_va : stk) : sg == 1 ? (is_v ? st_vn : st_kn) : (is_v ? st_vh : st_kh));
     auto issue = [&](bool v, int64_t row, uint32_t bar, int bytes) {
       const bool mine = (is_v == v) && lane < 6 && c_row > 0;
+      if (dead) return;
       if (row + kAttBatch <= seg_rows) {
         if (lane == 0) mbar_expect(bar, bytes);
         __syncwarp();
@@ -326,8 +328,8 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
     // waits for the batch of rows [row, row + 32)
     auto landed = [&](int64_t row, uint32_t bar, uint32_t& phase) {
       if (row + kAttBatch <= seg_rows) {
-        if (!dead) dead = !mbar_wait(bar, phase);
-        phase ^= 1u;
+        if (!dead) dead = !__all_sync(0xffffffffu, mbar_wait(bar, phase));
+        if (!dead) phase ^= 1u;
       } else {
         cp_async_wait<0>();
       }
@@ -880,6 +882,10 @@ __global__ void __launch_bounds__(kAttThreads, QT == 1 ? 2 : 1)
       if (unit + 1 == u_stop - J.unit0) break;
       issue(true, row0 + kAttUnit, bar_v, bytes_v);
     }
+  }
+  if (dead) {                                        // the copies issued and not waited for
+    (void)mbar_wait(bar_k, phase_k);
+    (void)mbar_wait(bar_v, phase_v);
   }
 }
 

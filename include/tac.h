@@ -231,6 +231,11 @@ int tac_decode(const void* codes, const void* norms, const tac_layer_cfg* cfg, t
  */
 int tac_encode_multi(const tac_encode_job* jobs, int njobs, tac_stream_t stream);
 
+/* Kernel launches tac_encode_multi or tac_encode_multi_ws makes for these jobs
+ * (host only): one for each group of a small call, two (the encode and its
+ * fix-up) in a larger one.  -1 (tac_last_error) for a call it would reject. */
+int tac_encode_launches(const tac_encode_job* jobs, int njobs);
+
 /*
  * The encode's re-decision workspace.  The fast path decides every code in
  * fp32 and certifies it against a bound on its own error (Alg. 1's edge test,

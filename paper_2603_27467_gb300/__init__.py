@@ -118,6 +118,8 @@ def load():
         lib.tac_encode_multi.argtypes = [P(_EncJob), i32, vp]
         lib.tac_encode_workspace_bytes.restype = i64
         lib.tac_encode_workspace_bytes.argtypes = [P(_EncJob), i32, P(ctypes.c_int64)]
+        lib.tac_encode_launches.restype = i32
+        lib.tac_encode_launches.argtypes = [P(_EncJob), i32]
         lib.tac_encode_multi_ws.restype = i32
         lib.tac_encode_multi_ws.argtypes = [P(_EncJob), i32, vp, i64, vp]
         lib.tac_decode_multi.restype = i32
@@ -566,22 +568,33 @@ def attend_multi_static(jobs, stream=None):
 
 
 def launch_count(jobs) -> int:
-    """Kernel launches one (not small) encode_multi / decode_multi call makes
-    for `jobs`: jobs with rows are grouped by kernel (d, dtype, n, norm bits,
-    norm mode), at most MAX_JOBS jobs per group; a decode group is one launch,
-    an encode group two (the encode and its fix-up).  A small encode call (see
-    tac_encode_multi) makes fewer: one per (d, dtype)."""
+    """Kernel launches one encode_multi / decode_multi call makes for `jobs`.
+    Jobs with rows are grouped by kernel (d, dtype, n, norm bits, norm mode), at
+    most MAX_JOBS jobs per group; a decode group is one launch, an encode group
+    two (the encode and its fix-up).  A small encode call (see tac_encode_multi)
+    is one launch per (d, dtype) and MAX_JOBS jobs."""
+    jobs = list(jobs)
+    if not jobs:
+        return 0
+    if isinstance(jobs[0], EncodeJob):
+        # the library's own plan, from the jobs' shapes (it looks at no memory)
+        arr, at = (_EncJob * len(jobs))(), 0
+        for j in jobs:
+            rows, ok = j.x.shape[0], 1 << 12           # an aligned address that is never read
+            _ENC_FMT.pack_into(arr, at, _cfg_bytes(j.cfg), ok, _dtype_code(j.x), rows, j.cfg.d, ok, ok, rows,
+                               0 if j.slot is None else ok, 0)
+            at += _ENC_FMT.size
+        n = load().tac_encode_launches(arr, len(jobs))
+        if n < 0:
+            raise TacError(TAC_E_INVAL, last_error())
+        return int(n)
     groups: dict = {}
-    per = 1
     for j in jobs:
-        t = j.x if isinstance(j, EncodeJob) else j.y
-        if isinstance(j, EncodeJob):
-            per = 2
-        if t.shape[0] == 0:
+        if j.y.shape[0] == 0:
             continue
-        key = (j.cfg.d, str(t.dtype), j.cfg.n_angle, j.cfg.norm_bits, j.cfg.norm_mode)
+        key = (j.cfg.d, str(j.y.dtype), j.cfg.n_angle, j.cfg.norm_bits, j.cfg.norm_mode)
         groups[key] = groups.get(key, 0) + 1
-    return per * sum(-(-c // MAX_JOBS) for c in groups.values())
+    return sum(-(-c // MAX_JOBS) for c in groups.values())
 
 
 def fwht_debug(x, signs: np.ndarray, d: int, stream=None):

@@ -631,6 +631,15 @@ int64_t tac_encode_workspace_bytes(const tac_encode_job* jobs, int njobs, int64_
   return w.rec;
 }
 
+int tac_encode_launches(const tac_encode_job* jobs, int njobs) {
+  static thread_local std::vector<EncGroup> groups;
+  bool small = false;
+  int64_t min_ws = 0;
+  if (plan_encode(jobs, njobs, "tac_encode_launches", groups, EncPlan::kSmallOrShapes, &small, &min_ws)) return -1;
+  ok();
+  return (int)groups.size() * (small ? 1 : 2);
+}
+
 int tac_encode_multi_ws(const tac_encode_job* jobs, int njobs, void* workspace, int64_t workspace_bytes,
                         tac_stream_t stream) {
   static const char* who = "tac_encode_multi_ws";

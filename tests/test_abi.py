@@ -266,17 +266,27 @@ def test_launch_count_matches_the_grouping(tac_host):
     """launch_count (the bench's gpu_launches): jobs with rows grouped by kernel
     shape (d, dtype, n, norm bits, norm mode), at most MAX_JOBS to a group; an
     encode group launches the encode kernel and its fix-up, a decode group one
-    kernel."""
+    kernel.  A small encode call is grouped by (d, dtype) alone, one launch each:
+    fewer than 16384 warp tiles and 10240 more for each of up to four shapes."""
     import torch
     tac = tac_host
     k_cfg, v_cfg = tac.LayerCfg(128, 64, 8, 0), tac.LayerCfg(128, 256, 4, 1)
-    x = torch.zeros((4, 128), dtype=torch.bfloat16)
-    empty = torch.zeros((0, 128), dtype=torch.bfloat16)
-    enc = [tac.EncodeJob(k_cfg, x, None), tac.EncodeJob(k_cfg, x, None), tac.EncodeJob(v_cfg, x, None),
-           tac.EncodeJob(v_cfg, empty, None), tac.EncodeJob(k_cfg, x.float(), None)]
-    assert tac.launch_count(enc) == 2 * 3            # (k, bf16), (v, bf16), (k, fp32); the empty job adds none
-    many = [tac.EncodeJob(k_cfg, x, None)] * (tac.MAX_JOBS + 1)
+
+    def rows(n, dtype=torch.bfloat16):
+        return torch.empty((n, 128), dtype=dtype, device="meta")
+
+    enc = [tac.EncodeJob(k_cfg, rows(4), None), tac.EncodeJob(k_cfg, rows(4), None), tac.EncodeJob(v_cfg, rows(4), None),
+           tac.EncodeJob(v_cfg, rows(0), None), tac.EncodeJob(k_cfg, rows(4, torch.float32), None)]
+    assert tac.launch_count(enc) == 2                # (128, bf16), (128, fp32); the empty job adds none
+    limit = 16384 + 3 * 10240                        # three shapes
+    enc[0] = tac.EncodeJob(k_cfg, rows(4 * (limit - 3) - 4), None)
+    assert tac.launch_count(enc) == 2                # one tile below the limit
+    enc[0] = tac.EncodeJob(k_cfg, rows(4 * (limit - 3) - 3), None)
+    assert tac.launch_count(enc) == 2 * 3            # (k, bf16), (v, bf16), (k, fp32)
+    many = [tac.EncodeJob(k_cfg, rows(4), None)] * (tac.MAX_JOBS + 1)
+    assert tac.launch_count(many) == 2
+    many = [tac.EncodeJob(k_cfg, rows(2000), None)] * (tac.MAX_JOBS + 1)
     assert tac.launch_count(many) == 2 * 2
-    dec = [tac.DecodeJob(k_cfg, None, x), tac.DecodeJob(v_cfg, None, x), tac.DecodeJob(v_cfg, None, empty)]
+    dec = [tac.DecodeJob(k_cfg, None, rows(4)), tac.DecodeJob(v_cfg, None, rows(4)), tac.DecodeJob(v_cfg, None, rows(0))]
     assert tac.launch_count(dec) == 2
     assert tac.launch_count([]) == 0

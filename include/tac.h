@@ -211,7 +211,9 @@ int tac_decode(const void* codes, const void* norms, const tac_layer_cfg* cfg, t
  * (fewer than 16384 warp tiles - 4-row d = 128 tiles, 8-row d = 64 tiles, ... -
  * plus 10240 for each kernel shape, up to four) is one launch for each (d,
  * dtype) and TAC_MAX_JOBS jobs, which takes every codebook and re-decides its
- * own codes; it uses no workspace.  In larger calls jobs that share the kernel
+ * own codes; it uses no workspace.  (A call with `slot` and angle records of no
+ * multiple of 4 bytes - odd code widths at d <= 32 - never counts as small.)  In
+ * larger calls jobs that share the kernel
  * shape (d, dtype, n_angle, norm_bits, norm_mode) run in one launch (one per
  * TAC_MAX_JOBS such jobs).  With several launches they run
  * concurrently, largest first: the first on `stream`, the others on

@@ -405,7 +405,8 @@ int64_t enc_min_bytes(int64_t tile_rows_total, int64_t njobs) {
 // limit grows with the launches it saves.  Measured (us, shape kernels / this
 // one): 4 shapes, d = 128, bf16: 128 tiles 37 / 12, 8192 tiles 38 / 21, 32768
 // tiles 58 / 47, 65536 tiles 78 / 84; one shape, d = 64, fp32 norms: 22000
-// tiles 31 / 29, 66000 tiles 54 / 70.
+// tiles 31 / 29, 66000 tiles 54 / 70.  Calls with scattered records that share
+// words (see plan_encode) are not small.
 constexpr int64_t kSmallEncodeTiles = 16384, kSmallEncodePerShape = 10240;
 constexpr int kSmallEncodeShapes = 4;
 
@@ -456,11 +457,19 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
   if (how == EncPlan::kSmallOrShapes) {
     int64_t total = 0;
     int shapes = 0;
+    bool shared_words = false;
     for (size_t k = 0; k < live.size(); ++k) {
+      const tac_encode_job& J = jobs[live[k]];
       total += job_tiles(live[k]);
       shapes += k == 0 || kernel_key(live[k]) != kernel_key(live[k - 1]);
+      // Scattered records whose bytes are no multiple of 4 (odd code widths at
+      // d <= 32) share 32-bit words: re-deciding a code rewrites its word
+      // atomically while another CTA may still store the neighbour's bytes, an
+      // order the memory model leaves open within one kernel.  The launches by
+      // shape re-decide in a kernel of their own.
+      shared_words = shared_words || (J.slot && angle_row_bytes(&J.cfg) % 4 != 0);
     }
-    *small = total < kSmallEncodeTiles + kSmallEncodePerShape * std::min(shapes, kSmallEncodeShapes);
+    *small = !shared_words && total < kSmallEncodeTiles + kSmallEncodePerShape * std::min(shapes, kSmallEncodeShapes);
     if (*small) {
       key_shift = 17;                                  // (d, dtype)
       *min_ws = 0;

@@ -290,3 +290,19 @@ def test_launch_count_matches_the_grouping(tac_host):
     dec = [tac.DecodeJob(k_cfg, None, rows(4)), tac.DecodeJob(v_cfg, None, rows(4)), tac.DecodeJob(v_cfg, None, rows(0))]
     assert tac.launch_count(dec) == 2
     assert tac.launch_count([]) == 0
+
+
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+def test_scattered_records_that_share_words_are_not_small(tac_host, d):
+    """Re-deciding a code rewrites its 32-bit word, so records that share words are
+    re-decided in a launch after the encode, never beside other CTAs' stores."""
+    import torch
+    tac = tac_host
+    x, slot = torch.empty((5, d), device="meta"), torch.empty(5, dtype=torch.int64, device="meta")
+    for n in (2, 4, 8, 16, 32, 48, 56, 64, 128, 256):
+        cfg = tac.LayerCfg(d, n, 8, 0)
+        w = (n - 1).bit_length()
+        shared = d // 2 * w % 32 != 0
+        assert tac.launch_count([tac.EncodeJob(cfg, x, None)]) == 1
+        assert tac.launch_count([tac.EncodeJob(cfg, x, None, slot)]) == (2 if shared else 1)
+        assert shared == (d == 16 and w % 4 != 0 or d == 32 and w % 2 != 0)

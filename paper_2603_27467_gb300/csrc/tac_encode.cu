@@ -1117,9 +1117,7 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
       hmin = TAME ? sqrt_ftz(smin * k2) : sqrt_approx(smin * k2);   // smin * sigma may still be subnormal
       hmax = kEvenK2 ? rms * rk2 : sqrt_ftz(smax_s * k2);
       if (!TAME) hmax *= sr;
-      const float range = hmax - hmin, rr = rcp_approx(range);
-      sc = (float)Lq * rr;
-      sc = __fmaf_rn(__fmaf_rn(-range, sc, (float)Lq), rr, sc);     // Lq / range to within u
+      sc = (float)Lq * rcp_approx(hmax - hmin);
       qs = sc * rk2;                            // f(s) = sqrt(s)
       qo = __fmaf_rn(-hmin, sc, 0.5f);
       if (!(hmax > hmin) || !(sc <= 3.0e38f)) { qs = 0.f; qo = 0.5f; }

@@ -31,6 +31,7 @@ U = 2.0**-24
 ANGLE_BAND = 1e-5      # rad: angle codes may differ only this close to a bin edge
 NORM_BAND = 1e-4       # code units: norm codes may differ only this close to a midpoint
 MISMATCH_RATE = 1e-6   # largest share of codes allowed to differ inside a band
+SMALL_LIMIT = 16384 + 10240   # warp tiles: smaller calls of one codebook shape take the small-call kernel
 E_SQRT = 2.0**-23      # relative error bound of the hardware square root the kernels use
 
 
@@ -64,6 +65,31 @@ def gpu_codes(orc, cache, rows: int | None = None, slots: np.ndarray | None = No
     k = orc.unpack_record(codes, cfg.d, code_bits(cfg.n_angle))
     c = orc.unpack_record(norms, cfg.d, cfg.norm_bits)
     return k, c, hdr
+
+
+def encode_by_shape(tac, x, cfg, status=None):
+    """tac.encode of x as part of a call too large for the small-call kernel (rows of
+    zeros make up its size): the kernel of the codebook's shape and its fix-up kernel."""
+    import torch
+    rows = (SMALL_LIMIT + 1) * (32 // (cfg.d // 16))
+    zeros = torch.zeros((rows, cfg.d), dtype=x.dtype, device=x.device)
+    cache = tac.Cache.empty(cfg, x.shape[0], device=x.device)
+    jobs = [tac.EncodeJob(cfg, x, cache, None, status), tac.EncodeJob(cfg, zeros, tac.Cache.empty(cfg, rows, device=x.device))]
+    assert tac.launch_count(jobs) == 2
+    tac.encode_multi(jobs)
+    return cache
+
+
+def assert_same_records(tac, a, b):
+    """Two caches of one configuration hold the same bytes (NaN headers included)."""
+    import torch
+    n = a.capacity
+    used = n * tac.norm_row_bytes(a.cfg)
+    off = tac.header_offset(a.cfg, n)
+    assert torch.equal(a.codes[: tac.codes_bytes(a.cfg, n)], b.codes[: tac.codes_bytes(a.cfg, n)])
+    assert torch.equal(a.norms[:used], b.norms[:used])
+    if a.cfg.norm_mode != tac.NORM_FP32:
+        assert torch.equal(a.norms[off: off + 8 * n], b.norms[off: off + 8 * n])
 
 
 def _gamma(x64: np.ndarray) -> np.ndarray:

@@ -40,6 +40,8 @@ def check_roundtrip(tac, orc, x, d, n, b, mode, seed=0, layer=0, kv=0, label="",
     rows = x.shape[0]
     cfg = tac.layer_cfg(d, n, b, mode, seed, layer, kv)
     cache = tac.encode(x, cfg)
+    # the same records from the kernels of a large call
+    parity.assert_same_records(tac, cache, parity.encode_by_shape(tac, x, cfg))
     torch.cuda.synchronize()
     x64 = parity.to_f64(x)
     s = orc.signs(seed, layer, kv, d)
@@ -192,7 +194,7 @@ def test_exact_bin_centres_and_ties(tac_gpu, orc):
     for n in (4, 8, 64, 256):
         cfg = tac_gpu.layer_cfg(d, n, 8, 0, 0, 0, 0)
         cache = tac_gpu.encode(xt, cfg)
-        torch.cuda.synchronize()
+        parity.assert_same_records(tac_gpu, cache, parity.encode_by_shape(tac_gpu, xt, cfg))
         k, c, hdr = parity.gpu_codes(orc, cache, 4)
         want = orc.encode(x, s, n, 8, 0)["k"]
         assert np.array_equal(k, want), (n, k[:, :3], want[:, :3])
@@ -315,6 +317,9 @@ def test_nonfinite_rows(tac_gpu, orc, dt, b, mode):
     y = tac_gpu.decode(cache, cfg, dtype=torch.float32)
     torch.cuda.synchronize()
     assert int(status.item()) == tac_gpu.TAC_E_NONFINITE
+    status.zero_()
+    parity.assert_same_records(tac_gpu, cache, parity.encode_by_shape(tac_gpu, x, cfg, status))
+    assert int(status.item()) == tac_gpu.TAC_E_NONFINITE
     k, c, hdr = parity.gpu_codes(orc, cache, x.shape[0])
     assert np.all(k[bad] == 0)
     if mode == parity.FP32_MODE:
@@ -341,24 +346,27 @@ def test_small_workspace_rows_redecided_whole(tac_gpu, orc, room):
     """With the minimum workspace (no queue room) every queued code's row is
     re-decided whole through the bitmap; with a queue of a few dozen entries
     some codes go through the queue and the rest of the rows whole.  The
-    records satisfy the same parity rule as with the recommended workspace."""
+    records satisfy the same parity rule as with the recommended workspace.  The
+    call is too large for the small-call kernel, which has no queue; the first 6000
+    rows are compared."""
     torch = _torch()
     w = workloads.CONFIGS["mistral7b"]
     for kv in (workloads.K, workloads.V):
         d, n, b, mode = w.codebook(0, kv)
-        x = _rows(w, 6000, seed=5, layer=0, kv=kv)
+        x = _rows(w, 4 * (parity.SMALL_LIMIT + 1), seed=5, layer=0, kv=kv)
         cfg = tac_gpu.layer_cfg(d, n, b, mode, 0, 0, kv)
         cache = tac_gpu.Cache.empty(cfg, x.shape[0])
         jobs = [tac_gpu.EncodeJob(cfg, x, cache)]
+        assert tac_gpu.launch_count(jobs) == 2
         rec, mn = tac_gpu.encode_workspace_bytes(jobs)
         size = mn if room == "min" else mn + 32 * 40
-        wsb = torch.empty(size, dtype=torch.uint8, device="cuda")
+        wsb = torch.zeros(size, dtype=torch.uint8, device="cuda")
         tac_gpu.encode_multi(jobs, workspace=wsb)
         torch.cuda.synchronize()
-        x64 = parity.to_f64(x)
+        x64 = parity.to_f64(x[:6000])
         s = orc.signs(0, 0, kv, d)
         ref = orc.encode(x64, s, n, b, mode)
-        k, c, hdr = parity.gpu_codes(orc, cache, x.shape[0])
+        k, c, hdr = parity.gpu_codes(orc, cache, 6000)
         parity.compare_encode(orc, x64, ref, k, c, hdr, n, b, mode, label=f"workspace {room} kv={kv}")
         # the queue overflowed: the counter passed the queue's capacity
         appended = int(wsb[:8].cpu().numpy().view(np.uint64)[0])

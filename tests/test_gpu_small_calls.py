@@ -51,6 +51,11 @@ def test_small_calls_match_large_ones(tac_gpu, d, dtype):
     rw = 32 // (d // 16)
     rows = LARGE_TILES * rw + 3
     x = _rows(torch, d, dtype, rows)
+    # seven rows in eight of those not compared are zero: the re-decision queue then
+    # holds every entry (which codes a full one leaves to whole rows varies)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + 2)
+    x[1000: rows - 1000][torch.rand(rows - 2000, generator=g, device="cuda") < 0.875] = 0
     pieces = [(0, 400), (400, 1), (401, rw - 1), (500, rw), (600, rw + 1), (700, 5 * rw + 3), (rows - 1000, 1000)]
     pieces = [(a, k) for a, k in pieces if k > 0]
     g = torch.Generator(device="cuda")
@@ -89,6 +94,44 @@ def test_small_calls_match_large_ones(tac_gpu, d, dtype):
                 if ref is not None:
                     assert torch.equal(got[sel[ok]], ref[a:a + k][ok]), (n, b, m, a, k)
             assert int(s) == (tac.TAC_E_NONFINITE if a == 0 else 0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+def test_large_scattered_calls_match_dense_ones(tac_gpu, d, dtype):
+    """A call by shape whose rows go to a permutation of slots, some of them out of
+    range: the dense call's records, and nothing else is written.  Seven rows in eight
+    are zero, so that the re-decision queue holds every entry (which codes a full one
+    leaves to whole rows differs from run to run)."""
+    import torch
+    import parity
+    tac = tac_gpu
+    rows = (parity.SMALL_LIMIT + 1) * (32 // (d // 16)) + 3
+    cap = rows + 1000
+    x = _rows(torch, d, dtype, rows)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + 1)
+    x[400:][torch.rand(rows - 400, generator=g, device="cuda") < 0.875] = 0
+    slot = torch.randperm(cap, generator=g, device="cuda")[:rows]
+    slot[::97], slot[5::101], slot[rows - 1] = -1, cap, cap + 5
+    ok = (slot >= 0) & (slot < cap)
+    free = torch.ones(cap, dtype=torch.bool, device="cuda")
+    free[slot[ok]] = False
+    for n, b, m in SHAPES:
+        cfg = tac.layer_cfg(d, n, b, m, 0, 3, 0)
+        dense, scat = tac.Cache.empty(cfg, rows), tac.Cache.empty(cfg, cap)
+        scat.codes.fill_(0xA5)
+        scat.norms.fill_(0xA5)
+        jobs = [tac.EncodeJob(cfg, x, scat, slot)]
+        assert tac.launch_count(jobs) == 2
+        ws = torch.zeros(tac.encode_workspace_bytes(jobs)[0], dtype=torch.uint8, device="cuda")
+        tac.encode_multi(jobs, workspace=ws)
+        tac.encode_multi([tac.EncodeJob(cfg, x, dense)])
+        assert int(ws[:8].view(torch.int64)) <= rows * (d // 2) // 512 + 1024
+        for got, ref in zip(_view(torch, tac, scat), _view(torch, tac, dense)):
+            if ref is not None:
+                assert torch.equal(got[slot[ok]], ref[ok]), (n, b, m)
+                assert bool((got[free] == 0xA5).all()), (n, b, m)
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])

@@ -209,22 +209,22 @@ int tac_decode(const void* codes, const void* norms, const tac_layer_cfg* cfg, t
 /*
  * Batched encode.  Jobs may mix d, input dtypes and codebooks.  A small call
  * (fewer than 16384 warp tiles - 4-row d = 128 tiles, 8-row d = 64 tiles, ... -
- * plus 10240 for each kernel shape, up to four) is one launch for each (d,
- * dtype) and TAC_MAX_JOBS jobs, which takes every codebook and re-decides its
- * own codes; it uses no workspace.  (A call with `slot` and angle records of no
- * multiple of 4 bytes - odd code widths at d <= 32 - never counts as small.)  In
- * larger calls jobs that share the kernel
- * shape (d, dtype, n_angle, norm_bits, norm_mode) run in one launch (one per
- * TAC_MAX_JOBS such jobs).  With several launches they run
+ * plus 10240 for each kernel shape, up to four; a tile of fp32 rows counts 5/3)
+ * is one launch for each (d, dtype) and TAC_MAX_JOBS jobs, which takes every
+ * codebook and re-decides its own codes; it uses no workspace.  (A call with
+ * `slot` and angle records of no multiple of 4 bytes - odd code widths at d <= 32
+ * - never counts as small.)  In larger calls jobs that share the kernel shape (d,
+ * dtype, n_angle, norm_bits, norm_mode) run in one launch (one per TAC_MAX_JOBS
+ * such jobs).  With several launches they run
  * concurrently, largest first: the first on `stream`, the others on
  * library-owned streams that wait for `stream` at the call (an event), while
  * `stream` waits for them before the call returns (events), so the call's work
  * is ordered on `stream` as if it ran there alone and may be captured into a
  * CUDA graph.  A call with fewer than 640 warp tiles per SM in all gives each
  * launch a share of the SMs in proportion to its tiles, so that its launches
- * run side by side; larger calls give every launch the whole GPU.  Each launch is followed by its
- * fix-up kernel (see tac_encode_multi_ws): with shares of the SMs on the
- * launch's stream right after it, otherwise after all of the call's encode
+ * run side by side; larger calls give every launch the whole GPU.  Each launch is
+ * followed by its fix-up kernel (see tac_encode_multi_ws): with shares of the SMs
+ * on the launch's stream right after it, otherwise after all of the call's encode
  * launches (a second fork / join), the fix-ups side by side.  The first call
  * with several launches on a device creates three streams and four events
  * (kept for the process); make it outside stream capture.  With `slot` the

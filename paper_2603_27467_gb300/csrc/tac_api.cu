@@ -405,10 +405,15 @@ int64_t enc_min_bytes(int64_t tile_rows_total, int64_t njobs) {
 // limit grows with the launches it saves.  Measured (us, shape kernels / this
 // one): 4 shapes, d = 128, bf16: 128 tiles 37 / 12, 8192 tiles 38 / 21, 32768
 // tiles 58 / 47, 65536 tiles 78 / 84; one shape, d = 64, fp32 norms: 22000
-// tiles 31 / 29, 66000 tiles 54 / 70.  Calls with scattered records that share
+// tiles 31 / 29, 66000 tiles 54 / 70.  fp32 rows (twice the bytes of a tile to
+// stage, and more uncertified codes) meet at 0.6 of the limit that bf16 rows do:
+// with their tiles counted 5/3 no mix of d and shapes is slower than 0.97 of the
+// launches by shape just below the limit, 0.82 to 0.95 with them counted once (d =
+// 16, one shape, fp32 norms, 26000 tiles 33 / 40).  Calls with scattered records that share
 // words (see plan_encode) are not small.
 constexpr int64_t kSmallEncodeTiles = 16384, kSmallEncodePerShape = 10240;
 constexpr int kSmallEncodeShapes = 4;
+constexpr int64_t kSmallTileBf16 = 3, kSmallTileFp32 = 5;   // a tile's weight against 3 x the limit
 
 // How an encode call is grouped into launches: by kernel shape, or (a small
 // call) by (d, dtype) alone.
@@ -460,7 +465,7 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
     bool shared_words = false;
     for (size_t k = 0; k < live.size(); ++k) {
       const tac_encode_job& J = jobs[live[k]];
-      total += job_tiles(live[k]);
+      total += job_tiles(live[k]) * (J.x.dtype == TAC_FP32 ? kSmallTileFp32 : kSmallTileBf16);
       shapes += k == 0 || kernel_key(live[k]) != kernel_key(live[k - 1]);
       // Scattered records whose bytes are no multiple of 4 (odd code widths at
       // d <= 32) share 32-bit words: re-deciding a code rewrites its word
@@ -469,7 +474,8 @@ int plan_encode(const tac_encode_job* jobs, int njobs, const char* who, std::vec
       // shape re-decide in a kernel of their own.
       shared_words = shared_words || (J.slot && angle_row_bytes(&J.cfg) % 4 != 0);
     }
-    *small = !shared_words && total < kSmallEncodeTiles + kSmallEncodePerShape * std::min(shapes, kSmallEncodeShapes);
+    *small = !shared_words &&
+             total < kSmallTileBf16 * (kSmallEncodeTiles + kSmallEncodePerShape * std::min(shapes, kSmallEncodeShapes));
     if (*small) {
       key_shift = 17;                                  // (d, dtype)
       *min_ws = 0;

@@ -267,7 +267,8 @@ def test_launch_count_matches_the_grouping(tac_host):
     shape (d, dtype, n, norm bits, norm mode), at most MAX_JOBS to a group; an
     encode group launches the encode kernel and its fix-up, a decode group one
     kernel.  A small encode call is grouped by (d, dtype) alone, one launch each:
-    fewer than 16384 warp tiles and 10240 more for each of up to four shapes."""
+    fewer than 16384 warp tiles and 10240 more for each of up to four shapes, a tile
+    of fp32 rows counting 5/3."""
     import torch
     tac = tac_host
     k_cfg, v_cfg = tac.LayerCfg(128, 64, 8, 0), tac.LayerCfg(128, 256, 4, 1)
@@ -283,6 +284,8 @@ def test_launch_count_matches_the_grouping(tac_host):
     assert tac.launch_count(enc) == 2                # one tile below the limit
     enc[0] = tac.EncodeJob(k_cfg, rows(4 * (limit - 3) - 3), None)
     assert tac.launch_count(enc) == 2 * 3            # (k, bf16), (v, bf16), (k, fp32)
+    for tiles, launches in ((26624 * 3 // 5, 1), (26624 * 3 // 5 + 1, 2)):   # one shape, fp32 rows
+        assert tac.launch_count([tac.EncodeJob(k_cfg, rows(4 * tiles, torch.float32), None)]) == launches
     many = [tac.EncodeJob(k_cfg, rows(4), None)] * (tac.MAX_JOBS + 1)
     assert tac.launch_count(many) == 2
     many = [tac.EncodeJob(k_cfg, rows(2000), None)] * (tac.MAX_JOBS + 1)

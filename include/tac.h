@@ -258,7 +258,8 @@ int tac_encode_launches(const tac_encode_job* jobs, int njobs);
  * tac_encode_multi_ws is tac_encode_multi with the caller's workspace (device
  * memory, 16-byte aligned, at least the minimum; its contents need no
  * initialization; it must not be used by other work until the call's work on
- * `stream` is done).  TAC_E_INVAL if the workspace is too small.
+ * `stream` is done).  TAC_E_INVAL if the workspace is too small.  A small call
+ * checks the workspace in the same way and leaves it alone.
  */
 int64_t tac_encode_workspace_bytes(const tac_encode_job* jobs, int njobs, int64_t* min_bytes);
 int tac_encode_multi_ws(const tac_encode_job* jobs, int njobs, void* workspace, int64_t workspace_bytes,

@@ -438,8 +438,9 @@ def _enc_workspace(jobs, arr, workspace):
 
 def encode_multi(jobs, stream=None, workspace=None):
     """tac_encode_multi_ws: one encode launch and one fix-up launch per kernel
-    group, or one launch for a small call (see launch_count); allocates the re-decision workspace (torch) when
-    none is given.  Returns the workspace."""
+    group, or one launch for a small call (see launch_count); allocates the
+    re-decision workspace (torch) when none is given (a small call leaves it
+    alone).  Returns the workspace."""
     arr = _enc_array(jobs)
     workspace = _enc_workspace(jobs, arr, workspace)
     _check(load().tac_encode_multi_ws(arr, len(jobs), workspace.data_ptr(),

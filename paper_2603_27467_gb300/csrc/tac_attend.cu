@@ -20,7 +20,8 @@
 //                   its record, into hi (a multiple of 2^-10), the residue of the
 //                   product rounded to fp16 and, in jobs of few tokens, what that
 //                   leaves; the queries and the softmax weights into a multiple of
-//                   2^-6 and two residues, exact.  The parts of a query or a weight
+//                   2^-6 of the largest and two residues (all of an fp32 number to
+//                   2^-28 of the largest).  The parts of a query or a weight
 //                   are columns of the other operand (two of them side by side, in
 //                   the same lane's accumulators).  hi times the first part sums
 //                   exactly on the tensor cores, whose sums are truncated to 24
@@ -35,9 +36,9 @@
 // cost 4 %.  Copies are bulk copies, one lane a segment (six cp.async loops took
 // 2000 cycles of a batch's 12 000).
 // 16 sequences of 1k to 32k tokens (8 KV heads, 4 queries each, 244 MB of records)
-// take 173 us (1.4 TB/s), 229 us with fp32 products on the CUDA cores (114
+// take 174 us (1.4 TB/s), 229 us with fp32 products on the CUDA cores (114
 // instructions, 10 - 12 warps, a warp walking 256 tokens alone); 8 heads of 4097
-// tokens 16.6 and 59 us; 128 heads of 8192 tokens at d = 64 97 and 145 us.  The
+// tokens 16.5 and 59 us; 128 heads of 8192 tokens at d = 64 96 and 144 us.  The
 // error of fp32 outputs against 64 bits is 0.55 to 1.0 times that of the fp32
 // products over 70 shapes (1 to 8 queries, 1 to 20000 tokens, every norm storage),
 // 0.77 times on average.  Two fp16 parts of everything and sums over a CTA's units

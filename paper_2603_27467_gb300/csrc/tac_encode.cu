@@ -1189,11 +1189,12 @@ __device__ __forceinline__ void tile_body(const S& sh, const uint8_t* in, uint8_
   //    log2 within kEl absolute plus a rounding of the result, and the roundings
   //    of qo and of the final fma at magnitudes up to 2^(B+1).
   // Tighter bounds of the second part (r_min's and r_max's errors weighed by the
-  // pair's place between them, the logarithms' own magnitudes) narrow the bands
-  // to 0.8 (8-bit linear) and 0.5 (4-bit log): a 32k-token cache takes 2255 us, not 2350.
-  // Fewer rows are then re-decided whole, and in rows of nearly equal norms more
-  // codes of the transform's own error stay: one channel x300, fp32, 150 of
-  // 1.28e7 codes instead of 142.  Not taken.
+  // pair's place between them, the quotient brought within 2u by a Newton step, the
+  // logarithms' own magnitudes) narrow the bands to 0.8 (8-bit linear) and 0.5
+  // (4-bit log): a 32k-token cache took 2255 us, 2326 with these.  Fewer rows are
+  // then re-decided whole, and in rows of nearly equal norms more codes of the
+  // transform's own error stay: one channel x300, fp32, 150 of 1.28e7 codes
+  // instead of 142.  Not taken.
   // A row whose band reaches 1/4 (rows of nearly equal pair norms, non-finite
   // rows) has every norm code re-decided.
   constexpr float kKappa = norm_kappa<D>();

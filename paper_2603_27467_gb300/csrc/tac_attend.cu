@@ -32,9 +32,13 @@
 // Bound: instruction issue: 95 warp-instructions a token-head (d = 128, 4
 // queries), 50 of them to decode and split its 128 pairs (table offset 2, lookup
 // 1, norm code 3, products and split 3, packing 2 for each), issued in 60 % of the
-// cycles at 16 warps per SM (128 registers); the barriers of the units' merges
-// cost 4 %.  Copies are bulk copies, one lane a segment (six cp.async loops took
-// 2000 cycles of a batch's 12 000).
+// cycles at 16 warps per SM (128 registers).  Of a long call (128 heads of 32768
+// tokens, 560 us) merging every unit is 7 % and the third parts of queries and
+// weights 4 % (timing copies without them); handing a unit's sums over by
+// mbarriers and merging them half a batch later instead of two CTA barriers takes
+// 4 % off at d = 64 and spills at d = 128 (batch of 16 sequences 174 -> 192 us).
+// Copies are bulk copies, one lane a segment (six cp.async loops took 2000 cycles
+// of a batch's 12 000).
 // 16 sequences of 1k to 32k tokens (8 KV heads, 4 queries each, 244 MB of records)
 // take 174 us (1.4 TB/s), 229 us with fp32 products on the CUDA cores (114
 // instructions, 10 - 12 warps, a warp walking 256 tokens alone); 8 heads of 4097
@@ -42,7 +46,7 @@
 // error of fp32 outputs against 64 bits is 0.55 to 1.0 times that of the fp32
 // products over 70 shapes (1 to 8 queries, 1 to 20000 tokens, every norm storage),
 // 0.77 times on average.  Two fp16 parts of everything and sums over a CTA's units
-// took 158, 20.5 and 84 us and had 0.74 to 2.5 times that error.
+// took 158, 20.5 and 84 us (484 us for the long call) and had 0.74 to 2.5 times that error.
 // Every unit is merged and written by itself, in a fixed order, so a job's outputs
 // do not depend on the other jobs of the call or on how the units fall to the CTAs.
 // Codebooks (n, norm bits, norm mode) are runtime parameters: K and V may

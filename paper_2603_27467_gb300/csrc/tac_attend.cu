@@ -43,9 +43,9 @@
 // take 174 us (1.4 TB/s), 229 us with fp32 products on the CUDA cores (114
 // instructions, 10 - 12 warps, a warp walking 256 tokens alone); 8 heads of 4097
 // tokens 16.5 and 59 us; 128 heads of 8192 tokens at d = 64 96 and 144 us.  The
-// error of fp32 outputs against 64 bits is 0.55 to 1.0 times that of the fp32
-// products over 70 shapes (1 to 8 queries, 1 to 20000 tokens, every norm storage),
-// 0.77 times on average.  Two fp16 parts of everything and sums over a CTA's units
+// error of fp32 outputs against 64 bits is 0.56 to 1.0 times that of the fp32
+// products over 105 shapes (1 to 8 queries, 1 to 32000 tokens, every norm storage,
+// 3 draws each), 0.77 times on average.  Two fp16 parts of everything and sums over a CTA's units
 // took 158, 20.5 and 84 us (484 us for the long call) and had 0.74 to 2.5 times that error.
 // Every unit is merged and written by itself, in a fixed order, so a job's outputs
 // do not depend on the other jobs of the call or on how the units fall to the CTAs.
@@ -69,8 +69,9 @@ constexpr int kAttUnit = TAC_ATTEND_SPLIT;    // tokens of a unit: one batch for
 // Jobs of at most this many tokens split the decoded values in three parts.  With
 // two a value keeps 2^-23 of its record's scale, which shows where few tokens share
 // the softmax: 1.0 to 1.13 times the error of fp32 products up to 40 tokens (fp32
-// norms), 0.56 to 0.99 times with three.  The third part costs 4 instructions a
-// pair; with more tokens two parts stay below 0.93 times.
+// norms), 0.66 to 1.0 times with three.  The third part costs 4 instructions a
+// pair; from 257 tokens on two parts are at 0.79 to 0.95 times (eight shapes of 12000
+// to 32768 tokens, 10 draws each; single draws from 0.5 to 1.5).
 constexpr int kAttThree = kAttUnit;
 constexpr float kLog2e = 1.4426950408889634f;
 static_assert(kAttUnit == kAttWarps * kAttBatch, "a unit is one batch per warp");

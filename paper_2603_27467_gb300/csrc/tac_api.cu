@@ -407,9 +407,10 @@ int64_t enc_min_bytes(int64_t tile_rows_total, int64_t njobs) {
 // tiles 58 / 47, 65536 tiles 78 / 84; one shape, d = 64, fp32 norms: 22000
 // tiles 31 / 29, 66000 tiles 54 / 70.  fp32 rows (twice the bytes of a tile to
 // stage, and more uncertified codes) meet at 0.6 of the limit that bf16 rows do:
-// with their tiles counted 5/3 no mix of d and shapes is slower than 0.97 of the
-// launches by shape just below the limit, 0.82 to 0.95 with them counted once (d =
-// 16, one shape, fp32 norms, 26000 tiles 33 / 40).  Calls with scattered records that share
+// with their tiles counted 5/3 the mixes of d and shapes run at 0.94 to 1.15 times
+// the speed of the launches by shape just below the limit (two runs of one side
+// differ by up to 6 % there), with them counted once at 0.82 to 0.95 times (d = 16,
+// one shape, fp32 norms, 26000 tiles 33 / 40).  Calls with scattered records that share
 // words (see plan_encode) are not small.
 constexpr int64_t kSmallEncodeTiles = 16384, kSmallEncodePerShape = 10240;
 constexpr int kSmallEncodeShapes = 4;
